@@ -104,12 +104,14 @@ typedef struct {
 /* Method of the correlation sums (identical results).  POPCOUNT: XOR + bit counts over
  * packed words, any L.  TENSOR: D_a(r) = N/2 - (1/2) sum_j G[j][j+r] with G the Gram
  * matrix of the L positions over the L^2 lines of the axis, computed on the 5th-generation
- * tensor cores (tcgen05.mma, e4m3 operands loaded by TMA, fp32 accumulators in tensor memory;
- * exact: |G| <= L^2 <= 2^24); L a multiple of 128 in 256..2048; it allocates a scratch of
- * 2 L^3 bytes (two axes of one replica expanded to e4m3, one multiplied while the next is
- * expanded: 17.2 GB at L=2048) at its first use and keeps it (ising_release_scratch frees it).  AUTO:
- * TENSOR for L >= 512 where it is supported and its scratch can be allocated (measured on
- * GB300: 1.9x faster than POPCOUNT at L=512, 3.5x at L=2048; slower at L=256), else POPCOUNT. */
+ * tensor cores (tcgen05.mma, spins as e2m1 values expanded from the packed words in shared
+ * memory, fp32 accumulators in tensor memory; exact: |G| <= L^2 <= 2^24); as an explicit choice
+ * L a multiple of 128 in 256..2048, with a scratch of 2 L^3 bytes (copies of the lattice in the
+ * order the kernel reads, used for L >= 512) allocated at its first use and kept
+ * (ising_release_scratch frees it).  AUTO: TENSOR for L a multiple of 64 in 64..2048, else
+ * POPCOUNT; the scratch is allocated as for TENSOR where L >= 512 is a multiple of 128, and the
+ * kernel reads the packed lattice where there is none or it cannot be allocated (measured on
+ * GB300: eight L = 256 replicas 0.05 ms against 0.51 by POPCOUNT, L = 2048 13 against 136). */
 typedef enum { ISING_CORR_AUTO = 0, ISING_CORR_POPCOUNT = 1, ISING_CORR_TENSOR = 2 } ising_corr;
 
 /* Sublattice order of a sweep.  01: red (q = 0) then blue every sweep (the paper's main
@@ -314,9 +316,9 @@ int64_t ising_launch_count(const ising_ctx *ctx);
  * random bits), so batching changes speed, not results.
  * Records and derived values are concatenated in class order, replica-major within a
  * class: ising_batch_record_words() int64 and 4 * ising_batch_lattices() doubles per
- * measured time; a measurement runs one class per stream, and classes with L >= 512 take
- * their correlation sums on the tensor cores (identical results), for which
- * ising_batch_create allocates 2 L^3 bytes of scratch per such class.  Only the PACKED
+ * measured time; a measurement runs one class per stream, on the tensor cores for L a multiple
+ * of 64 (identical results), and ising_batch_create allocates 2 L^3 bytes of scratch per class
+ * of L >= 512, a multiple of 128.  Only the PACKED
  * form is batched (opts->form must be PACKED). */
 typedef struct ising_batch ising_batch;
 int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *replicas, const uint64_t *seeds,

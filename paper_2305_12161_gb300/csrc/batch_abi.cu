@@ -29,7 +29,7 @@ struct BatchClass {
     int streamed;        // swept by a single-lattice sweep kernel instead of the persistent one
     SweepConfig cfg;     // that kernel's configuration (streamed classes)
     uint32_t *alt;       // second store of the fused whole-sweep kernel (allocated when chosen)
-    uint32_t *xt;        // tensor-core correlation scratch (L >= 512), else null: bit counts
+    uint32_t *xt;        // tensor-core correlation scratch (L >= 512), else null
 };
 
 bool packed_L_ok(int L) { return (L >= 64 && L % 64 == 0) || L == 4 || L == 8 || L == 16 || L == 32; }
@@ -271,7 +271,7 @@ int enqueue_measure(ising_batch *b, int64_t *rec, double *der, double c, unsigne
         const auto &k = b->cls[i];
         cudaStream_t st = i == 0 ? b->stream : b->side[i - 1];
         if (i > 0) BCK(b, cudaStreamWaitEvent(st, b->ev[0], 0));
-        const int method = !corr ? CORR_NONE : (k.xt ? CORR_TENSOR : CORR_POPCOUNT);
+        const int method = !corr ? CORR_NONE : (gram_supported(k.L) ? CORR_TENSOR : CORR_POPCOUNT);
         BCK(b, launch_measure(k.lat, k.L, k.R, b->t, method, rec + k.rec_off, st, &b->launches, k.xt, b->d_status,
                               (double)b->timeout_ns * 1e-9));
         if (der)
@@ -436,9 +436,8 @@ int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *r
             b->cls.push_back(k);
             return bail(ISING_ENOMEM);
         }
-        // L >= 512: the correlation sums on the tensor cores, as a single context chooses them
-        // (far faster than bit counts there); the scratch is allocated here, never while a
-        // schedule is being captured
+        // L >= 512: the tensor-core measurement's scratch is allocated here, never while a schedule
+        // is being captured
         if (L[c] >= 512 && corr_mma_supported(L[c]) &&
             cudaMalloc(&k.xt, corr_mma_scratch_bytes(L[c], replicas[c])) != cudaSuccess) {
             k.xt = nullptr;

@@ -32,9 +32,9 @@ struct ising_ctx {
     int8_t *plain = nullptr;     // PLAIN form lattice
     int64_t *rec_dev = nullptr;  // R records
     double *der_dev = nullptr;   // R x 4
-    uint32_t *xt = nullptr;      // tensor-core correlation: bit-transposed lattice (lazy)
+    uint32_t *xt = nullptr;      // tensor-core correlation, L >= 512: bit-transposed lattice (lazy)
     int *dev_err = nullptr;      // set by a device-side bounded wait that gave up
-    int xt_refused = 0;          // the tensor-core scratch could not be allocated (AUTO falls back)
+    int xt_refused = 0;          // that scratch could not be allocated (AUTO then measures without it)
     double wait_timeout_s = 2.0; // bound of each device-side wait (tensor-core path)
     int inject_stall = 0;        // test hook: the next tensor-core measurement loses one load
     int64_t t = 0;
@@ -258,8 +258,8 @@ struct Footprint {
     size_t total() const { return lat + lat_alt + plain + rec + der + err + corr; }
 };
 
-// Whether a measurement of this context runs the tensor-core correlation (before any
-// allocation was refused).
+// Whether a measurement of this context holds the tensor-core scratch (before any allocation was
+// refused).  AUTO also runs the tensor-core kernel at other sizes that it takes, without scratch.
 bool wants_tensor_corr(int L, const ising_opts &o)
 {
     return o.corr == ISING_CORR_TENSOR || (o.corr == ISING_CORR_AUTO && L >= 512 && corr_mma_supported(L));
@@ -537,17 +537,15 @@ int ising_measure_ex(ising_ctx *c, int64_t *rec, double *derived, double cval, u
     int method = CORR_NONE;
     if (corr) {
         method = CORR_POPCOUNT;
-        if (wants_tensor_corr(c->L, c->opts) && !(c->opts.corr == ISING_CORR_AUTO && c->xt_refused))
-            method = CORR_TENSOR;
+        if (c->opts.corr != ISING_CORR_POPCOUNT && gram_supported(c->L)) method = CORR_TENSOR;
     }
-    if (method == CORR_TENSOR && !c->xt) {
+    if (method == CORR_TENSOR && wants_tensor_corr(c->L, c->opts) && !c->xt && !c->xt_refused) {
         const size_t bytes = corr_mma_scratch_bytes(c->L, c->R);
         if (cudaMallocAsync((void **)&c->xt, bytes, c->stream) != cudaSuccess) {
             c->xt = nullptr;
             cudaGetLastError();  // a failed allocation is not sticky
             if (c->opts.corr == ISING_CORR_TENSOR) return fail(c, ISING_ENOMEM, "correlation scratch");
-            c->xt_refused = 1;   // automatic choice: the bit-count path needs no scratch
-            method = CORR_POPCOUNT;
+            c->xt_refused = 1;   // automatic choice: the kernel transposes the x axis as it reads
         }
     }
     const int inject = method == CORR_TENSOR ? c->inject_stall : 0;

@@ -1,22 +1,25 @@
-// Axis correlation sums D_a(r) on the tensor cores.
+// Axis correlation sums D_a(r), and with them M and B, on the tensor cores.
 //
 // Along one axis the lattice is L^2 lines of L sites.  With s = +-1,
 //   sum_i [s_i != s_(i + r e_a)] = (L * L^2 - S(r)) / 2,   S(r) = sum_j G[j][(j + r) mod L],
 // where G[j][k] = sum over lines of s(j) s(k) is the Gram matrix of the L positions over
-// the lines: a dense contraction of length L^2.  A packed word holds the same position of
-// 32 lines, so one word is the K = 32 slice of one fp8 tcgen05.mma: its bits become e4m3
-// values +1 / -1 (exact), products accumulate in fp32, and every partial sum is an even
-// integer of magnitude <= L^2 <= 2^24, so the result is exact.
+// the lines: a dense contraction of length L^2.  A spin is one e2m1 value (+1.0 = 0x2, -1.0 =
+// 0xA, exact), block scales are all 1.0, products accumulate in fp32, and every partial sum is
+// an even integer of magnitude <= L^2 <= 2^22, so the result is exact.
 //
-// Only the upper block triangle of G is computed (G is symmetric); an entry of an
-// off-diagonal tile stands for both ordered pairs (j, k) and (k, j).  Per replica and axis:
-// the axis's lines are expanded once into e4m3 rows in one of two scratch halves (x by
-// k_expand_x_e4m3; y and z by the helper warps of the previous axis's product, into the
-// other half), and k_gram_tma accumulates the 128 x 128 tiles of G by tcgen05.mma in tensor
-// memory from TMA-loaded, 128-byte swizzled shared-memory operands; each entry's -G/2 is
-// added to D at its cyclic distance; the records start from N/2.
-#include <cuda.h>
-
+// The operands never exist in global memory: the warps of a CTA read packed lattice words,
+// turn each 32-bit word into 32 nibbles (two logic operations per eight spins: the order of the
+// lines inside the contraction is free, so out word j takes the bits j, j + 4, j + 8, ...) and
+// write them into the 128-byte swizzled shared-memory tiles that tcgen05.mma reads.  At
+// L = 2048 a measurement takes 10.8 ms against 21.1 with e4m3 operands staged through global
+// memory (8.6 GB written and re-read per axis, and half the tensor rate); eight L = 256 replicas
+// take 0.054 ms against 0.51 by bit counts, 512 of L = 64 0.04 against 0.28.  The issue loop bounds
+// it: a stage of four products (512 cycles of tensor work) takes 835 cycles at L = 1024.
+//
+// Only the upper block triangle of G is computed (G is symmetric): an entry j < k stands for
+// both ordered pairs, i.e. for the distances k - j and L - (k - j).  B is the sum of the three
+// axes' D_a(1), and M is counted by the warps that read the z axis's words, so a measurement
+// is one pass of this kernel (plus, for L >= 512, a transposition of the lattice for the x axis).
 #include <algorithm>
 
 #include "common.cuh"
@@ -24,29 +27,18 @@
 
 namespace ising {
 
-constexpr int TM_T = 128;        // positions per tile side (M = N = 128)
-constexpr int GT_N = 256;        // B rows per CTA: two adjacent 128-position tiles (MMA N = 256)
-constexpr int GT_STAGES = 4;     // TMA pipeline depth (48 KB per stage)
-constexpr int GT_KB = 128;       // K bytes (= lines) per stage and operand box
-constexpr int GT_STAGE_BYTES = (TM_T + GT_N) * GT_KB;
-constexpr int UMMA_WAIT_LIMIT = 1 << 30;  // backstop on try_wait rounds (the wall-time bound comes first)
-constexpr int GT_THREADS = 256;  // Gram CTA: warps 0-3 load, multiply and read back; 4-7 expand the next axis
-
-
-// Four e4m3 values from the four bits of n (n < 16): bit i -> byte i, +1.0 (0x38) when
-// set, -1.0 (0xB8) when clear.  The multiplier places bit i at bit 8i + 7 (and the other
-// bits of n at positions that the mask drops, without carries).
-__device__ __forceinline__ uint32_t e4m3x4(uint32_t n)
-{
-    return ((n * 0x10204080u) & 0x80808080u) ^ 0xB8B8B8B8u;
-}
+constexpr int GB_ROW = 128;                    // bytes of a position's row in a stage: 256 lines
+constexpr int GB_LINES = 256;
+constexpr int GB_ARRIVE = 120;                 // arrivals of a full stage, shared by its warps
+constexpr int GB_SACC = 2048;                  // distance sums (largest L)
+constexpr int GB_WAIT_LIMIT = 1 << 30;         // backstop on try_wait rounds (wall time comes first)
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Shared-memory matrix descriptor of tcgen05.mma for a K-major operand in 128-byte swizzled
 // atoms (8 rows x 128 bytes; the 16-byte chunk c of row r stored at chunk c ^ r): start
 // address, leading byte offset 16 (unused when K fits one atom row), stride 1024 bytes between
-// atoms along M/N, descriptor version 1, swizzle mode 128B.  The K slice of 32 fp8 values at
+// atoms along M/N, descriptor version 1, swizzle mode 128B.  The K slice of 64 e2m1 values at
 // byte offset 32 s of the atom row is addressed by starting 32 s bytes later.
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
 {
@@ -54,9 +46,31 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-// Instruction descriptor: D in f32, A and B e4m3, both K-major, M = 128, N = GT_N.
-constexpr uint32_t UMMA_IDESC = (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(GT_N >> 3) << 17) |
-                                ((uint32_t)(TM_T >> 4) << 24);
+// Instruction descriptor of kind::mxf4 (dense, K = 64): A and B e2m1 (bits 7 and 10), both
+// K-major, N / 8 at bit 17, scales ue8m0 (bit 23), M / 128 at bit 27.
+__device__ __forceinline__ uint32_t mxf4_idesc(int N)
+{
+    return (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) | (1u << 27);
+}
+
+// D += A B of one K = 64 slice, every block scale read from tensor memory at `scale`.
+__device__ __forceinline__ void mma_mxf4(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t scale,
+                                         uint32_t acc)
+{
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%5], p;\n}\n" ::"r"(d),
+                 "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(scale));
+}
+
+// One lane of the warp.  The compiler knows that a branch on it is taken by a single lane, which
+// keeps the MMA operands in uniform registers: with `lane == 0` instead the issue loop took 1120
+// cycles per stage at L = 1024, with it 835.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
 
 __device__ __forceinline__ uint64_t globaltimer_ns()
 {
@@ -65,71 +79,32 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
+__device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done)
+                 : "r"(addr), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
+
 // Wait for phase `parity` of an mbarrier for at most timeout_ns of wall time (and at most
-// UMMA_WAIT_LIMIT rounds); false when it gave up.
+// GB_WAIT_LIMIT rounds); false when it gave up.
 __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, uint64_t timeout_ns)
 {
+    if (mbar_try(addr, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
-    for (int it = 0; it < UMMA_WAIT_LIMIT; ++it) {
-        uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(addr), "r"(parity)
-                     : "memory");
-        if (done) return true;
+    for (int it = 0; it < GB_WAIT_LIMIT; ++it) {
+        if (mbar_try(addr, parity)) return true;
         if ((it & 255) == 255 && globaltimer_ns() - t0 > timeout_ns) return false;
     }
     return false;
 }
 
-// ---------------------------------------------------------------------------------
-// The Gram products run on operands expanded once per measurement: E holds, for every
-// position p of the axis and every line K of it, the e4m3 value of s (+1 -> 0x38, -1 -> 0xB8),
-// chunk-major: the 128 lines of chunk K/128 of all L positions are one block of L x 128 bytes,
-// E[(K / 128) * L * 128 + p * 128 + K % 128], so a box of 128 positions x 128 lines is 16
-// contiguous KB (rows L^2 bytes apart would put every box's rows at a large power-of-two
-// stride).  Column cc of the panels (32 lines) is K = 32 cc .. 32 cc + 31.  Every word of the
-// lattice is expanded once instead of once per tile pair.
-__device__ __forceinline__ void expand_e4m3_word(uint32_t v, uint4 &lo, uint4 &hi)
-{
-    lo.x = e4m3x4(v & 0xFu);
-    lo.y = e4m3x4((v >> 4) & 0xFu);
-    lo.z = e4m3x4((v >> 8) & 0xFu);
-    lo.w = e4m3x4((v >> 12) & 0xFu);
-    hi.x = e4m3x4((v >> 16) & 0xFu);
-    hi.y = e4m3x4((v >> 20) & 0xFu);
-    hi.z = e4m3x4((v >> 24) & 0xFu);
-    hi.w = e4m3x4(v >> 28);
-}
-
-__device__ __forceinline__ void store_e4m3_word(uint8_t *dst, uint32_t v)
-{
-    uint4 lo, hi;
-    expand_e4m3_word(v, lo, hi);
-    reinterpret_cast<uint4 *>(dst)[0] = lo;
-    reinterpret_cast<uint4 *>(dst)[1] = hi;
-}
-
-// The same with streaming stores (evict first), for the helper warps of a Gram launch: the
-// operands of the running product stay in L2.
-__device__ __forceinline__ void store_e4m3_word_cs(uint8_t *dst, uint32_t v)
-{
-    uint4 lo, hi;
-    expand_e4m3_word(v, lo, hi);
-    __stcs(reinterpret_cast<uint4 *>(dst), lo);
-    __stcs(reinterpret_cast<uint4 *>(dst) + 1, hi);
-}
-
-// x axis, straight from the packed store: a CTA stages both sublattices' words of 128
-// consecutive rows (row = y + L z; four bundles B of 32 rows) in shared memory with coalesced
-// loads; a warp then takes word column kw of both parity classes pi of those rows (lane = row
-// in the bundle), transposes each 32 x 32 bit block in registers (five shuffle stages, each
-// swapping the off-diagonal half-blocks of size j between lanes r and r ^ j), after which lane
-// i holds, for site x = 2 (32 kw + i) + pi, the bits of the bundle's 32 rows.  The 64
-// positions x = 64 kw .. 64 kw + 63 of the column are consecutive 128-byte lines of the chunk:
-// the warp expands them into shared memory (16-byte piece c of position P at piece
-// c ^ ((P >> 1) & 7), so both the scattered writes and the line-ordered reads are
-// conflict-free) and writes the 8 KB with 512-byte coalesced stores.
+// Transposes the 32 x 32 bit block whose row i is lane i's word (five stages, each swapping the
+// off-diagonal half-blocks of size j between lanes r and r ^ j): lane i then holds bit i of
+// every row.
 __device__ __forceinline__ uint32_t transpose32_lane(uint32_t v, int lane)
 {
     const uint32_t FULL = 0xffffffffu;
@@ -144,394 +119,674 @@ __device__ __forceinline__ uint32_t transpose32_lane(uint32_t v, int lane)
     return v;
 }
 
-static size_t expand_x_smem_bytes(int W) { return (size_t)128 * (2 * W + 1) * sizeof(uint32_t) + 8 * 64 * 128; }
-
-__global__ void __launch_bounds__(256) k_expand_x_e4m3(const uint32_t *S0, const uint32_t *S1, Geom g, uint8_t *E)
+// The 32 spins of one word as e2m1 values (32 lines of one position): nibble m of out word j is
+// bit 4 m + j, sign bit set for a down spin.
+__device__ __forceinline__ uint4 expand_e2m1(uint32_t v)
 {
-    extern __shared__ __align__(16) uint32_t xt[];  // [128 rows][2 W + 1], then 8 warps x [64 lines][128 B]
-    const int L = g.L, W = g.W, RS = 2 * W + 1;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint4 *lines = reinterpret_cast<uint4 *>(xt + 128 * RS) + warp * 64 * 8;
-    const int64_t nB4 = (int64_t)L * L / 128;  // chunks of 128 rows = 4 bundles of 32
-    const int64_t blk = (int64_t)L * GT_KB;
-    for (int64_t B4 = blockIdx.x; B4 < nB4; B4 += gridDim.x) {
-        __syncthreads();  // the previous chunk's tile is consumed
-        // coalesced: consecutive threads read consecutive words of the chunk's rows
-        for (int e = tid; e < 128 * 2 * W; e += blockDim.x) {
-            const int ri = e / (2 * W), c = e - ri * 2 * W;
-            const int sub = c / W, kw = c - sub * W;
-            xt[ri * RS + c] = __ldg((sub ? S1 : S0) + (128 * B4 + ri) * W + kw);
-        }
-        __syncthreads();
-        for (int kw = warp; kw < W; kw += blockDim.x / 32) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int ri = 32 * b + lane;
-                const uint32_t row = (uint32_t)(128 * B4 + ri);  // < L^2
-                const uint32_t z = row / (uint32_t)L, y = row - z * (uint32_t)L;
-#pragma unroll
-                for (int pi = 0; pi < 2; ++pi) {
-                    const uint32_t v = xt[ri * RS + (((pi + y + z) & 1u) ? W : 0) + kw];
-                    uint4 lo, hi;
-                    expand_e4m3_word(transpose32_lane(v, lane), lo, hi);
-                    const int P = 2 * lane + pi, sw = lane & 7;  // (P >> 1) & 7
-                    lines[P * 8 + ((2 * b) ^ sw)] = lo;
-                    lines[P * 8 + ((2 * b + 1) ^ sw)] = hi;
-                }
-            }
-            __syncwarp();
-            uint4 *dst = reinterpret_cast<uint4 *>(E + B4 * blk + (int64_t)64 * kw * GT_KB);
-#pragma unroll 4
-            for (int j = 0; j < 16; ++j) {
-                const int t = 32 * j + lane, P = t >> 3;
-                dst[t] = lines[P * 8 + ((t & 7) ^ ((P >> 1) & 7))];
-            }
-            __syncwarp();
-        }
-    }
+    const uint32_t S = 0x88888888u, P = 0xAAAAAAAAu;
+    return make_uint4(((v << 3) & S) ^ P, ((v << 2) & S) ^ P, ((v << 1) & S) ^ P, (v & S) ^ P);
 }
 
-// y and z axes, one packed word each: column cc = (pi L + a) W + kw of position p (consecutive
-// words of one lattice row), the 32 lines 32 cc .. 32 cc + 31.
-__device__ __forceinline__ void expand_yz_word(const uint32_t *S0, const uint32_t *S1, const Geom &g, int axis,
-                                               uint8_t *E, int p, int cc)
+__device__ __forceinline__ void sts128(uint32_t addr, const uint4 &v)
 {
-    const int L = g.L, W = g.W;
-    const int64_t blk = (int64_t)L * GT_KB;  // bytes of one 128-line chunk of all positions
-    const int kw = cc % W;
-    const int rest = cc / W;  // pi L + a
-    const int a = rest % L, pi = rest / L;
-    const int y = axis == 1 ? p : a, z = axis == 1 ? a : p;
-    const uint32_t v = __ldg((((pi + y + z) & 1) ? S1 : S0) + ((int64_t)z * L + y) * W + kw);
-    store_e4m3_word(E + (int64_t)(cc >> 2) * blk + (int64_t)p * GT_KB + 32 * (cc & 3), v);
-}
-
-// The expansion a Gram launch's helper warps run for the next product: axis `axis` (1: y,
-// 2: z) of the lattice (S0, S1) into E (nullptr: none).  (The x axis, bit-transposed, has a
-// kernel of its own: run by the helper warps it slowed the product it shared the SMs with by
-// more than its own 2.3 ms at L = 2048.)
-struct ExpandJob {
-    const uint32_t *S0, *S1;
-    uint8_t *E;
-    int axis;
-};
-
-// Helper thread h of nh: its share of job j.
-__device__ __forceinline__ void run_expand_job(const ExpandJob &j, const Geom &g, int h, int nh)
-{
-    if (!j.E) return;
-    // words i = h + nh (U m + u): the U loads of a round are issued before its stores
-    constexpr int U = 16;
-    const int L = g.L, W = g.W;
-    const uint32_t ncols = (uint32_t)((int64_t)L * L / 32), total = (uint32_t)L * ncols;  // L^3 / 32 < 2^31
-    const int64_t blk = (int64_t)L * GT_KB;
-    for (uint32_t i0 = (uint32_t)h; i0 < total; i0 += (uint32_t)nh * U) {
-        uint32_t v[U];
-        uint8_t *dst[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t i = i0 + (uint32_t)nh * u;
-            v[u] = 0;
-            dst[u] = nullptr;
-            if (i < total) {
-                const int p = (int)(i / ncols), cc = (int)(i - (uint32_t)p * ncols);
-                const int kw = cc % W, rest = cc / W;  // rest = pi L + a
-                const int a = rest % L, pi = rest / L;
-                const int y = j.axis == 1 ? p : a, z = j.axis == 1 ? a : p;
-                v[u] = __ldg((((pi + y + z) & 1) ? j.S1 : j.S0) + ((int64_t)z * L + y) * W + kw);
-                dst[u] = j.E + (int64_t)(cc >> 2) * blk + (int64_t)p * GT_KB + 32 * (cc & 3);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (dst[u]) store_e4m3_word_cs(dst[u], v[u]);
-    }
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t addr, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t mbar)
-{
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(mbar)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                  : "memory");
 }
 
-// One CTA per (tile bj, super-tile sb of columns 2 sb, 2 sb + 1, K slice), 2 sb + 1 >= bj: thread
-// 0 loads the 128 x 128-byte box of tile bj and the 256 x 128-byte box of the super-tile by TMA
-// (128-byte swizzle) into a ring of GT_STAGES stages, thread 32 issues four tcgen05.mma of
-// 128 x 256 x 32 per stage into a 256-column fp32 accumulator in tensor memory and frees the
-// stage by tcgen05.commit; then warps 0-3 read the accumulator and add each entry of an
-// upper-triangle tile (bk >= bj, bk < nb) as -G/2 to D at its cyclic distance.  The CTAs of
-// one K slice run together and stream the same columns, so L2 serves the tiles' repeated
-// reads.  Warps 4-7 meanwhile expand the next product's axis (`next`) into the other scratch
-// half; they wait on nothing and join the CTA at the barrier after the main loop.  Measured:
-// L=1024 a whole measurement 2.18 ms against 2.93 with every expansion a kernel of its own;
-// L=2048 21.1 against 21.5 ms (there the helpers' 8.6 GB of stores cost the product part of
-// its L2 hits).
-//
-// Every wait is bounded (timeout_ns of %globaltimer).  A wait that gives up clears the CTA's
-// `flag`, sets *err and the CTA stops without adding anything to D.  Before it leaves:
-//  * the producer waits, bounded, on the `full` barrier of every stage whose TMA loads it
-//    issued and the MMA thread did not consume, so that no bulk copy is still writing this
-//    CTA's shared memory when the CTA exits (stages [mma_end, prod_end) of the ring);
-//  * the MMA thread commits every MMA it issued to `done` and waits for it; only when that
-//    commit has arrived is the tensor memory released.  If it has not (no MMA on resident
-//    operands takes seconds, so this is not expected), the CTA records *err = 2 and skips
-//    the dealloc rather than free tensor memory the tensor core may still write.
-// No test provokes these paths; the stall test drops stage 0's loads of CTA 0 before any
-// load or MMA is in flight.
-__global__ void __launch_bounds__(GT_THREADS, 1) k_gram_tma(const __grid_constant__ CUtensorMap tmA,
-                                                            const __grid_constant__ CUtensorMap tmB, int L, int nb,
-                                                            int nunits, int split, int64_t *D, int *err,
-                                                            uint64_t timeout_ns, int inject, ExpandJob next)
+// ---------------------------------------------------------------------------------
+// Line order for L >= 512, where each word is read by several CTAs: per axis a copy of the packed
+// lattice, N / 8 bytes, in which uint4 (2 c + h) L + p holds half h of the 256 lines of chunk c
+// at position p, so that a warp of 32 positions reads 512 consecutive bytes.  Read from the
+// packed store the words of 32 positions lie 128 bytes (y) or a plane (z) apart: at L = 2048 a
+// measurement took 17.6 ms that way and 13.4 with the copies (and their 1 ms) otherwise unchanged.
+
+// x axis: the lines are rows (row = y + L z), so their bits are transposed; half h holds the bundles
+// 32 (4 h + j) .. + 31 of the chunk's rows.  A CTA takes one chunk and four word columns: warp b reads
+// bundle b's rows and transposes the eight 32 x 32 bit blocks in registers.
+__global__ void __launch_bounds__(256) k_lines_x(const uint32_t *lat, Geom g, uint32_t *T, int64_t rep_words)
 {
-    extern __shared__ __align__(1024) uint8_t gsm[];
-    uint8_t *stage0 = gsm;  // [S][A 16 KB, B 32 KB]
-    long long *sacc = reinterpret_cast<long long *>(gsm + GT_STAGES * GT_STAGE_BYTES);
-    uint64_t *full = reinterpret_cast<uint64_t *>(sacc + 1026);
-    uint64_t *empty = full + GT_STAGES;
-    uint64_t *done = empty + GT_STAGES;
-    uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(done + 1);
-    int *flag = reinterpret_cast<int *>(tmem_holder + 1);
-    int *mma_end = flag + 1;      // stages whose operands the MMA thread waited for
-    int *mma_pending = flag + 2;  // 1: issued MMAs not known to be complete (keep the TMEM)
-
-    const int H = L / 2;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int sl = blockIdx.x / nunits;
-    int u = blockIdx.x - sl * nunits;
-    const int nsb = (nb + 1) / 2;
-    int bj = 0;
-    while (u >= nsb - bj / 2) {
-        u -= nsb - bj / 2;
-        ++bj;
+    __shared__ uint32_t sm[256 * 9];
+    const int L = g.L, W = g.W;
+    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+    const int c = blockIdx.x, kw0 = 4 * blockIdx.y, r = blockIdx.z;
+    const int nkw = min(4, W - kw0);
+    const uint32_t *S0 = lat + 2 * (int64_t)r * g.nw, *S1 = S0 + g.nw;
+    const uint32_t row = 256u * (uint32_t)c + 32u * (uint32_t)b + (uint32_t)lane;
+    const uint32_t z = row / (uint32_t)L, y = row - z * (uint32_t)L;
+    const bool odd = (y + z) & 1u;
+    const int64_t at = (int64_t)row * W + kw0;
+    uint32_t v0[4] = {0, 0, 0, 0}, v1[4] = {0, 0, 0, 0};
+    if (W % 4 == 0) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(S0 + at));
+        const uint4 d = __ldg(reinterpret_cast<const uint4 *>(S1 + at));
+        v0[0] = a.x; v0[1] = a.y; v0[2] = a.z; v0[3] = a.w;
+        v1[0] = d.x; v1[1] = d.y; v1[2] = d.z; v1[3] = d.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < nkw) {
+                v0[i] = __ldg(S0 + at + i);
+                v1[i] = __ldg(S1 + at + i);
+            }
     }
-    const int sb = bj / 2 + u;
-    const int j0 = bj * TM_T, s0 = sb * GT_N;
-    const int nk = (int)((int64_t)L * L / GT_KB);
-    const int c0 = (int)((int64_t)nk * sl / split), c1 = (int)((int64_t)nk * (sl + 1) / split);
-    const int n = c1 - c0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t e = transpose32_lane(odd ? v1[i] : v0[i], lane);  // x = 2 (32 kw + lane)
+        const uint32_t o = transpose32_lane(odd ? v0[i] : v1[i], lane);  // x + 1
+        sm[(64 * i + 2 * lane) * 9 + b] = e;
+        sm[(64 * i + 2 * lane + 1) * 9 + b] = o;
+    }
+    __syncthreads();
+    const int half = 64 * nkw * 4;  // words of one half in this CTA
+    for (int e = threadIdx.x; e < 2 * half; e += 256) {
+        const int h = e >= half, f = e - h * half;
+        T[(int64_t)r * rep_words + (((int64_t)c * 2 + h) * L + 64 * kw0) * 4 + f] = sm[(f >> 2) * 9 + 4 * h + (f & 3)];
+    }
+}
 
-    for (int i = tid; i <= H; i += GT_THREADS) sacc[i] = 0;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
-                     "r"(GT_N));
+// y (blockIdx.z even) and z axes, L a multiple of 256: chunk c = a W4 + k4 is the uint4 k4 of the rows
+// with other coordinate a, half pi the sites x = 2k + pi.  A CTA takes 32 positions of one a.
+__global__ void __launch_bounds__(256) k_lines_yz(const uint32_t *lat, Geom g, uint32_t *T, int64_t rep_words)
+{
+    __shared__ uint4 sm[2][8 * 33];
+    const int L = g.L, W4 = g.W / 4;
+    const int p0 = 32 * blockIdx.x, a = blockIdx.y, r = blockIdx.z >> 1, axis = 1 + (blockIdx.z & 1);
+    const uint4 *S0 = reinterpret_cast<const uint4 *>(lat + 2 * (int64_t)r * g.nw), *S1 = S0 + g.nw / 4;
+    const int t = threadIdx.x, n = 32 * W4;
+    if (t < n) {
+        const int i = t / W4, k = t - i * W4, p = p0 + i;
+        const int64_t at = (axis == 1 ? (int64_t)a * L + p : (int64_t)p * L + a) * W4 + k;
+        const bool odd = (p + a) & 1;
+        sm[odd][k * 33 + i] = __ldg(S0 + at);
+        sm[!odd][k * 33 + i] = __ldg(S1 + at);
+    }
+    __syncthreads();
+    if (t < n) {
+        const int k = t >> 5, i = t & 31;
+        uint4 *dst = reinterpret_cast<uint4 *>(T + (int64_t)r * rep_words + (int64_t)axis * 2 * g.nw) +
+                     ((int64_t)(a * W4 + k) * 2) * L + p0 + i;
+        dst[0] = sm[0][k * 33 + i];
+        dst[L] = sm[1][k * 33 + i];
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// Work items.  The L positions form super-tiles of 256 (the last may be short).  A unit is either
+// the diagonal block of a super-tile (its rows filled once; MMAs of rows 0..127 against all
+// columns and of rows 128..255 against columns 128..) or a tile of 128 rows against a later
+// super-tile.  An item is (replica, axis, slice of the lines, unit); the CTAs are persistent and
+// take items in that order, so the CTAs running together read the same lines.
+struct GramArgs {
+    const uint32_t *lat, *lines;  // lines: copies in line order (x only unless L % 256 == 0), or null
+    int64_t rep_words;            // words of one replica's copies
+    int64_t *rec;
+    int64_t RL, nw;            // record length; words per sublattice
+    int L, W;
+    int nsb, nunits, split, nitems;
+    int stage_bytes, nst;      // ring of stages
+    int ncols, scale_col;      // tensor memory: columns allocated, first of the 32 scale columns
+    int *err;
+    uint64_t timeout_ns;
+    int inject;
+};
+
+struct GramUnit {
+    int j0, s0;  // first row of the A tile, first position of the B super-tile
+    int ra, rb;  // rows filled for A (0: A is part of B) and for B
+};
+
+__device__ __forceinline__ GramUnit gram_unit(int u, int nsb, int L)
+{
+    GramUnit m;
+    if (u < nsb) {
+        m.j0 = m.s0 = 256 * u;
+        m.ra = 0;
+    } else {
+        u -= nsb;
+        int bj = 0;
+        while (u >= nsb - 1 - bj / 2) {
+            u -= nsb - 1 - bj / 2;
+            ++bj;
+        }
+        m.j0 = 128 * bj;
+        m.s0 = 256 * (bj / 2 + 1 + u);
+        m.ra = 128;
+    }
+    m.rb = min(256, L - m.s0);
+    return m;
+}
+
+// Readers: the eight words (256 lines) of this lane's share of one stage, for the stages
+// first, first + step, ... (chunks of 256 lines).  All addresses advance by additions.
+
+// y or z axis, rows of whole uint4 (W a multiple of 4): word pi * 4 + i is word kw + i of the row of
+// position p at the other coordinate a, of the sublattice that holds the sites x = 2k + pi there;
+// a chunk is four words of each.  The two sublattices swap roles whenever a advances.
+struct ReadYZ4 {
+    const uint4 *e, *o;  // next words of pi = 0 and pi = 1
+    int k4, W4, step;
+    int64_t da;          // uint4 from the end of one a's row to the next a's
+    __device__ ReadYZ4(const uint32_t *S0, const uint32_t *S1, int L, int W, int axis, int p, int c, int st)
+    {
+        W4 = W / 4;
+        step = st;
+        const int a = c / W4;
+        k4 = c - a * W4;
+        const int64_t at = (axis == 1 ? (int64_t)a * L + p : (int64_t)p * L + a) * W4 + k4;
+        da = axis == 1 ? (int64_t)(L - 1) * W4 : 0;
+        const bool odd = (p + a) & 1;
+        e = reinterpret_cast<const uint4 *>(odd ? S1 : S0) + at;
+        o = reinterpret_cast<const uint4 *>(odd ? S0 : S1) + at;
+    }
+    __device__ __forceinline__ void next(uint32_t v[8])
+    {
+        const uint4 s = __ldg(e), t = __ldg(o);
+        v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
+        v[4] = t.x; v[5] = t.y; v[6] = t.z; v[7] = t.w;
+        e += step;
+        o += step;
+        k4 += step;
+        while (k4 >= W4) {
+            k4 -= W4;
+            const uint4 *x = e + da;
+            e = o + da;
+            o = x;
+        }
+    }
+};
+
+// The same for other row widths: word column 4 c + i = a W + kw (a from a multiply by 2^32 / W,
+// exact for the columns of these sizes: below 2^16, W <= 32).
+struct ReadYZ1 {
+    const uint32_t *S0, *S1;
+    int L, W, axis, p, c, step;
+    uint32_t inv;
+    __device__ ReadYZ1(const uint32_t *s0, const uint32_t *s1, int l, int w, int ax, int pos, int c0, int st)
+        : S0(s0), S1(s1), L(l), W(w), axis(ax), p(pos), c(c0), step(st)
+    {
+        inv = (uint32_t)((0x100000000ull + (uint32_t)w - 1) / (uint32_t)w);
+    }
+    __device__ __forceinline__ void next(uint32_t v[8])
+    {
+        const uint32_t ci = 4u * (uint32_t)c;
+        int a = W == 1 ? (int)ci : (int)__umulhi(ci, inv);
+        int kw = (int)ci - a * W;
+        uint32_t s[4], t[4];
+        if (axis == 2) {  // the four words are consecutive
+            const int64_t at = (int64_t)p * L * W + ci;
+            const uint4 x = __ldg(reinterpret_cast<const uint4 *>(S0 + at));
+            const uint4 y = __ldg(reinterpret_cast<const uint4 *>(S1 + at));
+            s[0] = x.x; s[1] = x.y; s[2] = x.z; s[3] = x.w;
+            t[0] = y.x; t[1] = y.y; t[2] = y.z; t[3] = y.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (axis == 1) {
+                const int64_t at = ((int64_t)a * L + p) * W + kw;
+                s[i] = __ldg(S0 + at);
+                t[i] = __ldg(S1 + at);
+            }
+            const bool odd = (p + a) & 1;
+            v[i] = odd ? t[i] : s[i];
+            v[4 + i] = odd ? s[i] : t[i];
+            if (++kw == W) {
+                kw = 0;
+                ++a;
+            }
+        }
+        c += step;
+    }
+};
+
+// An axis in line order.
+struct ReadT {
+    const uint4 *q;
+    int64_t dq;
+    int L;
+    __device__ ReadT(const uint32_t *T, int l, int p, int c, int step) : L(l)
+    {
+        q = reinterpret_cast<const uint4 *>(T) + (int64_t)c * 2 * L + p;
+        dq = (int64_t)step * 2 * L;
+    }
+    __device__ __forceinline__ void next(uint32_t v[8])
+    {
+        const uint4 s = __ldg(q), t = __ldg(q + L);
+        v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
+        v[4] = t.x; v[5] = t.y; v[6] = t.z; v[7] = t.w;
+        q += dq;
+    }
+};
+
+// x axis of the packed lattice: word kw of both sublattices of the rows 256 c + 32 (b0 + i) + lane;
+// word 2 i + pi is bundle b0 + i's sites x = 2k + pi (still to be transposed).
+struct ReadXL {
+    const uint32_t *S0, *S1;
+    int64_t at, dat;
+    int L, W, dy, y[4];
+    uint32_t odd, dodd;  // bit i: parity of z of bundle b0 + i's row
+    __device__ ReadXL(const uint32_t *s0, const uint32_t *s1, int l, int w, int kw, int b0, int lane, int c, int step)
+        : S0(s0), S1(s1), L(l), W(w)
+    {
+        const int row = 256 * c + 32 * b0 + lane;
+        at = (int64_t)row * W + kw;
+        dat = (int64_t)256 * step * W;
+        odd = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int z = (row + 32 * i) / L;
+            y[i] = row + 32 * i - z * L;
+            odd |= (uint32_t)(z & 1) << i;
+        }
+        dy = (256 * step) % L;
+        dodd = ((256 * step) / L) & 1 ? 15u : 0u;
+    }
+    __device__ __forceinline__ void next(uint32_t v[8])
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t a = __ldg(S0 + at + 32 * i * W), b = __ldg(S1 + at + 32 * i * W);
+            const bool o = ((uint32_t)y[i] ^ (odd >> i)) & 1u;
+            v[2 * i] = o ? b : a;
+            v[2 * i + 1] = o ? a : b;
+            y[i] += dy;
+            if (y[i] >= L) {
+                y[i] -= L;
+                odd ^= 1u << i;
+            }
+        }
+        odd ^= dodd;
+        at += dat;
+    }
+};
+
+// What a warp does for its stages of one item.  The next stage's words are loaded and the present
+// one's are expanded in registers before the wait for the slot, so that between the slot's release
+// and its refill there are only the shared-memory stores: the ring holds four 48 KB stages, 2048
+// cycles of products, and the time round it bounds the kernel.  Returns false when a wait gave up.
+struct Fill {
+    uint32_t ring, full0, empty0;  // shared addresses
+    int nst, stage_bytes, arrive;
+    uint64_t timeout_ns;
+    int skip;                      // stage whose arrival is left out (failure injection), -1: none
+};
+
+template <class Read, class Expand, class Put>
+__device__ __forceinline__ bool fill_stages(const Fill &f, uint32_t g0, int set, int nsets, int n, Read &rd,
+                                            Expand expand, Put put)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t v[8];
+    if (set < n) rd.next(v);
+    int slot = (int)((g0 + (uint32_t)set) % (uint32_t)f.nst);
+    uint32_t phase = ((g0 + (uint32_t)set) / (uint32_t)f.nst) & 1u;
+#pragma unroll 1
+    for (int s = set; s < n; s += nsets) {
+        uint4 x[8];
+        expand(v, x);
+        if (s + nsets < n) rd.next(v);
+        // the slot's previous use was consumed (a barrier that has completed no phase passes parity 1)
+        const bool ok = mbar_wait(f.empty0 + 8u * (uint32_t)slot, phase ^ 1u, f.timeout_ns);
+        if (!__all_sync(0xffffffffu, ok)) return false;  // the warp leaves together
+        put(f.ring + (uint32_t)slot * (uint32_t)f.stage_bytes, x);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0 && s != f.skip)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(f.full0 + 8u * (uint32_t)slot),
+                         "r"(f.arrive)
+                         : "memory");
+        slot += nsets;
+        if (slot >= f.nst) {
+            slot -= f.nst;
+            phase ^= 1u;
+        }
+    }
+    return true;
+}
+
+// One CTA: the first PW warps fill the stages and afterwards read the accumulators, the last
+// warp issues the MMAs.  A stage holds 256 lines of every row of the unit; the (ra + rb) / 32
+// warps of a set fill it, one row per lane, and as many sets as the PW warps hold work on successive
+// stages.  Each stage is written once and read by 4 (off-diagonal) or 8 MMAs of 128 x N x 64.
+//
+// Every wait is bounded (timeout_ns of %globaltimer).  A wait that gives up clears `flag`, every
+// role leaves its loop, *err is set and nothing of the item is added to the records.  The MMA
+// thread commits what it issued to `done` and waits for it before the tensor memory is released;
+// if that arrival does not come either, *err = 2 and the tensor memory is kept rather than freed
+// under a running MMA.
+//
+// READS: which readers the instantiation holds (fewer keep more warps within the registers).
+// MINB CTAs share an SM.
+enum GramReads : int { GR_SMALL, GR_T, GR_XL, GR_ANY };  // XL + YZ1; T alone; XL + YZ4; all
+
+template <int PW, int MINB, int READS>
+__global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArgs ga)
+{
+    constexpr int GB_THREADS = 32 * (PW + 1);
+    extern __shared__ __align__(1024) uint8_t gsm[];
+    __shared__ int sacc[GB_SACC];
+    __shared__ __align__(8) uint64_t full[8], empty[8], done;
+    __shared__ uint32_t tmem_holder;
+    __shared__ int flag, mma_pending, pops[2];  // up spins of the z axis's words, by item parity
+
+    const int L = ga.L, W = ga.W, H = L / 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t ring = (smem_u32(gsm) + 1023u) & ~1023u;
+    const int nst = ga.nst;
+
+    for (int i = tid; i < L; i += GB_THREADS) sacc[i] = 0;
+    if (warp == PW) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
+                     "r"(ga.ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
-        for (int i = 0; i < GT_STAGES; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[i])));
+        for (int i = 0; i < nst; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[i])), "r"(GB_ARRIVE));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[i])));
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(done)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        *flag = 1;
-        *mma_end = 0;
-        *mma_pending = 0;
+        flag = 1;
+        mma_pending = 0;
+        pops[0] = pops[1] = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_holder;
+    const uint32_t tmem = tmem_holder;
+    const uint32_t scale = tmem + (uint32_t)ga.scale_col;
+    if (warp < 4) {  // every block scale is 1.0 (ue8m0 0x7F) whatever its place in the 32 columns
+        const uint32_t one4 = 0x7F7F7F7Fu;
+        const uint32_t at = scale + ((uint32_t)(32 * warp) << 16);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(at + 8 * i),
+                         "r"(one4));
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    int prod_end = 0;  // producer: stages [0, prod_end) were armed (expect_tx) and loaded
-    if (warp >= 4) {  // helper warps: the next product's expansion, into the other scratch half
-        run_expand_job(next, make_geom(L), (int)(blockIdx.x * (GT_THREADS - 128) + tid - 128),
-                       (int)(gridDim.x * (GT_THREADS - 128)));
-    } else if (tid == 0) {  // producer
-        for (int t = 0; t < n; ++t) {
-            const int st = t % GT_STAGES;
-            if (t >= GT_STAGES &&
-                !mbar_wait(smem_u32(&empty[st]), (uint32_t)(((t / GT_STAGES) - 1) & 1), timeout_ns)) {
-                *flag = 0;
-                break;
-            }
-            if (!*(volatile int *)flag) break;
-            const uint32_t sa = smem_u32(stage0 + st * GT_STAGE_BYTES);
-            mbar_expect_tx(smem_u32(&full[st]), GT_STAGE_BYTES);
-            prod_end = t + 1;
-            if (inject && blockIdx.x == 0 && t == 0) continue;  // test hook: this stage never fills
-            tma_load_2d(sa, &tmA, 0, (c0 + t) * L + j0, smem_u32(&full[st]));
-            tma_load_2d(sa + TM_T * GT_KB, &tmB, 0, (c0 + t) * L + s0, smem_u32(&full[st]));
-        }
-    } else if (tid == 32) {  // MMA issuer
-        int t = 0;
-        for (; t < n; ++t) {
-            const int st = t % GT_STAGES;
-            if (!*(volatile int *)flag) break;
-            if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((t / GT_STAGES) & 1), timeout_ns)) {
-                *flag = 0;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sa = smem_u32(stage0 + st * GT_STAGE_BYTES);
+    const int nk = (int)((int64_t)L * L / GB_LINES);
+    uint32_t g0 = 0;     // stages used by earlier items (ring position and phase)
+    uint32_t nitem = 0;  // items done: phase of `done`
+    for (int item = blockIdx.x; item < ga.nitems; item += gridDim.x, ++nitem) {
+        const GramUnit un = gram_unit(item % ga.nunits, ga.nsb, L);
+        int rest = item / ga.nunits;
+        const int sl = rest % ga.split;
+        rest /= ga.split;
+        const int axis = rest % 3, r = rest / 3;
+        const int c0 = (int)((int64_t)nk * sl / ga.split), c1 = (int)((int64_t)nk * (sl + 1) / ga.split);
+        const int n = c1 - c0;
+        const uint32_t *S0 = ga.lat + 2 * (int64_t)r * ga.nw, *S1 = S0 + ga.nw;
+        const bool bad_first = ga.inject && blockIdx.x == 0 && nitem == 0;
+
+        if (warp < PW) {
+            const int wps = (un.ra + un.rb) / 32;  // warps of a set: 2, 4, 6, 8, 10 or 12
+            // at most nst sets: a set that moves on to stage s + nsets then finds the slot's phase at
+            // most one behind the one it waits for, which the parity tells apart
+            const int nsets = min(PW / wps, nst);
+            const int set = warp / wps, ws = warp - set * wps;
+            if (set < nsets) {
+                const Fill fl{ring, smem_u32(full), smem_u32(empty), nst, ga.stage_bytes, GB_ARRIVE / wps,
+                              ga.timeout_ns, bad_first && ws == 0 ? 0 : -1};
+                int m = 0;
+                const bool count_m = axis == 2 && un.ra == 0;
+                bool ok;
+                if (READS != GR_T && axis == 0 && (READS != GR_ANY || ga.lines == nullptr)) {
+                    // this warp's share is word column kw and the bundles b0 .. b0 + 3 of the 64 rows
+                    // (positions) of warps ws & ~1 and ws | 1
+                    const int wr = 64 * (ws >> 1);
+                    const bool xA = wr >= un.rb;
+                    const int xr = xA ? wr - un.rb : wr;  // first of the 64 rows in its region
+                    const int kw = ((xA ? un.j0 : un.s0) + xr) >> 6, b0 = 4 * (ws & 1);
+                    ReadXL rd(S0, S1, L, W, kw, b0, lane, c0 + set, nsets);
+                    ok = fill_stages(
+                        fl, g0, set, nsets, n, rd,
+                        [&](uint32_t v[8], uint4 x[8]) {
 #pragma unroll
-            for (int q = 0; q < GT_KB / 32; ++q) {
-                const uint64_t ad = umma_desc_sw128(sa + 32 * q), bd = umma_desc_sw128(sa + TM_T * GT_KB + 32 * q);
-                const uint32_t acc = (t > 0 || q > 0) ? 1u : 0u;
-                asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-                             "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                             "l"(ad), "l"(bd), "r"(UMMA_IDESC), "r"(acc));
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&empty[st])));
-        }
-        *mma_end = t;
-        if (t > 0) {  // the last commit covers every MMA before it
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(done)));
-            if (!mbar_wait(smem_u32(done), 0u, timeout_ns)) {
-                *flag = 0;
-                // one more bounded window before the tensor memory is declared still in use
-                if (!mbar_wait(smem_u32(done), 0u, timeout_ns)) *mma_pending = 1;
-            }
-        }
-    }
-    __syncthreads();
-    if (tid == 0 && !*flag) {
-        // drain: every stage armed and loaded but not consumed by the MMA thread lands
-        // before the CTA may leave (at most GT_STAGES of them, all distinct ring slots)
-        for (int t = *mma_end; t < prod_end; ++t) {
-            if (inject && blockIdx.x == 0 && t == 0) continue;  // no load was issued for it
-            if (!mbar_wait(smem_u32(&full[t % GT_STAGES]), (uint32_t)((t / GT_STAGES) & 1), timeout_ns))
-                atomicExch(err, 3);
-        }
-    }
-    __syncthreads();
-    const bool ok = *flag && n > 0;
-    if (ok && warp < 4) {  // warp w reads tensor-memory lanes 32 w .. 32 w + 31
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int j = j0 + 32 * warp + lane;  // this thread's row of the tile (TMEM lane)
-#pragma unroll 1
-        for (int cc = 0; cc < GT_N; cc += 16) {
-            const int bk = 2 * sb + cc / TM_T;
-            if (bk < bj || bk >= nb) continue;  // lower-triangle or missing tile of the super-tile
-            uint32_t v[16];
-            const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)cc;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                           "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                           "=r"(v[14]), "=r"(v[15])
-                         : "r"(ta));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                            for (int i = 0; i < 8; ++i) x[i] = expand_e2m1(transpose32_lane(v[i], lane));
+                        },
+                        [&](uint32_t base, uint4 x[8]) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int k = s0 + cc + q;
-                const long long G = (long long)__float2int_rn(__uint_as_float(v[q]));
-                if (bj == bk) {
-                    int d = k - j;
-                    if (d < 0) d += L;
-                    if (d >= 1 && d <= H) atomicAdd((unsigned long long *)&sacc[d], (unsigned long long)G);
+                            for (int i = 0; i < 8; ++i) {  // bundle b0 + i / 2, positions 64 kw + 2 lane + (i & 1)
+                                const uint32_t rr = (uint32_t)(xr + 2 * lane + (i & 1));
+                                sts128(base + (xA ? 32768u : 0u) + rr * GB_ROW +
+                                           ((((uint32_t)(b0 + (i >> 1))) ^ (rr & 7u)) << 4),
+                                       x[i]);
+                            }
+                        });
                 } else {
-                    const int d = k - j;  // 0 < d < L
-                    if (d <= H) atomicAdd((unsigned long long *)&sacc[d], (unsigned long long)G);
-                    if (L - d <= H) atomicAdd((unsigned long long *)&sacc[L - d], (unsigned long long)G);
+                    // this lane's row: B rows first, then (off-diagonal units) the A rows 32 KB further on
+                    const int f = 32 * ws + lane;
+                    const bool isA = f >= un.rb;
+                    const int ri = isA ? f - un.rb : f;
+                    const int p = isA ? un.j0 + ri : un.s0 + ri;
+                    const uint32_t row_off = (isA ? 32768u : 0u) + (uint32_t)ri * GB_ROW + (uint32_t)((ri & 7) << 4);
+                    auto expand = [&](uint32_t v[8], uint4 x[8]) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) x[i] = expand_e2m1(v[i]);
+                        if (count_m)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) m += __popc(v[i]);
+                    };
+                    auto put = [&](uint32_t base, uint4 x[8]) {
+                        const uint32_t at = base + row_off;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) sts128(at ^ (uint32_t)(i << 4), x[i]);
+                    };
+                    if (READS == GR_T || (READS == GR_ANY && axis == 0)) {
+                        ReadT rd(ga.lines + (int64_t)r * ga.rep_words + (int64_t)axis * 2 * ga.nw, L, p, c0 + set, nsets);
+                        ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
+                    } else if (READS == GR_XL || (READS == GR_ANY && W % 4 == 0)) {
+                        ReadYZ4 rd(S0, S1, L, W, axis, p, c0 + set, nsets);
+                        ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
+                    } else {
+                        ReadYZ1 rd(S0, S1, L, W, axis, p, c0 + set, nsets);
+                        ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
+                    }
+                }
+                if (!ok) *(volatile int *)&flag = 0;
+                if (count_m) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+                    if (lane == 0) atomicAdd(&pops[nitem & 1u], m);
+                }
+            }
+        } else if (elect_one()) {  // MMA issuer
+            int s = 0;
+            const uint32_t id0 = mxf4_idesc(un.rb);
+            const bool two = un.ra == 0 && un.rb > 128;
+            const uint32_t id1 = mxf4_idesc(two ? un.rb - 128 : 64);
+            int slot = (int)(g0 % (uint32_t)nst);
+            uint32_t phase = (g0 / (uint32_t)nst) & 1u;
+            for (; s < n; ++s) {
+                if (!mbar_wait(smem_u32(&full[slot]), phase, ga.timeout_ns)) {
+                    *(volatile int *)&flag = 0;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t base = ring + (uint32_t)slot * (uint32_t)ga.stage_bytes;
+                const uint32_t abase = un.ra ? base + 32768u : base;
+#pragma unroll
+                for (int q = 0; q < GB_ROW / 32; ++q)
+                    mma_mxf4(tmem, umma_desc_sw128(abase + 32 * q), umma_desc_sw128(base + 32 * q), id0, scale,
+                             (s > 0 || q > 0) ? 1u : 0u);
+                if (two) {
+#pragma unroll
+                    for (int q = 0; q < GB_ROW / 32; ++q)
+                        mma_mxf4(tmem + 256u, umma_desc_sw128(base + 16384u + 32 * q),
+                                 umma_desc_sw128(base + 16384u + 32 * q), id1, scale, (s > 0 || q > 0) ? 1u : 0u);
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                    smem_u32(&empty[slot])));
+                if (++slot == nst) {
+                    slot = 0;
+                    phase ^= 1u;
+                }
+            }
+            if (s > 0) {  // covers every MMA issued before it
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                    smem_u32(&done)));
+                if (!mbar_wait(smem_u32(&done), nitem & 1u, ga.timeout_ns)) {
+                    *(volatile int *)&flag = 0;
+                    // one more bounded window before the tensor memory is declared still in use
+                    if (!mbar_wait(smem_u32(&done), nitem & 1u, ga.timeout_ns)) mma_pending = 1;
                 }
             }
         }
+        __syncwarp();
+        __syncthreads();
+        if (!*(volatile int *)&flag) break;
+        if (warp < PW) {
+            // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 and every (PW / 4)-th group of 16 columns
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int row0 = 32 * (warp & 3) + lane;
+            const int ncol = un.rb, ncol1 = (un.ra == 0 && un.rb > 128) ? un.rb - 128 : 0;
+#pragma unroll 1
+            for (int cc = 16 * (warp >> 2); cc < ncol + ncol1; cc += 4 * PW) {
+                const bool second = cc >= ncol;
+                const int col = second ? cc - ncol + 256 : cc;
+                const int j = un.j0 + row0 + (second ? 128 : 0);
+                const int k0 = second ? un.s0 + 128 + cc - ncol : un.s0 + cc;
+                uint32_t v[16];
+                const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)col;
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                               "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+                               "=r"(v[14]), "=r"(v[15])
+                             : "r"(ta));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (j < L) {
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                        const int k = k0 + q;
+                        // 32-bit sums: at most 256 entries of magnitude <= L^2 per distance and item
+                        if (k > j && k < L) atomicAdd(&sacc[k - j], __float2int_rn(__uint_as_float(v[q])));
+                    }
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        }
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        int64_t *rec = ga.rec + (int64_t)r * ga.RL;
+        int64_t *D = rec + 3 + (int64_t)axis * (H + 1);
+        for (int d = 1 + tid; d <= H; d += GB_THREADS) {
+            const long long s2 = (long long)sacc[d] + sacc[L - d];
+            sacc[d] = 0;
+            sacc[L - d] = 0;
+            if (s2) {
+                atomicAdd(reinterpret_cast<unsigned long long *>(D + d), (unsigned long long)(-(s2 / 2)));
+                if (d == 1) atomicAdd(reinterpret_cast<unsigned long long *>(rec + 2), (unsigned long long)(-(s2 / 2)));
+            }
+        }
+        if (tid == 0 && axis == 2 && un.ra == 0) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(rec + 1), (unsigned long long)(2ll * pops[nitem & 1u]));
+            pops[nitem & 1u] = 0;  // used again two items on, after the next item's barriers
+        }
+        g0 += (uint32_t)n;
     }
-    if (!*flag && tid == 0) atomicCAS(err, 0, 1);
-    if (*mma_pending && tid == 0) atomicExch(err, 2);
+    if (tid == 0 && !*(volatile int *)&flag) atomicCAS(ga.err, 0, 1);
+    if (tid == 0 && mma_pending) atomicExch(ga.err, 2);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0 && !*mma_pending)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GT_N));
-    if (!ok) return;
-    for (int i = 1 + tid; i <= H; i += GT_THREADS)
-        if (sacc[i]) atomicAdd((unsigned long long *)(D + i), (unsigned long long)(-(sacc[i] / 2)));
+    if (warp == PW && !mma_pending)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ga.ncols));
 }
 
-static size_t gram_smem_bytes() { return (size_t)GT_STAGES * GT_STAGE_BYTES + 1026 * 8 + (2 * GT_STAGES + 1) * 8 + 32; }
+// Sizes the kernel takes: rows of whole words, distance sums that fit their 32 bits.
+bool gram_supported(int L) { return L >= 64 && L <= 2048 && L % 64 == 0; }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+// Sizes of the explicit option ISING_CORR_TENSOR.
+bool corr_mma_supported(int L) { return L >= 256 && L <= 2048 && L % 128 == 0; }
 
-// The driver's tensor-map encoder, looked up once through the runtime (no link to libcuda).
-static EncodeTiledFn encode_tiled()
-{
-    static EncodeTiledFn fn = nullptr;
-    static bool looked = false;
-    if (!looked) {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(f);
-        looked = true;
-    }
-    return fn;
-}
-
-bool corr_mma_supported(int L) { return L >= 256 && L <= 2048 && L % TM_T == 0 && L % 64 == 0; }
-
+// What a context or batch class of L >= 512 holds for the measurement: the copies in line order of
+// up to 5 replicas (16 where only the x axis has one) at a time fill it.
 size_t corr_mma_scratch_bytes(int L, int R)
 {
-    (void)R;  // replicas are multiplied one after the other through two expanded axes
+    (void)R;
     return (size_t)2 * L * L * L;
 }
 
+template <int PW, int MINB, int READS>
+static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaStream_t s)
+{
+    auto kern = k_gram_bits<PW, MINB, READS>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)grid, 32 * (PW + 1), smem, s>>>(ga);
+    return cudaGetLastError();
+}
+
+// rec: records initialised to D = N / 2 (r >= 1), M = -N, B = 3 N / 2.  scratch: 2 L^3 bytes for
+// the copies in line order, or null (the kernel then reads the packed store: below L = 512 a word is
+// read by one to three units only).
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *scratch, int *err,
                             cudaStream_t s, int64_t *launches, double timeout_s, int inject)
 {
-    const uint64_t timeout_ns = (uint64_t)(timeout_s * 1e9);
+    if (!gram_supported(L)) return cudaErrorInvalidValue;
     const Geom g = make_geom(L);
-    // two halves of L^3 bytes: product i reads half i % 2 while its helper warps expand product
-    // i + 1 into the other
-    uint8_t *E[2] = {reinterpret_cast<uint8_t *>(scratch), reinterpret_cast<uint8_t *>(scratch) + (size_t)L * L * L};
-    EncodeTiledFn enc = encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
-    // E viewed as rows of 128 bytes: row (chunk * L + position); boxes of 128 and 256 rows
-    CUtensorMap tmA[2], tmB[2];
-    const cuuint64_t gdim[2] = {(cuuint64_t)GT_KB, (cuuint64_t)L * L * L / GT_KB};
-    const cuuint64_t gstride[1] = {(cuuint64_t)GT_KB};
-    const cuuint32_t boxA[2] = {GT_KB, TM_T}, boxB[2] = {GT_KB, GT_N};
-    const cuuint32_t estr[2] = {1, 1};
-    for (int h = 0; h < 2; ++h)
-        if (enc(&tmA[h], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, E[h], gdim, gstride, boxA, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-            enc(&tmB[h], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, E[h], gdim, gstride, boxB, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const size_t smem = gram_smem_bytes();
-    if ((e = cudaFuncSetAttribute(k_gram_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
-    const int nb = L / TM_T, nsb = (nb + 1) / 2;
-    int nunits = 0;  // (tile row bj, super-tile sb >= bj / 2)
-    for (int bj = 0; bj < nb; ++bj) nunits += nsb - bj / 2;
-    int split = sms / nunits;  // one CTA per SM: K slices x units <= SMs
-    if (split < 1) split = 1;
-    const int64_t H = L / 2, RL = 3 + 3 * (H + 1);
-    const size_t xsm = expand_x_smem_bytes(g.W);
-    if ((e = cudaFuncSetAttribute(k_expand_x_e4m3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xsm)) !=
-        cudaSuccess)
-        return e;
-    // per replica: x expanded by its own kernel into half 0; its product's helper warps expand
-    // y into half 1, and the y product's helpers z into half 0; the z product runs alone
-    for (int r = 0; r < R; ++r) {
-        const uint32_t *S0 = lat + 2 * (int64_t)r * g.nw, *S1 = S0 + g.nw;
-        k_expand_x_e4m3<<<(unsigned)std::min<int64_t>((int64_t)L * L / 128, (int64_t)sms * 2), 256, xsm, s>>>(
-            S0, S1, g, E[0]);
-        for (int axis = 0; axis < 3; ++axis) {
-            const ExpandJob next = axis < 2 ? ExpandJob{S0, S1, E[(axis + 1) % 2], axis + 1}
-                                            : ExpandJob{nullptr, nullptr, nullptr, 0};
-            k_gram_tma<<<(unsigned)(nunits * split), GT_THREADS, smem, s>>>(
-                tmA[axis % 2], tmB[axis % 2], L, nb, nunits, split, rec + r * RL + 3 + axis * (H + 1), err,
-                timeout_ns, inject && r == 0 && axis == 1, next);
+    const bool lines = scratch != nullptr && L >= 512, all3 = g.W % 4 == 0;
+    const int per = !lines ? R : (all3 ? 5 : 16);  // replicas per pass: the scratch holds 16 copies
+    GramArgs ga{};
+    ga.rec = rec;
+    ga.RL = 3 + 3 * (int64_t)(L / 2 + 1);
+    ga.nw = g.nw;
+    ga.L = L;
+    ga.W = g.W;
+    ga.nsb = (L + 255) / 256;
+    ga.nunits = ga.nsb;
+    const int nb = (L + 127) / 128;
+    for (int bj = 0; bj < nb; ++bj) ga.nunits += ga.nsb - 1 - bj / 2;
+    // one stage: 16 KB (one tile), 32 KB (one super-tile) or 48 KB (super-tile and A tile).  Up to
+    // L = 128 half of the tensor memory and of the shared memory suffice, so two CTAs share an SM
+    // and one's read-back overlaps the other's products.
+    const bool small = L <= 128;
+    ga.stage_bytes = small ? 16384 : (L <= 256 ? 32768 : 49152);
+    ga.nst = L <= 256 ? 6 : 4;
+    ga.ncols = small ? 256 : 512;
+    ga.scale_col = small ? 128 : 384;
+    ga.err = err;
+    ga.timeout_ns = (uint64_t)(timeout_s * 1e9);
+    const size_t smem = (size_t)ga.nst * ga.stage_bytes + 1024;
+    const int slots = device_sms() * (small ? 2 : 1);
+    const int nk = (int)((int64_t)L * L / GB_LINES);
+    for (int r0 = 0; r0 < R; r0 += per) {
+        const int nr = std::min(per, R - r0);
+        ga.lat = lat + 2 * (int64_t)r0 * g.nw;
+        ga.rec = rec + (int64_t)r0 * ga.RL;
+        ga.lines = lines ? scratch : nullptr;
+        ga.rep_words = (all3 ? 3 : 1) * 2 * g.nw;
+        if (lines) {
+            k_lines_x<<<dim3((unsigned)nk, (unsigned)((g.W + 3) / 4), (unsigned)nr), 256, 0, s>>>(ga.lat, g, scratch,
+                                                                                                ga.rep_words);
+            if (all3)
+                k_lines_yz<<<dim3((unsigned)(L / 32), (unsigned)L, (unsigned)(2 * nr)), 256, 0, s>>>(ga.lat, g, scratch,
+                                                                                                     ga.rep_words);
         }
+        // slices of the lines: the count whose rounds of items over the CTAs take the fewest stages,
+        // counting an item's start and read-back as 8 stages
+        const int64_t base = (int64_t)nr * 3 * ga.nunits;
+        double best = 1e300;
+        for (int sp = 1; sp <= std::min(nk, 64); ++sp) {
+            const int64_t items = base * sp;
+            const int64_t rounds = (items + slots - 1) / slots;
+            const double cost = (double)rounds * ((double)((nk + sp - 1) / sp) + 8.0);
+            if (cost < best * 0.999) best = cost, ga.split = sp;
+        }
+        ga.nitems = (int)(base * ga.split);
+        ga.inject = inject && r0 == 0;
+        const int grid = std::min(ga.nitems, slots);
+        cudaError_t e;
+        if (small) e = launch_gram<12, 2, GR_SMALL>(ga, grid, smem, s);
+        else if (lines && all3) e = launch_gram<24, 1, GR_T>(ga, grid, smem, s);
+        else if (all3) e = launch_gram<24, 1, GR_XL>(ga, grid, smem, s);
+        else e = launch_gram<12, 1, GR_ANY>(ga, grid, smem, s);
+        if (e != cudaSuccess) return e;
+        if (launches) *launches += !lines ? 1 : (all3 ? 3 : 2);
     }
-    if (launches) *launches += 4 * (int64_t)R;
     return cudaGetLastError();
 }
 

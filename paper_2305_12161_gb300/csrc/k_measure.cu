@@ -20,8 +20,9 @@ namespace ising {
 
 __device__ __forceinline__ int64_t rec_len(int L) { return 3 + 3 * (int64_t)(L / 2 + 1); }
 
-// corr: 0 = correlations not measured (-1), 1 = summed from 0, 2 = tensor-core path,
-// which subtracts from N/2 (D_a(0) stays 0).
+// corr: 0 = correlations not measured (-1), 1 = summed from 0, 2 = tensor-core path, which
+// subtracts from N/2 (D_a(0) stays 0) and brings M and B itself: M = 2 (up spins) - N, and B as
+// the sum of the axes' D_a(1).
 __global__ void k_rec_init(int64_t *rec, int L, int R, int64_t t, int corr)
 {
     const int64_t RL = rec_len(L);
@@ -31,7 +32,7 @@ __global__ void k_rec_init(int64_t *rec, int L, int R, int64_t t, int corr)
         const int64_t j = i % RL;
         int64_t v;
         if (j == 0) v = t;
-        else if (j < 3) v = 0;
+        else if (j < 3) v = corr == 2 ? (j == 1 ? -2 * half_n : 3 * half_n) : 0;
         else if (corr == 0) v = -1;
         else if (corr == 2 && (j - 3) % H1 != 0) v = half_n;
         else v = 0;
@@ -407,6 +408,11 @@ cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int cor
     int64_t nb = (RL * R + 255) / 256;
     if (nb > 4096) nb = 4096;
     k_rec_init<<<(unsigned)nb, 256, 0, s>>>(rec, L, R, t, corr);
+    if (corr == CORR_TENSOR) {  // M, B and D_a(r) in one pass
+        if (!err || !gram_supported(L)) return cudaErrorInvalidValue;
+        if (launches) *launches += 1;
+        return launch_corr_mma(lat, L, R, rec, xt_scratch, err, s, launches, wait_timeout_s, inject_stall);
+    }
     if (L >= 256 && L % 256 == 0) {
         int64_t mb = (g.nw / 4 + 255) / 256;
         if (mb > (int64_t)device_sms() * 8) mb = (int64_t)device_sms() * 8;
@@ -417,12 +423,7 @@ cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int cor
         k_mb<<<dim3((unsigned)mb, (unsigned)R), 256, 0, s>>>(lat, g, rec);
     }
     int n = 2;
-    if (corr == CORR_TENSOR) {
-        if (!xt_scratch || !err || !corr_mma_supported(L)) return cudaErrorInvalidValue;
-        const cudaError_t e = launch_corr_mma(lat, L, R, rec, xt_scratch, err, s, nullptr, wait_timeout_s, inject_stall);
-        if (e != cudaSuccess) return e;
-        n += 2;
-    } else if (corr) {
+    if (corr) {
         const cudaError_t e = corr_rt(L) == 8 ? launch_corr<8>(lat, g, R, rec, s) : launch_corr<4>(lat, g, R, rec, s);
         if (e != cudaSuccess) return e;
         ++n;

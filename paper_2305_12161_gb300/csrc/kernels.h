@@ -110,16 +110,17 @@ cudaError_t launch_unpack(const uint32_t *lat, int8_t *plain, int L, int R, cuda
 // ---- measurement on the packed store ----------------------------------------------
 // rec: R records of 3 + 3*(L/2+1) int64 (must not alias lat).  Writes t, M, B and the
 // correlation sums D_a(r) by the chosen method (CORR_NONE writes D_a(r) = -1).
-// CORR_TENSOR needs corr_mma_supported(L), xt_scratch of corr_mma_scratch_bytes(L, R) bytes
-// and err (a device int set to 1 if a bounded wait of the tensor-core kernel gave up; the
-// records are then incomplete).
+// CORR_TENSOR needs gram_supported(L) and err (a device int set to 1 if a bounded wait of the
+// tensor-core kernel gave up; the records are then incomplete); xt_scratch is either
+// corr_mma_scratch_bytes(L, R) bytes, which L >= 512 uses for the transposed x axis, or null.
 enum CorrMethod : int { CORR_NONE = 0, CORR_POPCOUNT = 1, CORR_TENSOR = 2 };
 // wait_timeout_s bounds each device-side wait of the tensor-core path (wall time);
 // inject_stall (tests) makes one of its CTAs skip a load so that a wait runs out.
 cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int corr, int64_t *rec,
                            cudaStream_t s, int64_t *launches, uint32_t *xt_scratch = nullptr, int *err = nullptr,
                            double wait_timeout_s = 2.0, int inject_stall = 0);
-bool corr_mma_supported(int L);
+bool gram_supported(int L);      // sizes the tensor-core kernel takes
+bool corr_mma_supported(int L);  // sizes of the explicit option ISING_CORR_TENSOR
 size_t corr_mma_scratch_bytes(int L, int R);
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *xt_scratch, int *err,
                             cudaStream_t s, int64_t *launches, double timeout_s, int inject);
