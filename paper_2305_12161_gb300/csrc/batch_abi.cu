@@ -28,6 +28,7 @@ struct BatchClass {
     int64_t der_off;     // offset (in replicas) of this class's derived rows
     int streamed;        // swept by a single-lattice sweep kernel instead of the persistent one
     SweepConfig cfg;     // that kernel's configuration (streamed classes)
+    int automatic;       // cfg is the default: long segments may run the resident sweep instead
     uint32_t *alt;       // second store of the fused whole-sweep kernel (allocated when chosen)
     uint32_t *xt;        // tensor-core correlation scratch (L >= 512), else null
 };
@@ -61,12 +62,13 @@ struct ising_batch {
     BatchTask *d_tasks = nullptr;
     unsigned *d_barriers = nullptr;
     int ngroups = 0;
-    int *d_status = nullptr;
+    int *d_status = nullptr;  // [0] status, [1, 2] counters of the resident sweep's barriers
     unsigned long long *d_cta_ns = nullptr;
     int smem = 0, occ = 0, sms = 0, capacity = 0;
     double w_local = 1.0, w_group = 1.0;
     uint64_t timeout_ns = 2000000000ull;
     int missing_cta = -1;
+    int no_resident = 0;     // the device refused the resident sweep's launch
     int stream_min_L = 256;  // classes with L >= this (and L % 256 == 0) are streamed
     // measurement scratch
     int64_t *d_rec = nullptr;
@@ -208,8 +210,24 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
     while (n > 0) {
         const int chunk = (int)std::min<int64_t>(n, 1 << 30);
         int nstreamed = 0, si = 0;
-        for (const auto &k : b->cls) nstreamed += k.streamed;
-        const bool persistent = !b->h_tasks.empty();
+        // classes swept resident in shared memory (k_resident.cu), on the batch's stream one after the
+        // other (each fills the GPU): streamed classes on their default kernel, and the persistent
+        // kernel's classes when every one of them can be (the tuner's probes, which time that kernel's
+        // CTAs, and the failure injection into it keep it)
+        std::vector<ResidentPlan> rp(b->cls.size());
+        std::vector<char> res(b->cls.size(), 0);
+        bool all_small = cta_ns == nullptr && b->missing_cta < 0;
+        for (size_t i = 0; i < b->cls.size(); ++i) {
+            const auto &k = b->cls[i];
+            res[i] = !b->no_resident && (k.automatic || !k.streamed) && resident_plan(k.L, k.R, b->sms, &rp[i]) &&
+                     chunk >= rp[i].min_n;
+            if (!k.streamed && !res[i]) all_small = false;
+        }
+        for (size_t i = 0; i < b->cls.size(); ++i) {
+            if (!b->cls[i].streamed) res[i] = res[i] && all_small;
+            else nstreamed += !res[i];
+        }
+        const bool persistent = !b->h_tasks.empty() && !all_small;
         // side streams: every streamed class when they overlap the persistent launch, else all
         // but the first, which follows the persistent launch on the batch's stream
         const int first_side = (b->overlap && persistent) ? 0 : 1;
@@ -223,11 +241,25 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
                                 b->stream));
             b->launches += 1;
         }
+        for (size_t i = 0; i < b->cls.size(); ++i) {
+            const auto &k = b->cls[i];
+            if (!res[i]) continue;
+            const cudaError_t e = launch_sweeps_resident(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, rp[i], b->d_status,
+                                                         (double)b->timeout_ns * 1e-9, b->stream, &b->launches);
+            if (e == cudaErrorNotSupported) {
+                // refused before this class's first launch: its sweeps one launch per half-sweep
+                b->no_resident = 1;
+                BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, k.cfg, b->stream, &b->launches));
+            } else {
+                BCK(b, e);
+            }
+        }
         if (first_side == 1 && nstreamed > 1) BCK(b, cudaEventRecord(b->ev[0], b->stream));
         // the streamed classes, each on its own stream: their short launches (a few
         // microseconds of work each) overlap instead of waiting for one another
-        for (const auto &k : b->cls) {
-            if (!k.streamed) continue;
+        for (size_t i = 0; i < b->cls.size(); ++i) {
+            const auto &k = b->cls[i];
+            if (!k.streamed || res[i]) continue;
             const int sj = si + (1 - first_side);  // side stream index + 1 (0: the batch's stream)
             cudaStream_t st = b->stream;
             if (sj > 0) {
@@ -289,11 +321,12 @@ int read_status(ising_batch *b)
     BCK(b, cudaMemcpyAsync(&st, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     BCK(b, cudaStreamSynchronize(b->stream));
     // status codes: 1 a group barrier of the batch kernel (or the first wait of a tensor-core
-    // correlation CTA) ran out, 2 and 3 later waits of the tensor-core correlation, 4 a copy
-    // wait of the fused sweep
+    // correlation CTA) ran out, 2 a later wait of the tensor-core correlation, 4 a copy wait of
+    // the fused sweep, 5 a wait of the resident sweep
     if (st == BATCH_STATUS_TIMEOUT)
         return bfail(b, ISING_ETIMEOUT, "a group barrier of the batch kernel or a correlation wait timed out");
     if (st == 4) return bfail(b, ISING_ETIMEOUT, "fused sweep of a streamed class: a bounded wait for a copy gave up");
+    if (st == 5) return bfail(b, ISING_ETIMEOUT, "resident sweep: a bounded wait for a neighbour's planes gave up");
     if (st) return bfail(b, ISING_ETIMEOUT, "tensor-core correlation: a bounded device-side wait gave up");
     return ISING_OK;
 }
@@ -307,6 +340,7 @@ int assign_modes(ising_batch *b)
     for (auto &k : b->cls) {
         k.streamed = b->stream_min_L > 0 && k.L >= b->stream_min_L && k.L % 256 == 0;
         k.cfg = default_sweep_config(k.L, k.R);
+        k.automatic = 1;
         if (k.streamed) continue;
         const Geom g = make_geom(k.L);
         for (int r = 0; r < k.R; ++r)
@@ -430,7 +464,7 @@ int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *r
     int64_t rec_off = 0, der_off = 0;
     for (int c = 0; c < nclass; ++c) {
         BatchClass k{L[c], replicas[c], seeds[c], nullptr, rec_off, der_off, 0, SweepConfig{VARIANT_WORD, 0, 0, 0},
-                     nullptr, nullptr};
+                     1, nullptr, nullptr};
         const int64_t bytes = lattice_bytes(L[c]) * replicas[c];
         if (cudaMalloc(&k.lat, (size_t)bytes) != cudaSuccess) {
             b->cls.push_back(k);
@@ -458,8 +492,8 @@ int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *r
     }
     b->nlat = der_off;
     b->rec_words = rec_off;
-    if (cudaMalloc(&b->d_status, sizeof(int)) != cudaSuccess) return bail(ISING_ENOMEM);
-    if (cudaMemsetAsync(b->d_status, 0, sizeof(int), b->stream) != cudaSuccess) return bail(ISING_ECUDA);
+    if (cudaMalloc(&b->d_status, 4 * sizeof(int)) != cudaSuccess) return bail(ISING_ENOMEM);
+    if (cudaMemsetAsync(b->d_status, 0, 4 * sizeof(int), b->stream) != cudaSuccess) return bail(ISING_ECUDA);
     if (cudaMalloc(&b->d_rec, sizeof(int64_t) * (size_t)b->rec_words) != cudaSuccess) return bail(ISING_ENOMEM);
     if (cudaMalloc(&b->d_der, sizeof(double) * 4 * (size_t)b->nlat) != cudaSuccess) return bail(ISING_ENOMEM);
     if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return bail(ISING_ECUDA);
@@ -716,7 +750,11 @@ int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out)
         if ((s = ising_batch_set_class_opts(b, c, &dflt)) != ISING_OK || (s = segment_ms(&ms_dflt)) != ISING_OK ||
             (s = ising_batch_set_class_opts(b, c, &alone)) != ISING_OK || (s = segment_ms(&ms_alone)) != ISING_OK)
             break;
-        if (ms_dflt <= ms_alone) s = ising_batch_set_class_opts(b, c, &dflt);
+        // a size with a resident sweep keeps its default, which runs it in all but the shortest
+        // segments: the probes are too short to show it
+        ResidentPlan rp{};
+        if (ms_dflt <= ms_alone || resident_plan(b->cls[c].L, b->cls[c].R, b->sms, &rp))
+            s = ising_batch_set_class_opts(b, c, &dflt);
     }
     // the streamed classes beside the persistent launch, or after it
     if (s == ISING_OK && !b->h_tasks.empty() && ising_batch_streamed_classes(b) > 0) {
@@ -751,6 +789,7 @@ int ising_batch_set_class_opts(ising_batch *b, int cls, const ising_opts *o)
         return bfail(b, ISING_ENOMEM, "second store of the fused sweep");
     }
     k.cfg = cfg;
+    k.automatic = o->variant == 0;
     if (b->gexec) {  // the cached schedule graph holds the old kernels
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;

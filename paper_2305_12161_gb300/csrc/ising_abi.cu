@@ -33,7 +33,8 @@ struct ising_ctx {
     int64_t *rec_dev = nullptr;  // R records
     double *der_dev = nullptr;   // R x 4
     uint32_t *xt = nullptr;      // tensor-core correlation, L >= 512: bit-transposed lattice (lazy)
-    int *dev_err = nullptr;      // set by a device-side bounded wait that gave up
+    int *dev_err = nullptr;      // [0] set by a device-side bounded wait that gave up, [1, 2] counters of
+                                 // the resident sweep's barriers
     int xt_refused = 0;          // that scratch could not be allocated (AUTO then measures without it)
     double wait_timeout_s = 2.0; // bound of each device-side wait (tensor-core path)
     int inject_stall = 0;        // test hook: the next tensor-core measurement loses one load
@@ -41,6 +42,7 @@ struct ising_ctx {
     int poisoned = 0;
     int64_t launches = 0;
     SweepConfig cfg{};
+    int no_resident = 0;  // the device refused the resident sweep's launch
     DcbGeom dcb{};  // double-checkerboard blocks (scheme DOUBLE)
     RadialPlans *radial = nullptr;  // cuFFT plans of the radial measurement (first use)
     char err[256] = {0};
@@ -282,6 +284,18 @@ Footprint footprint_of(int L, int R, const ising_opts &o, const SweepConfig &cfg
 
 }  // namespace
 
+// The automatic variant's resident sweep for a call of n sweeps (k_resident.cu): no plan for the size,
+// too few sweeps, a device that refused it, or a capture that would need a cooperative launch: the
+// context's half-sweep kernel instead.
+static bool use_resident(const ising_ctx *c, int64_t n, ResidentPlan *rp)
+{
+    if (c->opts.variant != 0 || c->opts.form != ISING_FORM_PACKED || c->opts.scheme != ISING_SCHEME_CHECKERBOARD ||
+        c->no_resident || !resident_plan(c->L, c->R, device_sms(), rp) || n < rp->min_n)
+        return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return rp->cluster || (cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone);
+}
+
 extern "C" {
 
 int64_t ising_footprint_bytes(int L, int R, const ising_opts *opts)
@@ -404,6 +418,17 @@ int ising_sweep(ising_ctx *c, int64_t n)
     if (n == 0) return ISING_OK;
     DeviceGuard dg(c->device);
     cudaError_t e;
+    ResidentPlan rp{};
+    if (use_resident(c, n, &rp)) {
+        e = launch_sweeps_resident(c->lat, c->L, c->R, c->seed, c->opts.tie, c->t, n, c->opts.cycle, rp, c->dev_err,
+                                   c->wait_timeout_s, c->stream, &c->launches);
+        if (e == cudaSuccess) {
+            c->t += n;
+            return ISING_OK;
+        }
+        if (e != cudaErrorNotSupported) return cuda_fail(c, e, "sweep launch");
+        c->no_resident = 1;
+    }
     if (c->opts.scheme == ISING_SCHEME_DOUBLE)
         e = launch_sweeps_dcb(c->lat, c->L, c->R, c->seed, c->opts.tie, c->t, n, c->opts.cycle, c->dcb, c->stream,
                               &c->launches);
@@ -431,6 +456,7 @@ static int check_device_waits(ising_ctx *c)
     CK(c, cudaMemcpyAsync(&h, c->dev_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     if (h == 4) return fail(c, ISING_ETIMEOUT, "fused sweep: a bounded wait for a copy gave up");
+    if (h == 5) return fail(c, ISING_ETIMEOUT, "resident sweep: a bounded wait for a neighbour's planes gave up");
     if (h) return fail(c, ISING_ETIMEOUT, "tensor-core correlation: a bounded device-side wait gave up (code %d)", h);
     return ISING_OK;
 }
@@ -723,6 +749,8 @@ int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base,
     if (o.form != ISING_FORM_PACKED || o.scheme != ISING_SCHEME_CHECKERBOARD) return ISING_EINVAL;
     std::vector<SweepConfig> cands;
     cands.push_back(SweepConfig{VARIANT_WORD, 0, 0, 0});
+    ResidentPlan rp{};
+    if (resident_plan(L, replicas, device_sms(), &rp)) cands.push_back(SweepConfig{VARIANT_AUTO, 0, 0, 0});
     const int tzs[] = {4, 8, 16, 32, 64};
     if (L >= 256 && L % 256 == 0) {
         const int W4 = L / 256;
@@ -764,16 +792,18 @@ int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base,
         cudaEvent_t a = nullptr, b = nullptr;
         float ms = 0.f;
         bool ok = cudaEventCreate(&a) == cudaSuccess && cudaEventCreate(&b) == cudaSuccess;
-        ok = ok && ising_sweep(ctx, 2) == ISING_OK;
+        // the automatic variant's resident sweep is timed over a call long enough to use it
+        const int mcs = c.variant == VARIANT_AUTO ? std::max(probe_mcs, 64) : probe_mcs;
+        ok = ok && ising_sweep(ctx, c.variant == VARIANT_AUTO ? mcs : 2) == ISING_OK;
         ok = ok && cudaEventRecord(a, ctx->stream) == cudaSuccess;
-        ok = ok && ising_sweep(ctx, probe_mcs) == ISING_OK;
+        ok = ok && ising_sweep(ctx, mcs) == ISING_OK;
         ok = ok && cudaEventRecord(b, ctx->stream) == cudaSuccess;
         ok = ok && cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&ms, a, b) == cudaSuccess;
         if (a) cudaEventDestroy(a);
         if (b) cudaEventDestroy(b);
         ising_destroy(ctx);
         if (!ok) return ISING_ECUDA;
-        const double per = ms / probe_mcs;
+        const double per = ms / mcs;
         if (c.variant == VARIANT_ZFUSE) {
             if (per < best_fused_ms) best_fused_ms = per, best_fused = oc;
         } else if (per < best_single_ms) {

@@ -59,6 +59,36 @@ int mixed_first(uint64_t S, uint32_t t);
 // Menger-sponge start of iteration k for every replica (padding words must be zero).
 cudaError_t launch_init_menger(uint32_t *lat, int L, int R, uint64_t seed, int k, cudaStream_t s);
 
+// Many sweeps per launch with the lattices resident in shared memory (k_resident.cu); false where
+// no such plan exists.  err: four ints, the first an error code (5: a bounded wait gave up), the next
+// two zero counters of the kernel's barriers, left zero.
+struct ResidentPlan {
+    bool cluster;    // thread-block clusters (L = 64, 128), else a cooperative grid
+    int ctas;        // CTAs per lattice
+    int groups;      // Philox groups per thread and half-sweep
+    int per_launch;  // lattices per launch
+    int min_n;       // sweeps per call from which it is the faster way
+};
+bool resident_plan(int L, int R, int sms, ResidentPlan *out);
+// Returns cudaErrorNotSupported, with nothing enqueued, where the device cannot hold the launch.
+cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
+                                   int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
+                                   int64_t *launches);
+
+// Scope around a cooperative launch on stream s: it runs after the previous one of this process on
+// the current device (nothing is ordered while s is being captured).
+class CoopOrder {
+public:
+    explicit CoopOrder(cudaStream_t s);
+    ~CoopOrder();
+    CoopOrder(const CoopOrder &) = delete;
+    CoopOrder &operator=(const CoopOrder &) = delete;
+
+private:
+    cudaStream_t stream;
+    int dev = -1;
+};
+
 // Double-checkerboard update (Supp. Methods I A): blocks of bx*by*bz sites, red blocks
 // (block indices summing to an even number) then blue ones; inside a block the sites of one
 // parity, then the other.  A block row is the block's x-range of one row (y,z) of one

@@ -1,0 +1,93 @@
+"""Sweeps with the lattices resident in shared memory (the automatic variant of L = 64 .. 512) against
+the half-sweep kernels: every size class and exchange (cluster, grid, rows of whole and of split
+uint4), replica counts around a launch's capacity, calls below, at and above the length from which the
+resident sweep runs, both cycles, every rule.  Spins are compared bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ising():
+    from paper_2305_12161_gb300 import ising as m
+    m.lib()
+    return m
+
+
+def _same(ising, L, R, calls, t0=0, seed=5, **kw):
+    with ising.Ising(L, replicas=R, seed=seed, **kw) as a, \
+            ising.Ising(L, replicas=R, seed=seed, variant=ising.VARIANT_WORD, **kw) as b:
+        a.t = t0
+        b.t = t0
+        for n in calls:
+            a.sweep(n)
+            b.sweep(n)
+            for r in sorted({0, 1 % R, R // 2, R - 1}):
+                assert np.array_equal(a.get_packed(r), b.get_packed(r)), (L, R, n, r)
+        assert a.t == b.t
+
+
+@pytest.mark.parametrize("cycle", [0, 1])
+@pytest.mark.parametrize("L,R", [(64, 1), (64, 19), (64, 39), (64, 160), (64, 320), (128, 1), (128, 19), (128, 20),
+                                 (128, 80), (192, 1), (192, 13), (256, 1), (256, 2), (256, 9), (256, 10), (320, 1),
+                                 (320, 4), (384, 2), (448, 1), (512, 1), (512, 2)])
+def test_equals_the_half_sweep_kernel(ising, L, R, cycle):
+    _same(ising, L, R, [1, 2, 3, 12, 13], cycle=cycle)
+
+
+@pytest.mark.parametrize("rule", [1, 2])
+@pytest.mark.parametrize("L", [64, 128, 192, 256, 512])
+def test_other_rules(ising, L, rule):
+    _same(ising, L, 2, [13, 12], tie=rule)
+
+
+def test_counter_near_its_end_and_long_calls(ising):
+    _same(ising, 64, 3, [40], t0=2**32 - 1 - 40, seed=2**64 - 2)
+    _same(ising, 64, 2, [5000])
+    _same(ising, 256, 2, [4100])
+
+
+@pytest.mark.parametrize("L,n", [(64, 17), (192, 6)])
+def test_equals_the_oracle(ising, L, n):
+    want = oracle.init(L, 7, 0)
+    oracle.sweeps(want, 0, n, 7)
+    with ising.Ising(L, replicas=1, seed=7) as q:
+        q.sweep(n)
+        assert np.array_equal(q.get_spins(0), want)
+
+
+def test_contexts_on_several_streams(ising):
+    import torch
+    spec = [(256, 3, 1), (512, 1, 2), (320, 2, 3), (64, 5, 4), (256, 1, 5)]
+    ctx = [ising.Ising(L, replicas=R, seed=s, stream=torch.cuda.Stream()) for L, R, s in spec]
+    for _ in range(20):
+        for q in ctx:
+            q.sweep(16)
+    for (L, R, s), q in zip(spec, ctx):
+        q.sync()
+        with ising.Ising(L, replicas=R, seed=s) as p:
+            p.sweep(320)
+            for r in range(R):
+                assert np.array_equal(p.get_packed(r), q.get_packed(r)), (L, r)
+        q.destroy()
+
+
+@pytest.mark.parametrize("L", [64, 256])
+def test_captured_sweep_replays(ising, L):
+    import torch
+    stream = torch.cuda.Stream()
+    with ising.Ising(L, replicas=2, seed=9, stream=stream) as q, ising.Ising(L, replicas=2, seed=9) as p:
+        q.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            q.sweep(12)
+        for _ in range(2):  # the graph repeats the draws of t = 0 .. 11
+            with torch.cuda.stream(stream):
+                g.replay()
+            p.t = 0
+            p.sweep(12)
+        for r in range(2):
+            assert np.array_equal(p.get_packed(r), q.get_packed(r))
