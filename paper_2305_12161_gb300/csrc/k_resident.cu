@@ -258,7 +258,7 @@ struct ResGArgs {
     uint4 *lat;      // first replica of the launch
     int64_t nw4;
     uint64_t seed;
-    int L, W, P, NC;
+    int P, NC;
     uint32_t t0;
     int n, mixed;
     unsigned *bar;   // two zero counters: arrivals, departures (left zero)
@@ -336,22 +336,28 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned round, int 
 // as in k_resident.  W4 = 0 (any other row width): the plane's words in order between a copy of the
 // last row before the first and a copy of the first row after the last, so that rows y - 1 and
 // y + 1 of a group, which may straddle rows, are plain offsets.
-__host__ __device__ inline int resg_front(int W) { return (W + 3) / 4; }           // uint4 before row 0
-__host__ __device__ inline int resg_plane(int L, int W, int W4)
-{
-    return W4 > 0 ? L * W4 : L * W / 4 + 2 * resg_front(W);
-}
+template <int W>
+struct ResPlane {  // L = 64 W
+    static constexpr int L = 64 * W, U = 16 * W * W;              // groups of a plane
+    static constexpr int W4 = W == 4 ? 1 : (W == 8 ? 2 : 0);
+    static constexpr int F = W4 > 0 ? 0 : (W + 3) / 4;            // uint4 before row 0
+    static constexpr int PU = U + 2 * F;                          // uint4 of a plane
+};
+static int resg_plane(int W) { return 16 * W * W + (W == 4 || W == 8 ? 0 : 2 * ((W + 3) / 4)); }
 
 // Thread tid updates group slot tid % U of the four planes zl .. zl + 3, zl = 4 (tid / U).
-template <int RULE, int W4>
+// Sizes are compile-time constants: with the row width at run time a group took 76 ALU and 49 multiply
+// instructions at L = 512, now 74 and 40 (8.4 us per sweep, now 7.8).
+template <int RULE, int W>
 __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
 {
     extern __shared__ __align__(16) uint4 gsm_res[];  // [2][P][plane]
     __shared__ int s_fail;  // first step at which a poll gave up
     __shared__ uint2 keys[10];
-    const int tid = threadIdx.x, P = ra.P, L = ra.L, W = ra.W, NC = ra.NC;
-    const int U = L * W / 4, PU = resg_plane(L, W, W4), F = W4 > 0 ? 0 : resg_front(W);
-    const int hs = U / 2;  // W4: slots of one row parity
+    using RP = ResPlane<W>;
+    constexpr int L = RP::L, U = RP::U, PU = RP::PU, F = RP::F, W4 = RP::W4;
+    constexpr int hs = U / 2;  // W4: slots of one row parity
+    const int tid = threadIdx.x, P = ra.P, NC = ra.NC;
     const int c = (int)blockIdx.x % NC, r = (int)blockIdx.x / NC;
     const uint64_t S = ra.seed + (uint64_t)r;
     uint4 *lat = ra.lat + 2 * (int64_t)r * ra.nw4;
@@ -568,12 +574,12 @@ static cudaError_t res_rule(ResArgs ra, int R, int G, cudaStream_t s)
     }
 }
 
-template <int RULE, int W4>
+template <int RULE, int W>
 static cudaError_t launch_resg(const ResGArgs &ra, int R, cudaStream_t s)
 {
-    const int U = ra.L * ra.W / 4;
-    const size_t smem = (size_t)2 * ra.P * resg_plane(ra.L, ra.W, W4) * sizeof(uint4);
-    auto kern = k_resident_grid<RULE, W4>;
+    constexpr int U = ResPlane<W>::U;
+    const size_t smem = (size_t)2 * ra.P * ResPlane<W>::PU * sizeof(uint4);
+    auto kern = k_resident_grid<RULE, W>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
@@ -590,12 +596,16 @@ static cudaError_t launch_resg(const ResGArgs &ra, int R, cudaStream_t s)
 }
 
 template <int RULE>
-static cudaError_t resg_rule(const ResGArgs &ra, int R, cudaStream_t s)
+static cudaError_t resg_rule(const ResGArgs &ra, int W, int R, cudaStream_t s)
 {
-    switch (ra.L) {
-    case 256: return launch_resg<RULE, 1>(ra, R, s);
-    case 512: return launch_resg<RULE, 2>(ra, R, s);
-    default: return launch_resg<RULE, 0>(ra, R, s);
+    switch (W) {
+    case 3: return launch_resg<RULE, 3>(ra, R, s);
+    case 4: return launch_resg<RULE, 4>(ra, R, s);
+    case 5: return launch_resg<RULE, 5>(ra, R, s);
+    case 6: return launch_resg<RULE, 6>(ra, R, s);
+    case 7: return launch_resg<RULE, 7>(ra, R, s);
+    case 8: return launch_resg<RULE, 8>(ra, R, s);
+    default: return cudaErrorInvalidValue;
     }
 }
 
@@ -607,8 +617,6 @@ static cudaError_t resident_grid(uint32_t *lat, int L, int R, uint64_t seed, int
     ra.lat = reinterpret_cast<uint4 *>(lat);
     ra.nw4 = g.nw / 4;
     ra.seed = seed;
-    ra.L = L;
-    ra.W = g.W;
     ra.NC = NC;
     ra.P = L / NC;
     ra.t0 = (uint32_t)t0;
@@ -618,9 +626,9 @@ static cudaError_t resident_grid(uint32_t *lat, int L, int R, uint64_t seed, int
     ra.err = err;
     ra.timeout_ns = (uint64_t)(timeout_s * 1e9);
     switch (rule) {
-    case TIE_GLAUBER: return resg_rule<TIE_GLAUBER>(ra, R, s);
-    case TIE_ALWAYS: return resg_rule<TIE_ALWAYS>(ra, R, s);
-    default: return resg_rule<TIE_NEVER>(ra, R, s);
+    case TIE_GLAUBER: return resg_rule<TIE_GLAUBER>(ra, g.W, R, s);
+    case TIE_ALWAYS: return resg_rule<TIE_ALWAYS>(ra, g.W, R, s);
+    default: return resg_rule<TIE_NEVER>(ra, g.W, R, s);
     }
 }
 
@@ -688,8 +696,8 @@ CoopOrder::~CoopOrder()
 // Grid, L = 192 .. 512: a launch holds as many lattices as its CTAs fit one per SM, P = 4, 8, ...
 // planes each; the P with the least rounds x time per sweep, the time being linear in the groups of
 // a CTA above a floor of latency (measured: rows of whole uint4 1.2 + 1.35e-3 per group, at least
-// 3.4 us; other rows 3.5 + 2.05e-3, at least 4.9).  Per sweep: 8 x 256^3 6.7 us against 14.3 of the
-// half-sweep kernel, one 512^3 8.4 against 14.8 (four: 33.5 against 39.9), 2 x 320^3 10.1 against 28.7.
+// 3.4 us; other rows 3.5 + 2.05e-3, at least 4.9).  Per sweep: 8 x 256^3 6.6 us against 14.3 of the
+// half-sweep kernel, one 512^3 7.8 against 14.8 (four: 31.2 against 39.9), 2 x 320^3 9.5 against 28.7.
 //
 // min_n: sweeps per call from which the load, the two grid barriers and the write-back (16 - 18 us
 // a round) are earned back.
@@ -709,14 +717,15 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
         return true;
     }
     if (L < 192 || L > 512 || L % 64 != 0) return false;
-    const int W = L / 64, W4 = L == 256 ? 1 : (L == 512 ? 2 : 0), U = L * W / 4;
+    const int W = L / 64, U = L * W / 4;
+    const bool whole = W == 4 || W == 8;  // rows of whole uint4
     double best = 1e300;
     for (int P = 4; P <= L / 2; P += 4) {
         if (L % P != 0 || P * U / 4 > 1024 || L / P > sms) continue;
-        if ((size_t)2 * P * resg_plane(L, W, W4) * sizeof(uint4) > 220 * 1024) continue;
+        if ((size_t)2 * P * resg_plane(W) * sizeof(uint4) > 220 * 1024) continue;
         const int per = std::min(R, sms / (L / P));
         const int rounds = (R + per - 1) / per;
-        const double us = W4 > 0 ? std::max(3.4, 1.2 + 1.35e-3 * P * U) : std::max(4.9, 3.5 + 2.05e-3 * P * U);
+        const double us = whole ? std::max(3.4, 1.2 + 1.35e-3 * P * U) : std::max(4.9, 3.5 + 2.05e-3 * P * U);
         if (rounds * us < best) {
             best = rounds * us;
             p.ctas = L / P;
