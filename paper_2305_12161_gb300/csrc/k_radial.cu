@@ -17,10 +17,14 @@
 //   6. k_radial_finish: bin means, C(b) = sum_G / (N n_b), S(b) = sum_P / (N n_b), and the
 //      length l at which C first crosses c for r <= L/2.
 //
-// Binning: the lanes of a warp take consecutive elements of a row, whose bins form runs; a
-// segmented warp scan sums each run and its last lane adds the sum to the CTA's bins in
-// shared memory with one atomic, and the CTA's bins go to the global sums at the end.  The
-// number of vectors per bin does not depend on the state and is counted once per context.
+// Binning: reflecting any component leaves a vector's bin.  So one thread takes the values at
+// (x, +-dy, +-dz) together (and (L - x, +-dy, +-dz) for lags): one bin computation for up to eight.  The
+// integers of a lag pass are summed over a walk of the thread along dy or dz while the bin stays, then
+// added to the CTA's bins in shared memory.  The modes' |F|^2 are summed in their precision over runs
+// of equal bins of 32 consecutive x (a warp scan per row), then in double over the four rows and the
+// bins.  (With a bin, a scan and a 64-bit atomic per value and row these passes took 0.80 and 0.94 ms
+// at L = 512 for 1.07 and 0.54 GB, the count 0.69; now 0.43, 0.36 and 0.06.)
+// The number of vectors per bin does not depend on the state and is counted once per context.
 // The transform buffer and cuFFT's work area stay allocated in the context between calls.
 //
 // Bins: components as minimal images, squared length D, bin round(sqrt(D)) computed exactly
@@ -44,9 +48,16 @@ __host__ __device__ __forceinline__ int isqrt_exact(int v)
     return s;
 }
 
-__host__ __device__ __forceinline__ int bin_of(int D) { return (isqrt_exact(4 * D) + 1) >> 1; }
-
-__device__ __forceinline__ int min_image(int j, int L) { return j <= L / 2 ? j : j - L; }
+// round(sqrt(D)): the b with b^2 - b < D <= b^2 + b (D < 2^24, so the estimate is off by at most one).
+__device__ __forceinline__ int bin_of(int D)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"((float)D));
+    int b = __float2int_rn(r);
+    b += D > b * b + b;
+    b -= (b > 0) & (D <= b * b - b);
+    return b;
+}
 
 template <typename T>
 struct Cx;
@@ -71,56 +82,37 @@ struct Pair<double> {
 };
 
 constexpr int RAD_THREADS = 256;
+constexpr int RAD_FOLD_THREADS = 544;  // 0 .. L/2 of L = 1024 in one pass, of L = 2048 in two
 
 }  // namespace
 
 int64_t radial_nbins(int L) { return (int64_t)((isqrt_exact(3 * L * L) + 1) >> 1) + 1; }
 
-// Loops below run over rows (y, z) in a grid-stride loop and over the row's elements with
-// the CTA's warps, lane = consecutive element, so no 64-bit division is needed per element.
-
-// 1. A thread takes a pair of sites (x = 2k, 2k+1) of a row: both share compressed index k,
-// one on each sublattice.
+// 1. A warp takes a row, a lane four consecutive sites, two of each sublattice (rows are aligned
+// to a pair only, so two stores of a pair each).
 template <typename T>
-__global__ void k_unpack_real(const uint32_t *lat_r, T *buf, Geom g, int64_t P)
+__global__ void __launch_bounds__(RAD_THREADS) k_unpack_real(const uint32_t *lat_r, T *buf, Geom g, int64_t P)
 {
-    const int L = g.L, H = L / 2;
-    for (int row = blockIdx.x; row < L * L; row += gridDim.x) {
-        const int y = row % L, z = row / L;
-        const int q0 = (y + z) & 1;  // sublattice of x = 2k
-        const uint32_t *r0 = lat_r + (int64_t)q0 * g.nw + (int64_t)row * g.W;
-        const uint32_t *r1 = lat_r + (int64_t)(1 - q0) * g.nw + (int64_t)row * g.W;
-        T *dst = buf + (int64_t)row * P;
-        for (int k = threadIdx.x; k < H; k += blockDim.x) {
-            const int bit = k & 31;
-            const uint32_t w0 = __ldg(r0 + (k >> 5)), w1 = __ldg(r1 + (k >> 5));
-            typename Pair<T>::type v;  // one aligned store of the two sites (rows of even length)
-            v.x = ((w0 >> bit) & 1u) ? T(1) : T(-1);
-            v.y = ((w1 >> bit) & 1u) ? T(1) : T(-1);
-            *reinterpret_cast<typename Pair<T>::type *>(dst + 2 * k) = v;
+    const int L = g.L, Q = L / 4;  // L is a multiple of 4
+    const int lane = threadIdx.x & 31, nwarp = gridDim.x * (RAD_THREADS / 32);
+    for (int row = blockIdx.x * (RAD_THREADS / 32) + (threadIdx.x >> 5); row < L * L; row += nwarp) {
+        const int z = row / L, y = row - z * L;
+        const int64_t q0 = (y + z) & 1;  // sublattice of even x
+        const uint32_t *r0 = lat_r + q0 * g.nw + (int64_t)row * g.W, *r1 = lat_r + (1 - q0) * g.nw + (int64_t)row * g.W;
+        typename Pair<T>::type *dst = reinterpret_cast<typename Pair<T>::type *>(buf + (int64_t)row * P);
+#pragma unroll 4
+        for (int k = lane; k < Q; k += 32) {
+            const int bit = 2 * (k & 15);  // compressed index 2 k
+            const uint32_t w0 = __ldg(r0 + (k >> 4)) >> bit, w1 = __ldg(r1 + (k >> 4)) >> bit;
+            typename Pair<T>::type a, b;
+            a.x = (w0 & 1u) ? T(1) : T(-1);
+            a.y = (w1 & 1u) ? T(1) : T(-1);
+            b.x = (w0 & 2u) ? T(1) : T(-1);
+            b.y = (w1 & 2u) ? T(1) : T(-1);
+            dst[2 * k] = a;
+            dst[2 * k + 1] = b;
         }
     }
-}
-
-// The 32 lanes hold (bin b, value v) of consecutive elements (b < 0: no element).  Runs of
-// equal b are summed by a segmented inclusive scan in type V; each run's last lane adds its
-// sum to hist[b] (type H).
-template <typename V, typename H>
-__device__ __forceinline__ void run_add(int b, V v, H *hist)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int bp = __shfl_up_sync(FULL, b, 1);
-    const unsigned heads = __ballot_sync(FULL, lane == 0 || bp != b);
-    const int seg = __popc(heads & (FULL >> (31 - lane)));  // run number of this lane
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const V vo = __shfl_up_sync(FULL, v, d);
-        const int so = __shfl_up_sync(FULL, seg, d);
-        if (lane >= d && so == seg) v += vo;
-    }
-    const int bn = __shfl_down_sync(FULL, b, 1);
-    if ((lane == 31 || bn != b) && b >= 0) atomicAdd(&hist[b], (H)v);
 }
 
 template <typename V>
@@ -138,92 +130,179 @@ __device__ __forceinline__ void flush_bins(const V *h, V *global, int nb)
         if (h[i] != V(0)) atomicAdd(&global[i], h[i]);
 }
 
+// v added to a bin in shared memory.  A 64-bit integer bin is two 32-bit words and the carry is taken
+// from the first word's old value: native 32-bit atomics, where a 64-bit one is a compare-and-swap loop.
+__device__ __forceinline__ void bin_add(unsigned long long *bin, unsigned long long v)
+{
+    uint32_t *w = reinterpret_cast<uint32_t *>(bin);
+    const uint32_t lo = (uint32_t)v, old = atomicAdd(w, lo);
+    const uint32_t hi = (uint32_t)(v >> 32) + (uint32_t)(old + lo < old);
+    if (hi) atomicAdd(w + 1, hi);
+}
+
+template <typename V>
+struct BinRun {
+    V *hist;
+    V sum = V(0);
+    int bin = -1;
+    __device__ __forceinline__ void add(int b, V v)
+    {
+        if (b != bin) {
+            if (bin >= 0) bin_add(&hist[bin], sum);
+            bin = b;
+            sum = v;
+        } else {
+            sum += v;
+        }
+    }
+    __device__ __forceinline__ void flush()
+    {
+        if (bin >= 0) bin_add(&hist[bin], sum);
+        bin = -1;
+    }
+};
+
+// Rows (+-dy, +-dz) of one fold: n of them, row indices y + L z.
+struct FoldRows {
+    int n;
+    int row[4];
+};
+__device__ __forceinline__ FoldRows fold_rows(int L, int dy, int dz)
+{
+    const int yb = (dy == 0 || 2 * dy == L) ? -1 : L - dy, zb = (dz == 0 || 2 * dz == L) ? -1 : L - dz;
+    FoldRows f;
+    f.n = (yb < 0 ? 1 : 2) * (zb < 0 ? 1 : 2);
+    f.row[0] = dy + L * dz;
+    f.row[1] = yb >= 0 ? yb + L * dz : dy + L * zb;
+    f.row[2] = dy + L * zb;
+    f.row[3] = yb + L * zb;
+    return f;
+}
+
+// Calls fn(rows, x, D) for every fold of the CTA's share, x = thread (0 .. L/2, and past it up to a whole
+// warp), and end() after each run of folds.  A work item is `chunk` folds: for SHORT along the smaller
+// of dy and dz (fewer changes of bin), else along dy, which keeps rows that are also written next to
+// each other (k_power is slower by a fifth along the smaller one).
+template <bool SHORT, class Fn, class End>
+__device__ __forceinline__ void fold_walk(int L, int chunk, Fn fn, End end)
+{
+    const int H = L / 2, nc = H / chunk + 1, per = SHORT ? 2 * nc : nc;
+    for (int item = blockIdx.x; item < (H + 1) * per; item += gridDim.x) {
+        const int M = item / per, rest = item - M * per;
+        const bool ymajor = SHORT && rest >= nc;  // y the larger (strictly), else z
+        const int m0 = (rest - (ymajor ? nc : 0)) * chunk;
+        const int m1 = min(!SHORT ? H + 1 : (ymajor ? M : M + 1), m0 + chunk);
+        if (m0 >= m1) continue;
+        for (int x = threadIdx.x; (x & ~31) <= H; x += blockDim.x) {
+#pragma unroll 2
+            for (int m = m0; m < m1; ++m)
+                fn(ymajor ? fold_rows(L, M, m) : fold_rows(L, m, M), x, x * x + m * m + M * M);
+            end();
+        }
+    }
+}
+
 // 3. |F|^2 per mode of the half spectrum; S sums per bin; (P, 0) written back.
 template <typename T>
-__global__ void __launch_bounds__(RAD_THREADS) k_power(typename Cx<T>::type *F, int L, int nb, double *sumS)
+__global__ void __launch_bounds__(RAD_FOLD_THREADS) k_power(typename Cx<T>::type *F, int L, int chunk, int nb,
+                                                             double *sumS)
 {
     extern __shared__ double hs[];
     zero_bins(hs, nb);
-    const int H1 = L / 2 + 1;
+    const int H = L / 2, H1 = H + 1;
+    const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    for (int row = blockIdx.x; row < L * L; row += gridDim.x) {
-        const int ny = min_image(row % L, L), nz = min_image(row / L, L);
-        const int dyz = ny * ny + nz * nz;
-        typename Cx<T>::type *Fr = F + (int64_t)row * H1;
-        for (int x0 = threadIdx.x & ~31; x0 < H1; x0 += blockDim.x) {
-            const int nx = x0 + lane;
-            int b = -1;
-            T wp = T(0);  // single precision stays in fp32 up to the per-run double add
-            if (nx < H1) {
-                const typename Cx<T>::type f = Fr[nx];
-                const T p = f.x * f.x + f.y * f.y;
-                wp = (nx == 0 || nx == L / 2) ? p : T(2) * p;  // 0 < nx < L/2: also the partner -q
-                b = bin_of(nx * nx + dyz);
-                typename Cx<T>::type o;
-                o.x = p;
-                o.y = T(0);
-                Fr[nx] = o;
+    fold_walk<false>(
+        L, chunk,
+        [&](const FoldRows &r, int x, int D) {
+            const bool in = x <= H;
+            T v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                v[i] = T(0);
+                if (i < r.n && in) {
+                    typename Cx<T>::type *p = F + (int64_t)r.row[i] * H1 + x;
+                    const typename Cx<T>::type f = *p;
+                    const T q = f.x * f.x + f.y * f.y;
+                    v[i] = (x == 0 || x == H) ? q : T(2) * q;  // 0 < x < L/2: also the partner -q
+                    typename Cx<T>::type o;
+                    o.x = q;
+                    o.y = T(0);
+                    *p = o;
+                }
             }
-            run_add<T, double>(b, wp, hs);
-        }
-    }
+            // runs of equal bins among the 32 lanes; single precision stays in fp32 up to a run's sum
+            const int b = in ? bin_of(D) : -1;
+            const int bp = __shfl_up_sync(FULL, b, 1);
+            const unsigned heads = __ballot_sync(FULL, lane == 0 || bp != b);
+            const int start = 31 - __clz(heads & (FULL >> (31 - lane)));  // first lane of this lane's run
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const T w = __shfl_up_sync(FULL, v[i], d);
+                    if (lane - d >= start) v[i] += w;
+                }
+            const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
+            if (last && in) atomicAdd(&hs[b], (double)v[0] + (double)v[1] + (double)v[2] + (double)v[3]);
+        },
+        [] {});
     flush_bins(hs, sumS, nb);
 }
 
 // 5. G(k) = rint(g/N) per lag, summed per bin in int64.
 template <typename T>
-__global__ void __launch_bounds__(RAD_THREADS) k_radial_corr(const T *g, int L, int64_t P, int nb, double invN,
-                                                             unsigned long long *sumG, unsigned long long *inexact)
+__global__ void __launch_bounds__(RAD_FOLD_THREADS) k_radial_corr(const T *g, int L, int chunk, int64_t P, int nb,
+                                                                   double invN, unsigned long long *sumG,
+                                                                   unsigned long long *inexact)
 {
     extern __shared__ unsigned long long hg[];
     zero_bins(hg, nb);
-    const int lane = threadIdx.x & 31;
+    const int H = L / 2;
     unsigned long long bad = 0ull;
-    for (int row = blockIdx.x; row < L * L; row += gridDim.x) {
-        const int dy = min_image(row % L, L), dz = min_image(row / L, L);
-        const int dyz = dy * dy + dz * dz;
-        const T *gr = g + (int64_t)row * P;
-        for (int x0 = threadIdx.x & ~31; x0 < L; x0 += blockDim.x) {
-            const int x = x0 + lane;
-            int b = -1;
-            unsigned long long G = 0ull;
-            if (x < L) {
-                const int dx = min_image(x, L);
-                b = bin_of(dx * dx + dyz);
-                // invN is a power of two, so the scaling is exact in either precision
-                const T v = gr[x] * (T)invN;
-                const T r = rint(v);
-                if (fabs(v - r) > T(0.25)) ++bad;
-                // two's complement: the unsigned sums wrap to the signed result
-                G = (fabs(r) < T(2147483520)) ? (unsigned long long)(long long)(int)r
-                                               : (unsigned long long)(long long)r;
+    BinRun<unsigned long long> run{hg};
+    fold_walk<true>(
+        L, chunk,
+        [&](const FoldRows &r, int x, int D) {
+            if (x > H) return;
+            const int xr = (x == 0 || x == H) ? -1 : L - x;
+            T f[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < r.n) f[i] = g[(int64_t)r.row[i] * P + x];
+                if (i < r.n && xr >= 0) f[4 + i] = g[(int64_t)r.row[i] * P + xr];
             }
-            run_add<unsigned long long, unsigned long long>(b, G, hg);
-        }
-    }
+            unsigned long long G = 0ull;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if ((i & 3) < r.n && (i < 4 || xr >= 0)) {
+                    const T v = f[i] * (T)invN;
+                    const T q = rint(v);
+                    if (fabs(v - q) > T(0.25)) ++bad;
+                    // two's complement: the unsigned sums wrap to the signed result
+                    G += (fabs(q) < T(2147483520)) ? (unsigned long long)(long long)(int)q
+                                                   : (unsigned long long)(long long)q;
+                }
+            run.add(bin_of(D), G);
+        },
+        [&]() { run.flush(); });
     flush_bins(hg, sumG, nb);
     if (bad) atomicAdd(inexact, bad);
 }
 
 // Vectors per bin (independent of the state; once per context).
-__global__ void __launch_bounds__(RAD_THREADS) k_radial_count(int L, int nb, unsigned long long *count)
+__global__ void __launch_bounds__(RAD_FOLD_THREADS) k_radial_count(int L, int chunk, int nb, unsigned long long *count)
 {
     extern __shared__ unsigned long long hc[];
     zero_bins(hc, nb);
-    const int lane = threadIdx.x & 31;
-    for (int row = blockIdx.x; row < L * L; row += gridDim.x) {
-        const int dy = min_image(row % L, L), dz = min_image(row / L, L);
-        const int dyz = dy * dy + dz * dz;
-        for (int x0 = threadIdx.x & ~31; x0 < L; x0 += blockDim.x) {
-            const int x = x0 + lane;
-            int b = -1;
-            if (x < L) {
-                const int dx = min_image(x, L);
-                b = bin_of(dx * dx + dyz);
-            }
-            run_add<unsigned long long, unsigned long long>(b, b >= 0 ? 1ull : 0ull, hc);
-        }
-    }
+    const int H = L / 2;
+    BinRun<unsigned long long> run{hc};
+    fold_walk<true>(
+        L, chunk,
+        [&](const FoldRows &r, int x, int D) {
+            if (x <= H) run.add(bin_of(D), (unsigned long long)(r.n * ((x == 0 || x == H) ? 1 : 2)));
+        },
+        [&]() { run.flush(); });
     flush_bins(hc, count, nb);
 }
 
@@ -372,7 +451,12 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const unsigned grid = (unsigned)(sms * 4);
+    // threads for x = 0 .. L/2 in as few passes as 544 allow; folds per work item so that there are a
+    // few items per resident CTA
+    const int nx = L / 2 + 1, passes = (nx + RAD_FOLD_THREADS - 1) / RAD_FOLD_THREADS;
+    const int fold_threads = ((nx + passes - 1) / passes + 31) / 32 * 32;
+    const unsigned grid = (unsigned)(sms * std::max(1, 2048 / fold_threads));
+    const int chunk = std::max(1, std::min(16, nx * nx / (4 * (int)grid)));
     const size_t smem = (size_t)nb * sizeof(double);
     if (!p->count) {
         if ((e = cudaMallocAsync((void **)&p->count, sizeof(unsigned long long) * nb, s)) != cudaSuccess) {
@@ -383,11 +467,11 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
         if ((e = cudaFuncSetAttribute(k_radial_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
             cudaSuccess)
             return e;
-        k_radial_count<<<grid, RAD_THREADS, smem, s>>>(L, nb, p->count);
+        k_radial_count<<<grid, fold_threads, smem, s>>>(L, chunk, nb, p->count);
         if (launches) *launches += 1;
     }
 
-    k_unpack_real<T><<<grid, RAD_THREADS, 0, s>>>(lat_r, reinterpret_cast<T *>(p->buf), g, P);
+    k_unpack_real<T><<<(unsigned)(sms * 16), RAD_THREADS, 0, s>>>(lat_r, reinterpret_cast<T *>(p->buf), g, P);
     cufftHandle f = p->fwd[prec], iv = p->inv[prec];
     if ((cs = cufftSetStream(f, s)) != CUFFT_SUCCESS || (cs = cufftSetStream(iv, s)) != CUFFT_SUCCESS ||
         (cs = cufftSetWorkArea(f, p->wk)) != CUFFT_SUCCESS || (cs = cufftSetWorkArea(iv, p->wk)) != CUFFT_SUCCESS) {
@@ -405,7 +489,7 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
     }
     if ((e = cudaFuncSetAttribute(k_power<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
-    k_power<T><<<grid, RAD_THREADS, smem, s>>>(reinterpret_cast<C *>(p->buf), L, nb, sumS);
+    k_power<T><<<grid, fold_threads, smem, s>>>(reinterpret_cast<C *>(p->buf), L, chunk, nb, sumS);
     if (prec)
         cs = cufftExecZ2D(iv, reinterpret_cast<cufftDoubleComplex *>(p->buf), reinterpret_cast<cufftDoubleReal *>(p->buf));
     else
@@ -418,7 +502,7 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
     if ((e = cudaFuncSetAttribute(k_radial_corr<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
         cudaSuccess)
         return e;
-    k_radial_corr<T><<<grid, RAD_THREADS, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, P, nb, invN, sumG,
+    k_radial_corr<T><<<grid, fold_threads, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, chunk, P, nb, invN, sumG,
                                                        inexact);
     k_radial_finish<<<1, 256, 0, s>>>(L, nb, c, sumG, sumS, p->count, inexact, out, cnt);
     if (launches) *launches += 4;  // own kernels; the two cuFFT executions are library launches
