@@ -434,7 +434,7 @@ int ising_sweep(ising_ctx *c, int64_t n)
                               &c->launches);
     else if (c->opts.form == ISING_FORM_PLAIN)
         e = launch_sweeps_plain(c->plain, c->L, c->R, c->seed, c->opts.tie, c->t, n, c->opts.cycle, c->stream,
-                                &c->launches);
+                                &c->launches, c->cfg.pdl != 0);
     else if (c->cfg.variant == VARIANT_ZFUSE)
         e = launch_sweeps_fused(&c->lat, &c->lat_alt, c->L, c->R, c->seed, c->opts.tie, c->t, n, c->opts.cycle,
                                 c->cfg.tile_z, c->cfg.depth, c->dev_err, c->wait_timeout_s, c->stream, &c->launches,

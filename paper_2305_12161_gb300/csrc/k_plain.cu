@@ -56,6 +56,7 @@ __global__ void k_init_plain(int8_t *P, Geom g, uint64_t seed)
 template <int RULE>
 __global__ void k_sweep_plain(int8_t *P, Geom g, int q, uint32_t t, uint64_t S)
 {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int L = g.L;
@@ -128,6 +129,7 @@ __device__ __forceinline__ uint32_t fma_add(uint32_t a, uint32_t one, uint32_t b
 template <int RULE, int CH>
 __global__ void __launch_bounds__(256) k_sweep_plain16(int8_t *P, int L, int q, uint32_t t, uint64_t S, uint32_t one)
 {
+    pdl_enter();
     constexpr uint32_t FULL = 0xffffffffu, M2 = 0x02020202u, B7 = 0x80808080u;
     constexpr int NW = 4 * CH;            // 32-bit words of a thread
     const int W = L >> 4;                 // chunks per row (<= 256)
@@ -222,9 +224,11 @@ __global__ void __launch_bounds__(256) k_sweep_plain16(int8_t *P, int L, int q, 
     }
 }
 
+// Every half-sweep is launched with programmatic dependent launch (pdl): its CTAs are scheduled while the
+// previous one drains and wait for its completion in pdl_enter.
 template <int RULE>
-static void sweeps_plain_rule(int8_t *plain, const Geom &g, int R, uint64_t seed, int64_t t0, int64_t n, int cycle,
-                              cudaStream_t s, int64_t *launches)
+static cudaError_t sweeps_plain_rule(int8_t *plain, const Geom &g, int R, uint64_t seed, int64_t t0, int64_t n,
+                                     int cycle, cudaStream_t s, int64_t *launches, bool pdl)
 {
     const int64_t N = (int64_t)g.L * g.L * g.L;
     int64_t blocks = (g.nw + 7) / 8;
@@ -235,34 +239,40 @@ static void sweeps_plain_rule(int8_t *plain, const Geom &g, int R, uint64_t seed
     const dim3 grid16((unsigned)std::max(1, (g.L / rpc + 7) / 8), (unsigned)g.L);
     const int rpc2 = g.L >= 32 ? 256 / (g.L / 32) : 1;  // 32 bytes per thread
     const dim3 grid32((unsigned)std::max(1, (g.L / rpc2 + 7) / 8), (unsigned)g.L);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = g.L % 32 == 0 ? grid32 : (g.L % 16 == 0 ? grid16 : dim3((unsigned)blocks));
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    lc.attrs = attr;
+    lc.numAttrs = pdl ? 1 : 0;
     for (int64_t k = 0; k < n; ++k) {
         const uint32_t t = (uint32_t)(t0 + k);
         for (int h = 0; h < 2; ++h)
             for (int r = 0; r < R; ++r) {  // one launch per lattice
                 const uint64_t S = seed + (uint64_t)r;
                 const int q = cycle ? (mixed_first(S, t) ^ h) : h;
-                if (g.L % 32 == 0)
-                    k_sweep_plain16<RULE, 2><<<grid32, 256, 0, s>>>(plain + (int64_t)r * N, g.L, q, t, S, 1u);
-                else if (g.L % 16 == 0)
-                    k_sweep_plain16<RULE, 1><<<grid16, 256, 0, s>>>(plain + (int64_t)r * N, g.L, q, t, S, 1u);
-                else
-                    k_sweep_plain<RULE><<<(unsigned)blocks, 256, 0, s>>>(plain + (int64_t)r * N, g, q, t, S);
+                int8_t *p = plain + (int64_t)r * N;
+                const cudaError_t e = g.L % 32 == 0   ? cudaLaunchKernelEx(&lc, k_sweep_plain16<RULE, 2>, p, g.L, q, t, S, 1u)
+                                      : g.L % 16 == 0 ? cudaLaunchKernelEx(&lc, k_sweep_plain16<RULE, 1>, p, g.L, q, t, S, 1u)
+                                                      : cudaLaunchKernelEx(&lc, k_sweep_plain<RULE>, p, g, q, t, S);
+                if (e != cudaSuccess) return e;
             }
     }
     if (launches) *launches += 2 * n * R;
+    return cudaSuccess;
 }
 
 cudaError_t launch_sweeps_plain(int8_t *plain, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
-                                int cycle, cudaStream_t s, int64_t *launches)
+                                int cycle, cudaStream_t s, int64_t *launches, bool pdl)
 {
     if (n <= 0) return cudaSuccess;
     const Geom g = make_geom(L);
     switch (rule) {
-    case TIE_GLAUBER: sweeps_plain_rule<TIE_GLAUBER>(plain, g, R, seed, t0, n, cycle, s, launches); break;
-    case TIE_ALWAYS: sweeps_plain_rule<TIE_ALWAYS>(plain, g, R, seed, t0, n, cycle, s, launches); break;
-    default: sweeps_plain_rule<TIE_NEVER>(plain, g, R, seed, t0, n, cycle, s, launches); break;
+    case TIE_GLAUBER: return sweeps_plain_rule<TIE_GLAUBER>(plain, g, R, seed, t0, n, cycle, s, launches, pdl);
+    case TIE_ALWAYS: return sweeps_plain_rule<TIE_ALWAYS>(plain, g, R, seed, t0, n, cycle, s, launches, pdl);
+    default: return sweeps_plain_rule<TIE_NEVER>(plain, g, R, seed, t0, n, cycle, s, launches, pdl);
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------------

@@ -132,7 +132,7 @@ cudaError_t launch_radial(RadialPlans *p, const uint32_t *lat_r, int L, int prec
 // ---- plain form: one byte per spin, replica r at plain + r*N. --------------------
 cudaError_t launch_init_plain(int8_t *plain, int L, int R, uint64_t seed, cudaStream_t s);
 cudaError_t launch_sweeps_plain(int8_t *plain, int L, int R, uint64_t seed, int rule, int64_t t0,
-                                int64_t n_mcs, int cycle, cudaStream_t s, int64_t *launches);
+                                int64_t n_mcs, int cycle, cudaStream_t s, int64_t *launches, bool pdl);
 // plain -> packed (for the shared measurement kernels) and back.
 cudaError_t launch_pack(const int8_t *plain, uint32_t *lat, int L, int R, cudaStream_t s);
 cudaError_t launch_unpack(const uint32_t *lat, int8_t *plain, int L, int R, cudaStream_t s);
