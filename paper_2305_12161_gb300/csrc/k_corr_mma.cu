@@ -104,20 +104,35 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, uint64
 
 // Transposes the 32 x 32 bit block whose row i is lane i's word (five stages, each swapping the
 // off-diagonal half-blocks of size j between lanes r and r ^ j): lane i then holds bit i of
-// every row.
-__device__ __forceinline__ uint32_t transpose32_lane(uint32_t v, int lane)
-{
-    const uint32_t FULL = 0xffffffffu;
-    const uint32_t lows[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const int j = 16 >> k;
-        const uint32_t low = lows[k];
-        const uint32_t t = __shfl_xor_sync(FULL, v, j);
-        v = (lane & j) ? ((v & ~low) | ((t & ~low) >> j)) : ((v & low) | ((t & low) << j));
+// every row.  What depends on the lane (byte selectors, rotations, masks) is worked out once: a
+// stage is a shuffle and a byte permute, or a shuffle, a rotation and a select.
+struct Transpose32 {
+    uint32_t sel16, sel8, rot4, rot2, rot1, keep4, keep2, keep1;
+    __device__ explicit Transpose32(int lane)
+    {
+        sel16 = (lane & 16) ? 0x3276u : 0x5410u;
+        sel8 = (lane & 8) ? 0x3715u : 0x6240u;
+        rot4 = (lane & 4) ? 28u : 4u;
+        rot2 = (lane & 2) ? 30u : 2u;
+        rot1 = (lane & 1) ? 31u : 1u;
+        keep4 = (lane & 4) ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
+        keep2 = (lane & 2) ? 0xCCCCCCCCu : 0x33333333u;
+        keep1 = (lane & 1) ? 0xAAAAAAAAu : 0x55555555u;
     }
-    return v;
-}
+    __device__ __forceinline__ static uint32_t part(uint32_t v, int j, uint32_t rot, uint32_t keep)
+    {
+        const uint32_t t = __shfl_xor_sync(0xffffffffu, v, j);
+        return (v & keep) | (__funnelshift_l(t, t, rot) & ~keep);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t v) const
+    {
+        v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 16), sel16);
+        v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 8), sel8);
+        v = part(v, 4, rot4, keep4);
+        v = part(v, 2, rot2, keep2);
+        return part(v, 1, rot1, keep1);
+    }
+};
 
 // The 32 spins of one word as e2m1 values (32 lines of one position): nibble m of out word j is
 // bit 4 m + j, sign bit set for a down spin.
@@ -155,6 +170,7 @@ __global__ void __launch_bounds__(256) k_lines_x(const uint32_t *lat, Geom g, ui
     const uint32_t z = row / (uint32_t)L, y = row - z * (uint32_t)L;
     const bool odd = (y + z) & 1u;
     const int64_t at = (int64_t)row * W + kw0;
+    const Transpose32 tr(lane);
     uint32_t v0[4] = {0, 0, 0, 0}, v1[4] = {0, 0, 0, 0};
     if (W % 4 == 0) {
         const uint4 a = __ldg(reinterpret_cast<const uint4 *>(S0 + at));
@@ -171,8 +187,8 @@ __global__ void __launch_bounds__(256) k_lines_x(const uint32_t *lat, Geom g, ui
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint32_t e = transpose32_lane(odd ? v1[i] : v0[i], lane);  // x = 2 (32 kw + lane)
-        const uint32_t o = transpose32_lane(odd ? v0[i] : v1[i], lane);  // x + 1
+        const uint32_t e = tr(odd ? v1[i] : v0[i]);  // x = 2 (32 kw + lane)
+        const uint32_t o = tr(odd ? v0[i] : v1[i]);  // x + 1
         sm[(64 * i + 2 * lane) * 9 + b] = e;
         sm[(64 * i + 2 * lane + 1) * 9 + b] = o;
     }
@@ -222,7 +238,9 @@ struct GramArgs {
     int64_t *rec;
     int64_t RL, nw;            // record length; words per sublattice
     int L, W;
-    int nsb, nunits, split, nitems;
+    int nsb, nunits, nitems;
+    int split_x, split_yz;     // slices of the lines: x axis, y and z axes
+    int nrep;
     int stage_bytes, nst;      // ring of stages
     int ncols, scale_col;      // tensor memory: columns allocated, first of the 32 scale columns
     int *err;
@@ -507,17 +525,20 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    pdl_enter();  // what precedes touches no global memory and overlaps the previous kernel's end
 
     const int nk = (int)((int64_t)L * L / GB_LINES);
     uint32_t g0 = 0;     // stages used by earlier items (ring position and phase)
     uint32_t nitem = 0;  // items done: phase of `done`
     for (int item = blockIdx.x; item < ga.nitems; item += gridDim.x, ++nitem) {
-        const GramUnit un = gram_unit(item % ga.nunits, ga.nsb, L);
-        int rest = item / ga.nunits;
-        const int sl = rest % ga.split;
-        rest /= ga.split;
-        const int axis = rest % 3, r = rest / 3;
-        const int c0 = (int)((int64_t)nk * sl / ga.split), c1 = (int)((int64_t)nk * (sl + 1) / ga.split);
+        const int items_x = ga.nrep * ga.split_x * ga.nunits, items_y = ga.nrep * ga.split_yz * ga.nunits;
+        const int axis = item < items_x ? 0 : (item < items_x + items_y ? 1 : 2);
+        const int split = axis == 0 ? ga.split_x : ga.split_yz;
+        int rest = item - (axis == 0 ? 0 : (axis == 1 ? items_x : items_x + items_y));
+        const GramUnit un = gram_unit(rest % ga.nunits, ga.nsb, L);
+        rest /= ga.nunits;
+        const int r = rest / split, sl = rest - r * split;
+        const int c0 = (int)((int64_t)nk * sl / split), c1 = (int)((int64_t)nk * (sl + 1) / split);
         const int n = c1 - c0;
         const uint32_t *S0 = ga.lat + 2 * (int64_t)r * ga.nw, *S1 = S0 + ga.nw;
         const bool bad_first = ga.inject && blockIdx.x == 0 && nitem == 0;
@@ -541,12 +562,13 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
                     const bool xA = wr >= un.rb;
                     const int xr = xA ? wr - un.rb : wr;  // first of the 64 rows in its region
                     const int kw = ((xA ? un.j0 : un.s0) + xr) >> 6, b0 = 4 * (ws & 1);
+                    const Transpose32 tr(lane);
                     ReadXL rd(S0, S1, L, W, kw, b0, lane, c0 + set, nsets);
                     ok = fill_stages(
                         fl, g0, set, nsets, n, rd,
                         [&](uint32_t v[8], uint4 x[8]) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) x[i] = expand_e2m1(transpose32_lane(v[i], lane));
+                            for (int i = 0; i < 8; ++i) x[i] = expand_e2m1(tr(v[i]));
                         },
                         [&](uint32_t base, uint4 x[8]) {
 #pragma unroll
@@ -716,8 +738,15 @@ static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaSt
     auto kern = k_gram_bits<PW, MINB, READS>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, 32 * (PW + 1), smem, s>>>(ga);
-    return cudaGetLastError();
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3(32 * (PW + 1));
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kern, ga);
 }
 
 // rec: records initialised to D = N / 2 (r >= 1), M = -N, B = 3 N / 2.  scratch: 2 L^3 bytes for
@@ -766,17 +795,22 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
                 k_lines_yz<<<dim3((unsigned)(L / 32), (unsigned)L, (unsigned)(2 * nr)), 256, 0, s>>>(ga.lat, g, scratch,
                                                                                                      ga.rep_words);
         }
-        // slices of the lines: the count whose rounds of items over the CTAs take the fewest stages,
-        // counting an item's start and read-back as 8 stages
-        const int64_t base = (int64_t)nr * 3 * ga.nunits;
+        // slices of the lines: the counts whose items take the fewest stages over the CTAs, counting an
+        // item's start and read-back as 8 stages, and a stage of the x axis as 1.5 where the kernel
+        // transposes it (so that axis is cut finer: eight L = 256 replicas 54 -> X256 us)
+        ga.nrep = nr;
+        const int64_t base = (int64_t)nr * ga.nunits;
+        const double wx = lines ? 1.0 : 1.5;
         double best = 1e300;
         for (int sp = 1; sp <= std::min(nk, 64); ++sp) {
-            const int64_t items = base * sp;
+            const int sx = std::min(nk, (int)(wx * sp + 0.5));
+            const int64_t items = base * (sx + 2 * sp);
+            const double tx = wx * ((nk + sx - 1) / sx) + 8.0, ty = (double)((nk + sp - 1) / sp) + 8.0;
             const int64_t rounds = (items + slots - 1) / slots;
-            const double cost = (double)rounds * ((double)((nk + sp - 1) / sp) + 8.0);
-            if (cost < best * 0.999) best = cost, ga.split = sp;
+            const double cost = (double)rounds * std::max(tx, ty);
+            if (cost < best * 0.999) best = cost, ga.split_x = sx, ga.split_yz = sp;
         }
-        ga.nitems = (int)(base * ga.split);
+        ga.nitems = (int)(base * (ga.split_x + 2 * ga.split_yz));
         ga.inject = inject && r0 == 0;
         const int grid = std::min(ga.nitems, slots);
         cudaError_t e;

@@ -47,14 +47,90 @@ __device__ __forceinline__ uint4 xshift(const uint4 &C, uint32_t edge_left_w, ui
     return X;
 }
 
+// Both halves of a product: as one wide multiply (WIDE) or as two (mul_hi_lo).  The multiplier is busy
+// 4.2 cycles per warp with the wide or the high one and 2.1 with the low one.
+template <bool WIDE>
+__device__ __forceinline__ void fused_mul(uint32_t a, uint32_t b, uint32_t &hi, uint32_t &lo)
+{
+    if constexpr (WIDE)
+        asm("{\n.reg .b64 p;\nmul.wide.u32 p, %2, %3;\nmov.b64 {%1, %0}, p;\n}\n" : "=r"(hi), "=r"(lo) : "r"(a), "r"(b));
+    else
+        mul_hi_lo(a, b, hi, lo);
+}
+
+// What a draw needs of one replica and phase.  One replica per launch: kernel parameters, read as
+// constant-bank operands.  Several: a copy in shared memory, keys two rounds to a uint4 (k0, k1 of
+// round 2 i, then of 2 i + 1), so that a draw reads five uint4 and one for the lead: a constant bank
+// indexed by the block cost a load per word.
+struct FusedDrawSm {
+    uint4 keys[5];
+    uint4 lead[2];  // x0_2, x2_2, x2_3 of phases A and B
+};
+
+template <bool WIDE>
+__device__ __forceinline__ U4 fused_draw(uint32_t c0, uint32_t x0_2, uint32_t x2_2, uint32_t x2_3, const uint4 *keys)
+{
+    const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
+    uint32_t h0, l0, h1, l1;
+    const uint32_t k10 = keys[0].y, k02 = keys[1].x;
+    fused_mul<WIDE>(M0, c0, h0, l0);
+    const uint32_t a2 = h0 ^ k10, a3 = l0;
+    fused_mul<WIDE>(M1, a2, h1, l1);
+    const uint32_t b0 = h1 ^ x0_2, b1 = l1, b2 = a3 ^ x2_2;
+    fused_mul<WIDE>(M0, b0, h0, l0);
+    fused_mul<WIDE>(M1, b2, h1, l1);
+    U4 o{h1 ^ b1 ^ k02, l1, h0 ^ x2_3, l0};
+    auto round = [&](uint32_t ka, uint32_t kb) {
+        fused_mul<WIDE>(M0, o.x, h0, l0);
+        fused_mul<WIDE>(M1, o.z, h1, l1);
+        o.x = h1 ^ o.y ^ ka;
+        o.z = h0 ^ o.w ^ kb;
+        o.y = l1;
+        o.w = l0;
+    };
+    round(keys[1].z, keys[1].w);
+#pragma unroll
+    for (int i = 2; i < 5; ++i) {
+        const uint4 k = keys[i];
+        round(k.x, k.y);
+        round(k.z, k.w);
+    }
+    return o;
+}
+
+// philox4x32_10_lead with the product form chosen
+template <bool WIDE>
+__device__ __forceinline__ U4 fused_draw(uint32_t c0, const PhiloxLead &ld, const PhiloxKeys &k)
+{
+    const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
+    uint32_t h0, l0, h1, l1;
+    fused_mul<WIDE>(M0, c0, h0, l0);
+    const uint32_t a2 = h0 ^ k.k1[0], a3 = l0;
+    fused_mul<WIDE>(M1, a2, h1, l1);
+    const uint32_t b0 = h1 ^ ld.x0_2, b1 = l1, b2 = a3 ^ ld.x2_2;
+    fused_mul<WIDE>(M0, b0, h0, l0);
+    fused_mul<WIDE>(M1, b2, h1, l1);
+    U4 o{h1 ^ b1 ^ k.k0[2], l1, h0 ^ ld.x2_3, l0};
+#pragma unroll
+    for (int i = 3; i < 10; ++i) {
+        fused_mul<WIDE>(M0, o.x, h0, l0);
+        fused_mul<WIDE>(M1, o.z, h1, l1);
+        o.x = h1 ^ o.y ^ k.k0[i];
+        o.z = h0 ^ o.w ^ k.k1[i];
+        o.y = l1;
+        o.w = l0;
+    }
+    return o;
+}
+
 // New spins of one uint4, as new_spins4 without the tie test: Glauber draws the group's
 // Philox word from the launch's constant first rounds (the same word as philox4x32_10 of
 // the counter (group, t, q, 0)).  The adders come before the draw, as in new_spins4: with
 // the draw first the kernel ran 3% slower.
-template <int RULE>
+template <int RULE, class Draw>
 __device__ __forceinline__ uint4 fused_spins4(const uint4 &s, const uint4 &C, const uint4 &X, const uint4 &ym,
                                               const uint4 &yp, const uint4 &zm, const uint4 &zp, uint32_t group,
-                                              const PhiloxLead &ld, const PhiloxKeys &keys)
+                                              Draw draw)
 {
     const uint32_t s1x = C.x ^ X.x ^ ym.x, c1x = maj3(C.x, X.x, ym.x);
     const uint32_t s1y = C.y ^ X.y ^ ym.y, c1y = maj3(C.y, X.y, ym.y);
@@ -66,7 +142,7 @@ __device__ __forceinline__ uint4 fused_spins4(const uint4 &s, const uint4 &C, co
     const uint32_t s2w = yp.w ^ zm.w ^ zp.w, c2w = maj3(yp.w, zm.w, zp.w);
     uint4 tau;
     if constexpr (RULE == TIE_GLAUBER) {
-        const U4 o = philox4x32_10_lead(group, ld, keys);
+        const U4 o = draw(group);
         tau = make_uint4(s.x ^ o.x, s.y ^ o.y, s.z ^ o.z, s.w ^ o.w);
     } else if constexpr (RULE == TIE_ALWAYS) {
         tau = make_uint4(~s.x, ~s.y, ~s.z, ~s.w);
@@ -197,6 +273,11 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
     uint64_t *full = reinterpret_cast<uint64_t *>(anew + 3 * NEW);  // [NS]
     pdl_enter();
     const FusedRep &rp = fa.rep[MR == 1 ? 0 : blockIdx.y];
+    // wide products: 426 -> 420 us per sweep at L = 2048, 481 -> 466 in the first tiling there (81 -> 74
+    // at L = 1024); not for the balanced tiling of shorter rows (66.5 -> 67.1) nor with the keys in shared
+    // memory
+    constexpr bool WIDE = MR == 1 && (!BAL || W4 == 8);
+    __shared__ __align__(16) FusedDrawSm s_draw;
     const int L = fa.L;
     const int tid = threadIdx.x;
     const int nty = (L + TYO - 1) / TYO;
@@ -235,6 +316,26 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
         copy_rows(dst, rp.Bcur + wrapL(z0 - 2 + g) * plane4, y0 - 2, RB, mbar);
         if (g >= 2) copy_rows(dst + 16u * NB, rp.Acur + wrapL(z0 - 3 + g) * plane4, y0 - 1, RA, mbar);
     };
+    if constexpr (MR > 1) {
+        if (tid < 5) {
+            s_draw.keys[tid] = make_uint4(rp.keys.k0[2 * tid], rp.keys.k1[2 * tid], rp.keys.k0[2 * tid + 1],
+                                          rp.keys.k1[2 * tid + 1]);
+        } else if (tid < 7) {
+            const PhiloxLead &ld = tid == 5 ? rp.leadA : rp.leadB;
+            s_draw.lead[tid - 5] = make_uint4(ld.x0_2, ld.x2_2, ld.x2_3, 0u);
+        }
+    }
+    auto draw_of = [&](const int ph, const PhiloxLead &ld) {  // draws of phase A (ph 0) or B (1)
+        return [&, ph](uint32_t group) -> U4 {
+            if constexpr (MR > 1) {
+                const uint4 l = s_draw.lead[ph];
+                return fused_draw<false>(group, l.x, l.y, l.z, s_draw.keys);
+            } else {
+                return fused_draw<WIDE>(group, ld, rp.keys);
+            }
+        };
+    };
+    const auto drawA = draw_of(0, rp.leadA), drawB = draw_of(1, rp.leadB);
     if (tid == 0) {
         s_fail = 0x7fffffff;
         for (int i = 0; i < NS; ++i)
@@ -298,7 +399,7 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
             const uint32_t e = __shfl_sync(FULL, P ? bc.x : bc.w, P ? srcr : srcl, W4);
             const uint4 X = xshift(bc, e, e, P);
             a0 = fused_spins4<RULE>(S2[NB + rN], bc, X, S1[rB - W4], S1[rB + W4], bm, S2[rB],
-                                                (uint32_t)oA, rp.leadA, rp.keys);
+                                                (uint32_t)oA, drawA);
             An[rN] = a0;
             if (bown && k >= 1 && k <= TZ) rp.Anxt[oA] = a0;
         }
@@ -310,7 +411,7 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
             const uint32_t e = __shfl_sync(HMASK, ph ? hbc.x : hbc.w, ph ? srcr : srcl, W4);
             const uint4 X = xshift(hbc, e, e, ph);
             An[hN] = fused_spins4<RULE>(S2[NB + hN], hbc, X, S1[hB - W4], S1[hB + W4], S0[hB], S2[hB],
-                                                    (uint32_t)(oA + dh), rp.leadA, rp.keys);
+                                                    (uint32_t)(oA + dh), drawA);
         }
         // B on plane zB = zA - 1, own column: new A of planes zB - 1, zB, zB + 1 are in the
         // new-A slots of steps k - 2 and k - 1, and a0
@@ -321,8 +422,7 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
             const uint32_t e = __shfl_sync(FULL, P ? a1.x : a1.w, P ? srcr : srcl, W4);
             const uint4 X = xshift(a1, e, e, P);
             const int32_t oB = oA >= plane4 ? oA - plane4 : oA - plane4 + vol4;
-            const uint4 nb = fused_spins4<RULE>(bm, a1, X, A1[rNm], A1[rNp], A2[rN], a0, (uint32_t)oB, rp.leadB,
-                                                rp.keys);
+            const uint4 nb = fused_spins4<RULE>(bm, a1, X, A1[rNm], A1[rNp], A2[rN], a0, (uint32_t)oB, drawB);
             if (bown) rp.Bnxt[oB] = nb;
         }
         oA += plane4;

@@ -25,6 +25,7 @@ __device__ __forceinline__ int64_t rec_len(int L) { return 3 + 3 * (int64_t)(L /
 // the sum of the axes' D_a(1).
 __global__ void k_rec_init(int64_t *rec, int L, int R, int64_t t, int corr)
 {
+    pdl_enter();
     const int64_t RL = rec_len(L);
     const int64_t H1 = L / 2 + 1;
     const int64_t half_n = (int64_t)L * L * L / 2;
@@ -407,7 +408,15 @@ cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int cor
     const int64_t RL = 3 + 3 * (int64_t)(L / 2 + 1);
     int64_t nb = (RL * R + 255) / 256;
     if (nb > 4096) nb = 4096;
-    k_rec_init<<<(unsigned)nb, 256, 0, s>>>(rec, L, R, t, corr);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)nb);
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute attr[1] = {pdl_attribute()};
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    const cudaError_t ie = cudaLaunchKernelEx(&lc, k_rec_init, rec, L, R, t, corr);
+    if (ie != cudaSuccess) return ie;
     if (corr == CORR_TENSOR) {  // M, B and D_a(r) in one pass
         if (!err || !gram_supported(L)) return cudaErrorInvalidValue;
         if (launches) *launches += 1;
