@@ -318,6 +318,17 @@ __device__ __forceinline__ uint4 new_spins4(const uint4 &s, const uint4 &C, cons
                       maj3(c1z, c2z, maj3(s1z, s2z, tau.z)), maj3(c1w, c2w, maj3(s1w, s2w, tau.w)));
 }
 
+// x-neighbour words (other than C itself) of the 128 sites of uint4 C with the direction p of each
+// lane, e the edge word of the adjacent uint4: bit k - 1 (p = 0) or k + 1.  A warp with one direction
+// shifts without the five selects.
+__device__ __forceinline__ uint4 xshift_lane(const uint4 &C, uint32_t e, bool p)
+{
+    const uint32_t n = p ? 31u : 1u;
+    const uint32_t a0 = p ? C.x : e, a1 = p ? C.y : C.x, a2 = p ? C.z : C.y, a3 = p ? C.w : C.z, a4 = p ? e : C.w;
+    return make_uint4(__funnelshift_l(a0, a1, n), __funnelshift_l(a1, a2, n), __funnelshift_l(a2, a3, n),
+                      __funnelshift_l(a3, a4, n));
+}
+
 // Neighbour words of storage word sw of sublattice q, read from the other sublattice
 // array O.  X is the x-neighbour that is not at the same k (k-1 for p = 0, k+1 for
 // p = 1; the other x-neighbour is C itself), Ym/Yp/Zm/Zp are the rows y-1, y+1,

@@ -244,8 +244,11 @@ static constexpr size_t fused_smem_bytes()
     return sizeof(uint4) * (size_t)(NS * T::SLOT + 3 * T::RA * W4) + 8 * NS;
 }
 
-// Thread tid owns column cx = lane % W4 of one thread row (the rows of a warp share their
-// parity, as in the half-sweep kernel) for both sublattices.  Copy group g (one TMA bulk copy
+// Thread tid owns column cx = lane % W4 of one thread row for both sublattices.  W4 = 8: the rows of a
+// warp share their parity, as in the half-sweep kernel, so the x direction is the warp's.  Shorter
+// rows: a warp's rows are consecutive and the direction is the lane's (five selects more per update);
+// rows two apart made every shared-memory access a two-way bank conflict (two 1024^3: 141 -> 127 us per
+// sweep, in 32-plane blocks 140 -> 122; one 66.4 -> 64.9).  Copy group g (one TMA bulk copy
 // per contiguous run of rows, issued by thread 0, completing on the mbarrier of slot g % NS)
 // brings B plane z0 - 2 + g and, for g >= 2, old-A plane z0 - 1 + (g - 2); step k reads the
 // slots of groups k, k + 1, k + 2 and, after the step's barrier, thread 0 refills the slot of
@@ -348,7 +351,9 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
 
     const int warp = tid >> 5, lane = tid & 31;
     const int cx = lane & (W4 - 1);
-    const int ty = (warp >> 1) * 2 * RW + (warp & 1) + 2 * (lane / W4);  // thread row
+    constexpr bool MIX = W4 < 8;
+    const int ty = MIX ? warp * RW + lane / W4 : (warp >> 1) * 2 * RW + (warp & 1) + 2 * (lane / W4);  // thread row
+    const bool lp = MIX && ((lane / W4) & 1);  // this lane's row is odd: the other direction
     const int yrow = BAL ? y0 - 1 + ty : y0 + ty;
     const int32_t own = wrapL(yrow) * W4 + cx;
     const int rN = (BAL ? ty : ty + 1) * W4 + cx;  // own row in an A slot
@@ -372,6 +377,18 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
     bad |= !fused_mbar_wait(full0 + 8u, 0u, fa.timeout_ns);
     int g_done = bad ? -1 : 1;
     int32_t oA = wrapL(z0 - 1) * plane4 + own;  // plane zA, own column
+    // x-neighbour words of the lane's uint4 C; direction P of the warp's (MIX: of the even) rows
+    auto x_of = [&](const uint4 &C, auto Pc) -> uint4 {
+        constexpr int P = decltype(Pc)::value;
+        if constexpr (MIX) {
+            const bool p = P ? !lp : lp;
+            const uint32_t e = __shfl_sync(FULL, p ? C.x : C.w, p ? srcr : srcl, W4);
+            return xshift_lane(C, e, p);
+        } else {
+            const uint32_t e = __shfl_sync(FULL, P ? C.x : C.w, P ? srcr : srcl, W4);
+            return xshift(C, e, e, P);
+        }
+    };
     // one step: A on plane zA = z0 - 1 + k (tile rows and halo rows), then B on zA - 1
     auto step = [&](const int k, auto Pc) -> bool {
         constexpr int P = decltype(Pc)::value;
@@ -396,8 +413,7 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
         uint4 a0;
         {
             const uint4 bc = S1[rB];
-            const uint32_t e = __shfl_sync(FULL, P ? bc.x : bc.w, P ? srcr : srcl, W4);
-            const uint4 X = xshift(bc, e, e, P);
+            const uint4 X = x_of(bc, Pc);
             a0 = fused_spins4<RULE>(S2[NB + rN], bc, X, S1[rB - W4], S1[rB + W4], bm, S2[rB],
                                                 (uint32_t)oA, drawA);
             An[rN] = a0;
@@ -419,8 +435,7 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
             const uint4 *A1 = anew + na1 * NEW;  // step k - 1: plane zB
             const uint4 *A2 = anew + na2 * NEW;  // step k - 2: plane zB - 1
             const uint4 a1 = A1[rN];
-            const uint32_t e = __shfl_sync(FULL, P ? a1.x : a1.w, P ? srcr : srcl, W4);
-            const uint4 X = xshift(a1, e, e, P);
+            const uint4 X = x_of(a1, Pc);
             const int32_t oB = oA >= plane4 ? oA - plane4 : oA - plane4 + vol4;
             const uint4 nb = fused_spins4<RULE>(bm, a1, X, A1[rNm], A1[rNp], A2[rN], a0, (uint32_t)oB, drawB);
             if (bown) rp.Bnxt[oB] = nb;
@@ -430,8 +445,9 @@ __global__ void __launch_bounds__(256, MINB) k_mcs_fused(const __grid_constant__
         return true;
     };
     // x direction of A on plane zA at k = 0 (and of B on zA - 1): parity of yrow + zA + A,
-    // yrow's parity is the warp's (plus one in the balanced tiling); it alternates with k
-    const int p0 = ((warp & 1) + (BAL ? 1 : 0) + z0 - 1 + (int)A) & 1;
+    // yrow's parity is the warp's (MIX: of its even rows; plus one in the balanced tiling); it
+    // alternates with k
+    const int p0 = ((MIX ? 0 : (warp & 1)) + (BAL ? 1 : 0) + z0 - 1 + (int)A) & 1;
     bool ok = !__syncthreads_or(bad);
     if (ok) {
         // TZ + 2 steps in pairs; for odd TZ the last pair has one step

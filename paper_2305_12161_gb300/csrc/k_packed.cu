@@ -218,7 +218,9 @@ __global__ void __launch_bounds__(1024) k_sweep_zmarch(uint32_t *lat, Geom g, in
 // planes ahead into registers.  Philox round keys are computed once per thread.  The rows
 // a warp computes share their parity, so the direction of the x-neighbour shift (which
 // alternates with y + z) is the same for the whole warp; own-word pointer and Philox
-// counter advance by one plane per step.
+// counter advance by one plane per step.  That holds for W4 = 8; shorter rows two apart would make
+// every shared-memory access a two-way bank conflict, so there a warp's rows are consecutive and the
+// direction is the lane's (per sweep 8 x 256^3 14.5 -> 13.4 us, 512^3 15.0 -> 14.1, 1024^3 79.3 -> 77.5).
 template <int RULE, int W4>
 __global__ void __launch_bounds__(256) k_sweep_zfast(uint32_t *lat, Geom g, int q, uint32_t t, uint64_t seed, int TZ)
 {
@@ -253,8 +255,9 @@ __global__ void __launch_bounds__(256) k_sweep_zfast(uint32_t *lat, Geom g, int 
     // compute: the rows of a warp share their parity, so the x-neighbour direction (which
     // alternates with y + z) is uniform across the warp
     const int warp = tid >> 5, lane = tid & 31;
+    constexpr bool MIX = W4 < 8;
     const int cx = lane % W4;
-    const int ty = (warp >> 1) * 2 * RW + (warp & 1) + 2 * (lane / W4);
+    const int ty = MIX ? warp * RW + lane / W4 : (warp >> 1) * 2 * RW + (warp & 1) + 2 * (lane / W4);
     const int y = y0 + ty;
     const int64_t own = (int64_t)y * W4 + cx;  // own column within a plane
 
@@ -298,7 +301,10 @@ __global__ void __launch_bounds__(256) k_sweep_zfast(uint32_t *lat, Geom g, int 
         sA = sB;
         if (i + 2 < TZ) sB = sp[2 * plane4];
         uint4 X;
-        if (p == 0) {
+        if constexpr (MIX) {
+            const uint32_t *row = reinterpret_cast<const uint32_t *>(Oz + (ty + 1) * W4);
+            X = xshift_lane(cc, row[p ? 4 * cxr : 4 * cxl + 3], p != 0);
+        } else if (p == 0) {
             const uint32_t e = Oz[(ty + 1) * W4 + cxl].w;
             X.x = __funnelshift_l(e, cc.x, 1);
             X.y = __funnelshift_l(cc.x, cc.y, 1);
