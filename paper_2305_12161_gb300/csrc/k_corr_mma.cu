@@ -13,8 +13,9 @@
 // write them into the 128-byte swizzled shared-memory tiles that tcgen05.mma reads.  At
 // L = 2048 a measurement takes 10.8 ms against 21.1 with e4m3 operands staged through global
 // memory (8.6 GB written and re-read per axis, and half the tensor rate); eight L = 256 replicas
-// take 0.054 ms against 0.51 by bit counts, 512 of L = 64 0.04 against 0.28.  The issue loop bounds
-// it: a stage of four products (512 cycles of tensor work) takes 835 cycles at L = 1024.
+// take 0.054 ms against 0.51 by bit counts, 512 of L = 64 0.04 against 0.28.  Shared memory bounds
+// it at L = 2048: a stage of four products (512 cycles of tensor work) writes and reads 48 KB each, 768
+// cycles, and takes 990.
 //
 // Only the upper block triangle of G is computed (G is symmetric): an entry j < k stands for
 // both ordered pairs, i.e. for the distances k - j and L - (k - j).  B is the sum of the three
@@ -461,8 +462,11 @@ __device__ __forceinline__ bool fill_stages(const Fill &f, uint32_t g0, int set,
     return true;
 }
 
-// One CTA: the first PW warps fill the stages and afterwards read the accumulators, the last
-// warp issues the MMAs.  A stage holds 256 lines of every row of the unit; the (ra + rb) / 32
+// One CTA: the first PW warps fill the stages and afterwards read the accumulators, the last two
+// warps issue the MMAs, one stage each in turn: while one's products run, it commits them and the other
+// waits for its stage (four 512^3 0.28 -> 0.26 ms; at L = 2048 shared memory, written 48 and read 48 KB
+// per stage, binds and nothing changed).  The turn passes through an mbarrier between tcgen05 fences, so
+// the products reach the accumulators in the order of the stages.  A stage holds 256 lines of every row of the unit; the (ra + rb) / 32
 // warps of a set fill it, one row per lane, and as many sets as the PW warps hold work on successive
 // stages.  Each stage is written once and read by 4 (off-diagonal) or 8 MMAs of 128 x N x 64.
 //
@@ -477,12 +481,12 @@ __device__ __forceinline__ bool fill_stages(const Fill &f, uint32_t g0, int set,
 enum GramReads : int { GR_SMALL, GR_T, GR_XL, GR_ANY };  // XL + YZ1; T alone; XL + YZ4; all
 
 template <int PW, int MINB, int READS>
-__global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArgs ga)
+__global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArgs ga)
 {
-    constexpr int GB_THREADS = 32 * (PW + 1);
+    constexpr int GB_THREADS = 32 * (PW + 2);
     extern __shared__ __align__(1024) uint8_t gsm[];
     __shared__ int sacc[GB_SACC];
-    __shared__ __align__(8) uint64_t full[8], empty[8], done;
+    __shared__ __align__(8) uint64_t full[8], empty[8], turn[2], done;
     __shared__ uint32_t tmem_holder;
     __shared__ int flag, mma_pending, pops[2];  // up spins of the z axis's words, by item parity
 
@@ -502,7 +506,9 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[i])), "r"(GB_ARRIVE));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[i])));
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&done)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&turn[0])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&turn[1])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;" ::"r"(smem_u32(&done)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         flag = 1;
         mma_pending = 0;
@@ -530,6 +536,7 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
     const int nk = (int)((int64_t)L * L / GB_LINES);
     uint32_t g0 = 0;     // stages used by earlier items (ring position and phase)
     uint32_t nitem = 0;  // items done: phase of `done`
+    uint32_t nturn = 0;  // turns this issuer has waited for: phase of its `turn`
     for (int item = blockIdx.x; item < ga.nitems; item += gridDim.x, ++nitem) {
         const int items_x = ga.nrep * ga.split_x * ga.nunits, items_y = ga.nrep * ga.split_yz * ga.nunits;
         const int axis = item < items_x ? 0 : (item < items_x + items_y ? 1 : 2);
@@ -616,18 +623,21 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
                     if (lane == 0) atomicAdd(&pops[nitem & 1u], m);
                 }
             }
-        } else if (elect_one()) {  // MMA issuer
-            int s = 0;
+        } else if (elect_one()) {  // MMA issuer w: the item's stages s with s % 2 == w
+            const int w = warp - PW;
             const uint32_t id0 = mxf4_idesc(un.rb);
             const bool two = un.ra == 0 && un.rb > 128;
             const uint32_t id1 = mxf4_idesc(two ? un.rb - 128 : 64);
-            int slot = (int)(g0 % (uint32_t)nst);
-            uint32_t phase = (g0 / (uint32_t)nst) & 1u;
-            for (; s < n; ++s) {
-                if (!mbar_wait(smem_u32(&full[slot]), phase, ga.timeout_ns)) {
-                    *(volatile int *)&flag = 0;
-                    break;
+            int slot = (int)((g0 + (uint32_t)w) % (uint32_t)nst);
+            uint32_t phase = ((g0 + (uint32_t)w) / (uint32_t)nst) & 1u;
+            bool issued = false, ok = true;
+            for (int s = w; s < n; s += 2) {
+                ok = mbar_wait(smem_u32(&full[slot]), phase, ga.timeout_ns);
+                if (ok && s > 0) {
+                    ok = mbar_wait(smem_u32(&turn[w]), nturn & 1u, ga.timeout_ns);
+                    ++nturn;
                 }
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = ring + (uint32_t)slot * (uint32_t)ga.stage_bytes;
                 const uint32_t abase = un.ra ? base + 32768u : base;
@@ -641,21 +651,31 @@ __global__ void __launch_bounds__(32 * (PW + 1), MINB) k_gram_bits(const GramArg
                         mma_mxf4(tmem + 256u, umma_desc_sw128(base + 16384u + 32 * q),
                                  umma_desc_sw128(base + 16384u + 32 * q), id1, scale, (s > 0 || q > 0) ? 1u : 0u);
                 }
+                issued = true;
+                if (s + 1 < n) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&turn[w ^ 1])) : "memory");
+                }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                     smem_u32(&empty[slot])));
-                if (++slot == nst) {
-                    slot = 0;
+                slot += 2;
+                if (slot >= nst) {
+                    slot -= nst;
                     phase ^= 1u;
                 }
             }
-            if (s > 0) {  // covers every MMA issued before it
+            if (!ok) *(volatile int *)&flag = 0;
+            // `done` completes with both issuers' arrivals: a commit covers every MMA issued before it
+            if (issued)
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                     smem_u32(&done)));
-                if (!mbar_wait(smem_u32(&done), nitem & 1u, ga.timeout_ns)) {
-                    *(volatile int *)&flag = 0;
-                    // one more bounded window before the tensor memory is declared still in use
-                    if (!mbar_wait(smem_u32(&done), nitem & 1u, ga.timeout_ns)) mma_pending = 1;
-                }
+            else
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&done)) : "memory");
+            // the other issuer may spend two bounded waits first, and one more bounded window passes before
+            // the tensor memory is declared still in use
+            if (!mbar_wait(smem_u32(&done), nitem & 1u, 3 * ga.timeout_ns)) {
+                *(volatile int *)&flag = 0;
+                mma_pending = 1;
             }
         }
         __syncwarp();
@@ -740,7 +760,7 @@ static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaSt
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)grid);
-    lc.blockDim = dim3(32 * (PW + 1));
+    lc.blockDim = dim3(32 * (PW + 2));
     lc.dynamicSmemBytes = smem;
     lc.stream = s;
     cudaLaunchAttribute attr[1] = {pdl_attribute()};

@@ -357,7 +357,8 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
     using RP = ResPlane<W>;
     constexpr int L = RP::L, U = RP::U, PU = RP::PU, F = RP::F, W4 = RP::W4;
     constexpr int hs = U / 2;  // W4: slots of one row parity
-    const int tid = threadIdx.x, P = ra.P, NC = ra.NC;
+    constexpr bool ONE = W >= 6;  // four planes per CTA at these sizes: every thread has both boundaries
+    const int tid = threadIdx.x, P = ONE ? 4 : ra.P, NC = ONE ? L / 4 : ra.NC;
     const int c = (int)blockIdx.x % NC, r = (int)blockIdx.x / NC;
     const uint64_t S = ra.seed + (uint64_t)r;
     uint4 *lat = ra.lat + 2 * (int64_t)r * ra.nw4;
@@ -386,9 +387,9 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
             }
         }
     res_keys(keys, S);
-    const int s = tid % U, zl = 4 * (tid / U);
+    const int s = ONE ? tid : tid % U, zl = ONE ? 0 : 4 * (tid / U);
     const uint32_t grp0 = (uint32_t)((c * P + zl) * U + unit_of(s));
-    const bool lo = zl == 0, hi = zl + 4 == P;
+    const bool lo = ONE || zl == 0, hi = ONE || zl + 4 == P;
     const int cu = c + 1 == NC ? 0 : c + 1, cd = c == 0 ? NC - 1 : c - 1;
     // messages of CTA k, sublattice q: towards the lower neighbour at +0, the upper one at + 2 U
     auto msg = [&](int k, int q, int dir) { return lat + (int64_t)q * ra.nw4 + (int64_t)k * P * U + 2 * dir * U + s; };
@@ -567,7 +568,7 @@ template <int RULE>
 static cudaError_t res_rule(ResArgs ra, int R, int G, cudaStream_t s)
 {
     switch (ra.L) {
-    case 64: return launch_res<RULE, RES_W1, 2, 512>(ra, R, s);
+    case 64: return G == 2 ? launch_res<RULE, RES_W1, 2, 512>(ra, R, s) : launch_res<RULE, RES_W1, 4, 256>(ra, R, s);
     case 128:
         return G == 2 ? launch_res<RULE, RES_W2, 2, 1024>(ra, R, s) : launch_res<RULE, RES_W2, 4, 1024>(ra, R, s);
     default: return cudaErrorInvalidValue;
@@ -688,10 +689,11 @@ CoopOrder::~CoopOrder()
 
 // Whether and how R lattices of size L are swept resident (host arithmetic; sms: the device's SMs).
 //
-// Clusters, L = 64 and 128: as many CTAs per lattice as keep the launch's CTAs within two per SM
-// (us per sweep, 64^3: 16 replicas 1.05 with 8 CTAs each, 1.58 with one; 64 replicas 1.29 with 4, 1.58
-// with one; against 8.2 and 12.3 of the half-sweep kernel.  128^3: 6 replicas 1.33 with 16 CTAs, 1.92
-// with 8; 64 replicas 5.4 with 2, 5.6 with 4; against 12.3 and 49).
+// Clusters, L = 64 and 128: as many CTAs per lattice as keep the launch's CTAs within two per SM, and
+// for many lattices two CTAs with more groups per thread (us per sweep, 64^3: 16 replicas 1.05 with 8
+// CTAs each, 1.58 with one; 64 replicas 1.29 with 4; 512 replicas 4.9 with 2, 6.1 with one; against 8.2,
+// 12.3 and 50 of the half-sweep kernel.  128^3: 6 replicas 1.33 with 16 CTAs, 1.92 with 8; 38 replicas
+// 4.7 with 8, 5.7 with 2; 64 replicas 5.7 with 2, 6.7 with 8; against 12.3, 30 and 49).
 //
 // Grid, L = 192 .. 512: a launch holds as many lattices as its CTAs fit one per SM, P = 4, 8, ...
 // planes each; the P with the least rounds x time per sweep, the time being linear in the groups of
@@ -705,11 +707,14 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
 {
     ResidentPlan p{};
     if (L == 64 || L == 128) {
-        const int most = L == 64 ? 8 : 16, least = L == 64 ? 1 : 2;
-        p.ctas = most;
-        while (p.ctas > least && (int64_t)R * p.ctas > 2 * (int64_t)sms) p.ctas /= 2;
-        if (L == 128 && p.ctas == 8) p.ctas = 4;  // slower than 4 at the counts that get there
-        p.groups = (L == 64 || p.ctas == 16) ? 2 : 4;
+        const int64_t two_per_sm = 2 * (int64_t)sms;
+        if (L == 64) {
+            p.ctas = R * 8 <= two_per_sm ? 8 : (R * 4 <= two_per_sm ? 4 : 2);
+            p.groups = p.ctas > 2 ? 2 : 4;
+        } else {
+            p.ctas = R * 16 <= two_per_sm ? 16 : (R * 8 <= two_per_sm ? 8 : 2);
+            p.groups = R * 16 <= sms ? 2 : 4;
+        }
         p.per_launch = std::min(R, 4096);
         p.min_n = 1;
         p.cluster = true;
@@ -721,7 +726,7 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
     const bool whole = W == 4 || W == 8;  // rows of whole uint4
     double best = 1e300;
     for (int P = 4; P <= L / 2; P += 4) {
-        if (L % P != 0 || P * U / 4 > 1024 || L / P > sms) continue;
+        if (L % P != 0 || P * U / 4 > 1024 || L / P > sms || (W >= 6 && P != 4)) continue;
         if ((size_t)2 * P * resg_plane(W) * sizeof(uint4) > 220 * 1024) continue;
         const int per = std::min(R, sms / (L / P));
         const int rounds = (R + per - 1) / per;
