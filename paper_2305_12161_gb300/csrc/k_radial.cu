@@ -202,6 +202,25 @@ __device__ __forceinline__ void fold_walk(int L, int chunk, Fn fn, End end)
     }
 }
 
+// Sum of four run sums in double.  Single precision: as an unevaluated pair of floats (Knuth's
+// two-sum, exact up to the last additions, 2^-48), because the device adds two doubles per clock and
+// SM: one addition instead of three.
+__device__ __forceinline__ double sum4(const double (&v)[4]) { return v[0] + v[1] + v[2] + v[3]; }
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+__device__ __forceinline__ double sum4(const float (&v)[4])
+{
+    float a, b, c, ea, eb, ec;
+    two_sum(v[0], v[1], a, ea);
+    two_sum(v[2], v[3], b, eb);
+    two_sum(a, b, c, ec);
+    return (double)c + (double)__fadd_rn(__fadd_rn(ea, eb), ec);
+}
+
 // 3. |F|^2 per mode of the half spectrum; S sums per bin; (P, 0) written back.
 template <typename T>
 __global__ void __launch_bounds__(RAD_FOLD_THREADS) k_power(typename Cx<T>::type *F, int L, int chunk, int nb,
@@ -244,14 +263,15 @@ __global__ void __launch_bounds__(RAD_FOLD_THREADS) k_power(typename Cx<T>::type
                     if (lane - d >= start) v[i] += w;
                 }
             const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-            if (last && in) atomicAdd(&hs[b], (double)v[0] + (double)v[1] + (double)v[2] + (double)v[3]);
+            if (last && in) atomicAdd(&hs[b], sum4(v));
         },
         [] {});
     flush_bins(hs, sumS, nb);
 }
 
-// 5. G(k) = rint(g/N) per lag, summed per bin in int64.
-template <typename T>
+// 5. G(k) = rint(g/N) per lag, summed per bin in int64.  SMALL: N <= 2^27, so eight values' sum stays
+// within 32 bits.
+template <typename T, bool SMALL>
 __global__ void __launch_bounds__(RAD_FOLD_THREADS) k_radial_corr(const T *g, int L, int chunk, int64_t P, int nb,
                                                                    double invN, unsigned long long *sumG,
                                                                    unsigned long long *inexact)
@@ -273,6 +293,7 @@ __global__ void __launch_bounds__(RAD_FOLD_THREADS) k_radial_corr(const T *g, in
                 if (i < r.n && xr >= 0) f[4 + i] = g[(int64_t)r.row[i] * P + xr];
             }
             unsigned long long G = 0ull;
+            int G32 = 0;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
                 if ((i & 3) < r.n && (i < 4 || xr >= 0)) {
@@ -280,10 +301,11 @@ __global__ void __launch_bounds__(RAD_FOLD_THREADS) k_radial_corr(const T *g, in
                     const T q = rint(v);
                     if (fabs(v - q) > T(0.25)) ++bad;
                     // two's complement: the unsigned sums wrap to the signed result
-                    G += (fabs(q) < T(2147483520)) ? (unsigned long long)(long long)(int)q
+                    if (SMALL) G32 += (int)q;
+                    else G += (fabs(q) < T(2147483520)) ? (unsigned long long)(long long)(int)q
                                                    : (unsigned long long)(long long)q;
                 }
-            run.add(bin_of(D), G);
+            run.add(bin_of(D), SMALL ? (unsigned long long)(long long)G32 : G);
         },
         [&]() { run.flush(); });
     flush_bins(hg, sumG, nb);
@@ -499,11 +521,9 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
         return cudaErrorUnknown;
     }
     const double invN = 1.0 / ((double)L * (double)L * (double)L);  // exact: N is a power of two
-    if ((e = cudaFuncSetAttribute(k_radial_corr<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-        cudaSuccess)
-        return e;
-    k_radial_corr<T><<<grid, fold_threads, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, chunk, P, nb, invN, sumG,
-                                                       inexact);
+    auto corr = (int64_t)L * L * L <= (1 << 27) ? k_radial_corr<T, true> : k_radial_corr<T, false>;
+    if ((e = cudaFuncSetAttribute(corr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    corr<<<grid, fold_threads, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, chunk, P, nb, invN, sumG, inexact);
     k_radial_finish<<<1, 256, 0, s>>>(L, nb, c, sumG, sumS, p->count, inexact, out, cnt);
     if (launches) *launches += 4;  // own kernels; the two cuFFT executions are library launches
     return cudaGetLastError();
