@@ -173,12 +173,13 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResArgs ra)
         if (RULE != TIE_GLAUBER) return;
         res_draws<G>(rnd, grp0, U, t, q, keys);
     };
-    auto half_p = [&](int q, auto PB) {  // PB: shift direction of plane zl
+    auto half_q = [&](auto QC) {  // sublattice q; its shift direction on plane zl is q (zl is even)
+        constexpr int q = decltype(QC)::value;
         const uint4 *O = rsm + (1 - q) * sub;
         uint4 *Q = rsm + q * sub;
         uint4 cm = O[col], cc = O[col + U];
         res_each<G>([&](auto I) {
-            constexpr int i = decltype(I)::value, p = (decltype(PB)::value + i) & 1, np = 1 - p;
+            constexpr int i = decltype(I)::value, p = (q + i) & 1, np = 1 - p;
             const uint4 *pl = O + (zl + i + 1) * U;  // the plane's words
             const uint4 cp = O[col + (i + 2) * U];
             const uint4 sv = Q[col + (i + 1) * U];
@@ -209,8 +210,8 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResArgs ra)
         });
     };
     auto half = [&](int q) {
-        if (q) half_p(q, std::integral_constant<int, 1>{});
-        else half_p(q, std::integral_constant<int, 0>{});
+        if (q) half_q(std::integral_constant<int, 1>{});
+        else half_q(std::integral_constant<int, 0>{});
     };
     auto first_of = [&](uint32_t t) -> uint32_t {  // sublattice updated first (Supp. Methods I B)
         if (!ra.mixed) return 0u;
@@ -347,7 +348,7 @@ static int resg_plane(int W) { return 16 * W * W + (W == 4 || W == 8 ? 0 : 2 * (
 
 // Thread tid updates group slot tid % U of the four planes zl .. zl + 3, zl = 4 (tid / U).
 // Sizes are compile-time constants: with the row width at run time a group took 76 ALU and 49 multiply
-// instructions at L = 512, now 74 and 40 (8.4 us per sweep, now 7.8).
+// instructions at L = 512, then 74 and 40 (8.4 us per sweep, then 7.8).
 template <int RULE, int W>
 __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
 {
@@ -436,7 +437,8 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
         res_draws<4>(rnd, grp0, (uint32_t)U, t, q, keys);
     };
     // one half-sweep of sublattice q as step `step`; tagO: step of the other sublattice's last update
-    auto half_p = [&](int q, uint32_t step, uint32_t tagO, auto PB) {
+    auto half_q = [&](auto QC, uint32_t step, uint32_t tagO, auto PB) {
+        const int q = QC;  // an integral constant, or the run-time value
         const uint4 *O = gsm_res + (1 - q) * sub + zl * PU + F;
         uint4 *Q = gsm_res + q * sub + zl * PU + F;
         bool ok = true;
@@ -504,8 +506,20 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
         if (!ok) atomicMin(&s_fail, (int)step);
     };
     auto half = [&](int q, uint32_t step, uint32_t tagO) {
-        if (W4 > 0 && ((yp + q) & 1)) half_p(q, step, tagO, std::integral_constant<int, 1>{});
-        else half_p(q, step, tagO, std::integral_constant<int, 0>{});
+        using I0 = std::integral_constant<int, 0>;
+        using I1 = std::integral_constant<int, 1>;
+        // the sublattice as a constant too (512^3 7.79 -> 7.51 us per sweep, 448^3 8.84 -> 8.03), but not for
+        // L = 256 (6.65 -> 6.81)
+        if constexpr (W == 4) {
+            if ((yp + q) & 1) half_q(q, step, tagO, I1{});
+            else half_q(q, step, tagO, I0{});
+        } else if (q) {
+            if (W4 > 0 && yp == 0) half_q(I1{}, step, tagO, I1{});
+            else half_q(I1{}, step, tagO, I0{});
+        } else {
+            if (W4 > 0 && yp != 0) half_q(I0{}, step, tagO, I1{});
+            else half_q(I0{}, step, tagO, I0{});
+        }
     };
     auto first_of = [&](uint32_t t) -> uint32_t {
         if (!ra.mixed) return 0u;
@@ -699,7 +713,7 @@ CoopOrder::~CoopOrder()
 // planes each; the P with the least rounds x time per sweep, the time being linear in the groups of
 // a CTA above a floor of latency (measured: rows of whole uint4 1.2 + 1.35e-3 per group, at least
 // 3.4 us; other rows 3.5 + 2.05e-3, at least 4.9).  Per sweep: 8 x 256^3 6.6 us against 14.3 of the
-// half-sweep kernel, one 512^3 7.8 against 14.8 (four: 31.2 against 39.9), 2 x 320^3 9.5 against 28.7.
+// half-sweep kernel, one 512^3 7.5 against 14.8 (four: 30.1 against 39.9), 2 x 320^3 9.0 against 28.7.
 //
 // min_n: sweeps per call from which the load, the two grid barriers and the write-back (16 - 18 us
 // a round) are earned back.
