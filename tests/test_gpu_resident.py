@@ -91,3 +91,25 @@ def test_captured_sweep_replays(ising, L):
             p.sweep(12)
         for r in range(2):
             assert np.array_equal(p.get_packed(r), q.get_packed(r))
+
+
+def test_batches_replayed_on_two_streams(ising):
+    # captured cooperative launches of two batches, replayed with nothing waiting between them
+    import torch
+    specs = [[(256, 3, 1), (512, 1, 9), (64, 4, 20)], [(256, 9, 30), (320, 1, 50)]]
+    times = [12, 40, 41, 80]
+    want = []
+    for classes in specs:
+        with ising.Batch(classes) as b:
+            want.append(b.run(times)[0])
+    batches = [ising.Batch(classes, stream=torch.cuda.Stream()) for classes in specs]
+    recs = [torch.empty((len(times), b.record_words), dtype=torch.int64, device="cuda") for b in batches]
+    torch.cuda.synchronize()
+    for _ in range(6):
+        for b, rec in zip(batches, recs):
+            b.reinit()
+            b.run(times, rec=rec, device=True)
+    for b, rec, w in zip(batches, recs, want):
+        b.sync()
+        assert np.array_equal(rec.cpu().numpy(), w)
+        b.destroy()
