@@ -10,12 +10,12 @@
 // The operands never exist in global memory: the warps of a CTA read packed lattice words,
 // turn each 32-bit word into 32 nibbles (two logic operations per eight spins: the order of the
 // lines inside the contraction is free, so out word j takes the bits j, j + 4, j + 8, ...) and
-// write them into the 128-byte swizzled shared-memory tiles that tcgen05.mma reads.  At
-// L = 2048 a measurement takes 10.8 ms against 21.1 with e4m3 operands staged through global
-// memory (8.6 GB written and re-read per axis, and half the tensor rate); eight L = 256 replicas
-// take 0.054 ms against 0.51 by bit counts, 512 of L = 64 0.04 against 0.28.  Shared memory bounds
-// it at L = 2048: a stage of four products (512 cycles of tensor work) writes and reads 48 KB each, 768
-// cycles, and takes 990.
+// write them into the shared-memory tiles (and, for off-diagonal units of line-order copies, the
+// tensor-memory A tile) that tcgen05.mma reads.  At L = 2048 a measurement takes 8.7 ms against
+// 21.1 with e4m3 operands staged through global memory (8.6 GB written and re-read per axis, and
+// half the tensor rate); eight L = 256 replicas take 0.054 ms against 0.51 by bit counts, 512 of
+// L = 64 0.04 against 0.28.  At L = 2048 the filling warps' instructions bound it: a stage of four
+// products is 512 cycles of tensor work and takes about 760.
 //
 // Only the upper block triangle of G is computed (G is symmetric): an entry j < k stands for
 // both ordered pairs, i.e. for the distances k - j and L - (k - j).  B is the sum of the three
@@ -47,6 +47,22 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
+// The same without swizzling, so that a row's eight 16-byte pieces lie at constant distances and the
+// filling warps need no address arithmetic between them: 8 rows x 16 bytes contiguous, 128 bytes from one such block to the next
+// along K, 1024 along M/N; a K slice of 64 e2m1 values starts every 256 bytes.
+__device__ __forceinline__ uint64_t umma_desc_plain(uint32_t saddr)
+{
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+// K slice q of the operand whose first row is at saddr.
+template <bool PLAIN>
+__device__ __forceinline__ uint64_t stage_desc(uint32_t saddr, int q)
+{
+    return PLAIN ? umma_desc_plain(saddr + 256 * q) : umma_desc_sw128(saddr + 32 * q);
+}
+
 // Instruction descriptor of kind::mxf4 (dense, K = 64): A and B e2m1 (bits 7 and 10), both
 // K-major, N / 8 at bit 17, scales ue8m0 (bit 23), M / 128 at bit 27.
 __device__ __forceinline__ uint32_t mxf4_idesc(int N)
@@ -61,6 +77,30 @@ __device__ __forceinline__ void mma_mxf4(uint32_t d, uint64_t ad, uint64_t bd, u
     asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
                  "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%5], [%5], p;\n}\n" ::"r"(d),
                  "l"(ad), "l"(bd), "r"(idesc), "r"(acc), "r"(scale));
+}
+
+// The same with the A operand in tensor memory: row i of the slice in lane i, its 64 values in eight
+// columns from `a` on.
+__device__ __forceinline__ void mma_mxf4_ta(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t scale,
+                                            uint32_t acc)
+{
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], [%1], %2, %3, [%5], [%5], p;\n}\n" ::"r"(
+                     d),
+                 "r"(a), "l"(bd), "r"(idesc), "r"(acc), "r"(scale));
+}
+
+// Tensor-memory columns of slot i's A tile (32 columns): beside the 256 accumulator columns of an
+// off-diagonal unit, around the scales at 384 .. 415.  An A tile there is neither written to nor read
+// from shared memory, and six stages fit the ring in place of four.
+__device__ __forceinline__ uint32_t a_column(uint32_t slot) { return (slot < 4u ? 256u : 288u) + 32u * slot; }
+
+// Four columns of this lane's row of an A tile, in the warp's quarter of the lanes.
+__device__ __forceinline__ void tst128(uint32_t at, const uint4 &x)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(x.x), "r"(x.y),
+                 "r"(x.z), "r"(x.w)
+                 : "memory");
 }
 
 // One lane of the warp.  The compiler knows that a branch on it is taken by a single lane, which
@@ -452,7 +492,7 @@ __device__ __forceinline__ bool fill_stages(const Fill &f, uint32_t g0, int set,
         // the slot's previous use was consumed (a barrier that has completed no phase passes parity 1)
         const bool ok = mbar_wait(f.empty0 + 8u * (uint32_t)slot, phase ^ 1u, f.timeout_ns);
         if (!__all_sync(0xffffffffu, ok)) return false;  // the warp leaves together
-        put(f.ring + (uint32_t)slot * (uint32_t)f.stage_bytes, x);
+        put((uint32_t)slot, x);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0 && s != f.skip)
@@ -468,10 +508,53 @@ __device__ __forceinline__ bool fill_stages(const Fill &f, uint32_t g0, int set,
     return true;
 }
 
+// The same with the words of the next AHEAD stages under way and the expansion after the wait
+// (put(slot, v) expands and stores): for the ring of six 32 KB stages, 3072 cycles of products, where the
+// loads' latency shows before the time from a slot's release to its refill.  It is the filling warps'
+// rate that binds there: at L = 2048 the products take 5.4 ms, and the kernel 8.5 with them left out
+// and 6.0 with the filling left out.  Whole measurement: 9.97 ms with the loop above; 9.11 with
+// two stages ahead, 8.97 without the swizzle, 8.72 with three, 8.73 with four.
+template <int AHEAD, class Read, class Put>
+__device__ __forceinline__ bool fill_stages_ahead(const Fill &f, uint32_t g0, int set, int nsets, int n, Read &rd,
+                                                  Put put)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t v[AHEAD][8];
+#pragma unroll
+    for (int a = 0; a < AHEAD; ++a)
+        if (set + a * nsets < n) rd.next(v[a]);
+    int slot = (int)((g0 + (uint32_t)set) % (uint32_t)f.nst);
+    uint32_t phase = ((g0 + (uint32_t)set) / (uint32_t)f.nst) & 1u;
+#pragma unroll 1
+    for (int s = set; s < n;) {
+#pragma unroll
+        for (int a = 0; a < AHEAD; ++a) {
+            if (s >= n) break;
+            const bool ok = mbar_wait(f.empty0 + 8u * (uint32_t)slot, phase ^ 1u, f.timeout_ns);
+            if (!__all_sync(0xffffffffu, ok)) return false;  // the warp leaves together
+            put((uint32_t)slot, v[a]);
+            if (s + AHEAD * nsets < n) rd.next(v[a]);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0 && s != f.skip)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(f.full0 + 8u * (uint32_t)slot),
+                             "r"(f.arrive)
+                             : "memory");
+            slot += nsets;
+            if (slot >= f.nst) {
+                slot -= f.nst;
+                phase ^= 1u;
+            }
+            s += nsets;
+        }
+    }
+    return true;
+}
+
 // One CTA: the first PW warps fill the stages and afterwards read the accumulators, the last two
 // warps issue the MMAs, one stage each in turn: while one's products run, it commits them and the other
-// waits for its stage (four 512^3 0.28 -> 0.26 ms; at L = 2048 shared memory, written 48 and read 48 KB
-// per stage, binds and nothing changed).  The turn passes through an mbarrier between tcgen05 fences, so
+// waits for its stage (four 512^3 0.28 -> 0.26 ms; at L = 2048, where the filling warps bind, nothing
+// changed).  The turn passes through an mbarrier between tcgen05 fences, so
 // the products reach the accumulators in the order of the stages.  A stage holds 256 lines of every row of the unit; the (ra + rb) / 32
 // warps of a set fill it, one row per lane, and as many sets as the PW warps hold work on successive
 // stages.  Each stage is written once and read by 4 (off-diagonal) or 8 MMAs of 128 x N x 64.
@@ -490,6 +573,7 @@ template <int PW, int MINB, int READS>
 __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArgs ga)
 {
     constexpr int GB_THREADS = 32 * (PW + 2);
+    constexpr bool TA = READS == GR_T;  // A tiles in tensor memory
     extern __shared__ __align__(1024) uint8_t gsm[];
     __shared__ int sacc[GB_SACC];
     __shared__ __align__(8) uint64_t full[8], empty[8], turn[2], done;
@@ -583,7 +667,8 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
 #pragma unroll
                             for (int i = 0; i < 8; ++i) x[i] = expand_e2m1(tr(v[i]));
                         },
-                        [&](uint32_t base, uint4 x[8]) {
+                        [&](uint32_t slot, uint4 x[8]) {
+                            const uint32_t base = ring + slot * (uint32_t)fl.stage_bytes;
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {  // bundle b0 + i / 2, positions 64 kw + 2 lane + (i & 1)
                                 const uint32_t rr = (uint32_t)(xr + 2 * lane + (i & 1));
@@ -606,12 +691,32 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
 #pragma unroll
                             for (int i = 0; i < 8; ++i) m += __popc(v[i]);
                     };
-                    auto put = [&](uint32_t base, uint4 x[8]) {
-                        const uint32_t at = base + row_off;
+                    auto put = [&](uint32_t slot, uint4 x[8]) {
+                        const uint32_t at = ring + slot * (uint32_t)fl.stage_bytes + row_off;
 #pragma unroll
                         for (int i = 0; i < 8; ++i) sts128(at ^ (uint32_t)(i << 4), x[i]);
                     };
-                    if (READS == GR_T || (READS == GR_ANY && axis == 0)) {
+                    if (TA) {
+                        ReadT rd(ga.lines + (int64_t)r * ga.rep_words + (int64_t)axis * 2 * ga.nw, L, p, c0 + set, nsets);
+                        const uint32_t off = (uint32_t)(ri >> 3) * 1024u + (uint32_t)(ri & 7) * 16u;
+                        ok = fill_stages_ahead<3>(fl, g0, set, nsets, n, rd, [&](uint32_t slot, uint32_t v[8]) {
+                            if (count_m)
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) m += __popc(v[i]);
+                            if (32 * ws >= un.rb) {  // rb is 256: A rows 32 (warp % 4) .. + 31
+                                const uint32_t at = tmem + a_column(slot) + ((uint32_t)(32 * (warp & 3)) << 16);
+                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) tst128(at + 4u * i, expand_e2m1(v[i]));
+                                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                            } else {
+                                const uint32_t at = ring + slot * (uint32_t)fl.stage_bytes + off;
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) sts128(at + (uint32_t)(i << 7), expand_e2m1(v[i]));
+                            }
+                        });
+                    } else if (READS == GR_ANY && axis == 0) {
                         ReadT rd(ga.lines + (int64_t)r * ga.rep_words + (int64_t)axis * 2 * ga.nw, L, p, c0 + set, nsets);
                         ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
                     } else if (READS == GR_XL || (READS == GR_ANY && W % 4 == 0)) {
@@ -647,15 +752,22 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t base = ring + (uint32_t)slot * (uint32_t)ga.stage_bytes;
                 const uint32_t abase = un.ra ? base + 32768u : base;
+                if (TA && un.ra) {  // the branch outside the loop: inside, a measurement at L = 2048 took 0.55 ms more
 #pragma unroll
-                for (int q = 0; q < GB_ROW / 32; ++q)
-                    mma_mxf4(tmem, umma_desc_sw128(abase + 32 * q), umma_desc_sw128(base + 32 * q), id0, scale,
-                             (s > 0 || q > 0) ? 1u : 0u);
+                    for (int q = 0; q < GB_ROW / 32; ++q)
+                        mma_mxf4_ta(tmem, tmem + a_column((uint32_t)slot) + 8u * q, stage_desc<TA>(base, q), id0,
+                                    scale, (s > 0 || q > 0) ? 1u : 0u);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < GB_ROW / 32; ++q)
+                        mma_mxf4(tmem, stage_desc<TA>(abase, q), stage_desc<TA>(base, q), id0, scale,
+                                 (s > 0 || q > 0) ? 1u : 0u);
+                }
                 if (two) {
 #pragma unroll
                     for (int q = 0; q < GB_ROW / 32; ++q)
-                        mma_mxf4(tmem + 256u, umma_desc_sw128(base + 16384u + 32 * q),
-                                 umma_desc_sw128(base + 16384u + 32 * q), id1, scale, (s > 0 || q > 0) ? 1u : 0u);
+                        mma_mxf4(tmem + 256u, stage_desc<TA>(base + 16384u, q), stage_desc<TA>(base + 16384u, q), id1,
+                                 scale, (s > 0 || q > 0) ? 1u : 0u);
                 }
                 issued = true;
                 if (s + 1 < n) {
@@ -795,7 +907,8 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
     ga.nunits = ga.nsb;
     const int nb = (L + 127) / 128;
     for (int bj = 0; bj < nb; ++bj) ga.nunits += ga.nsb - 1 - bj / 2;
-    // one stage: 16 KB (one tile), 32 KB (one super-tile) or 48 KB (super-tile and A tile).  Up to
+    // one stage: 16 KB (one tile), 32 KB (one super-tile) or 48 KB (super-tile and A tile; 32 where the
+    // A tile is in tensor memory, which needs whole super-tiles).  Up to
     // L = 128 half of the tensor memory and of the shared memory suffice, so two CTAs share an SM
     // and one's read-back overlaps the other's products.
     const bool small = L <= 128;
@@ -803,6 +916,7 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
     ga.nst = L <= 256 ? 6 : 4;
     ga.ncols = small ? 256 : 512;
     ga.scale_col = small ? 128 : 384;
+    if (lines && all3) ga.stage_bytes = 32768, ga.nst = 6;  // GR_T
     ga.err = err;
     ga.timeout_ns = (uint64_t)(timeout_s * 1e9);
     const size_t smem = (size_t)ga.nst * ga.stage_bytes + 1024;

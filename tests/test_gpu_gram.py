@@ -38,3 +38,15 @@ def test_record_equals_bit_counts(ising, L, R):
             a.sweep(n)
             b.sweep(n)
             assert np.array_equal(a.measure(), b.measure()), n
+
+
+@pytest.mark.parametrize("L,R", [(512, 1), (768, 2), (1024, 1), (1280, 1)])
+def test_line_order_units_equal_bit_counts(ising, L, R):
+    """Sizes of whole super-tiles with the line-order copies: diagonal and off-diagonal units follow
+    one another on a block, whose A tiles share tensor memory with the other's second accumulator."""
+    with ising.Ising(L, replicas=R, seed=23) as a, \
+            ising.Ising(L, replicas=R, seed=23, corr=ising.CORR_POPCOUNT) as b:
+        for n in (0, 3):
+            a.sweep(n)
+            b.sweep(n)
+            assert np.array_equal(a.measure(), b.measure()), n
