@@ -180,9 +180,9 @@ TRAFFIC_NCU = {("k_mcs_fused", 2048, 64, 26): (2.162e9, "ncu, profiles/k_mcs_fus
 def run_batched(torch, ising, inputs, K: int = 20, window: int = 20) -> dict:
     """Mixed batch 512x64^3 + 64x128^3 + 16x256^3 + 4x512^3 (each lattice its own seed):
     the batched form runs 10^4 MCS with K log-spaced measurements as one CUDA graph
-    (per segment a persistent launch for the 64^3 and 128^3 classes and the 256^3 and 512^3
-    classes streamed beside it on side streams; work list, streamed kernels and stream order
-    tuned by the autotuner); the plain form (one byte per spin, one launch per lattice) and
+    (per segment each class in one launch, or one per group of lattices, resident in shared
+    memory; the 256^3 and 512^3 classes streamed in the shortest segments; tuned by the autotuner);
+    the plain form (one byte per spin, one launch per lattice) and
     the packed form launched per class (on the kernels the batch chose) are compared with it
     on the same window of `window` MCS from the T = inf start."""
     stream = torch.cuda.Stream()
@@ -208,6 +208,7 @@ def run_batched(torch, ising, inputs, K: int = 20, window: int = 20) -> dict:
         out["plan"] = bt.plan()
         kernels = [bt.class_config(ci) for ci in range(len(BATCH_CLASSES))]
         out["streamed_beside_persistent"] = bt.overlap
+        # (what the segments too short for the resident sweep run)
         out["class_kernels"] = {f"{L}^3": ("persistent" if k["variant"] < 0 else
                                            f"variant {k['variant']}, tile_z {k['tile_z']}, depth {k['depth']}")
                                 for (L, _, _), k in zip(BATCH_CLASSES, kernels)}

@@ -70,7 +70,11 @@ typedef struct {
     int form;       /* ising_form */
     void *stream;   /* cudaStream_t to enqueue on; NULL: the library creates one */
     int device;     /* CUDA device ordinal; -1: the current device */
-    int variant;    /* packed sweep kernel variant, 0 = automatic (see ising_variants):
+    int variant;    /* packed sweep kernel variant, 0 = automatic: for L = 64, 128, 192 .. 512 (multiples
+                       of 64) calls of a few sweeps or more run in one launch (or one per group of
+                       replicas) with the lattices in shared memory, everything else a half-sweep
+                       kernel chosen for L (not while a cooperative launch would be captured); or
+                       one of (see ising_variants):
                        1 one thread per word (any L), 2 z-marching tiles (L multiple of 256),
                        3 z-marching specialised on the row width (L = 256, 512, 1024, 2048),
                        4 as 3 with a deeper copy pipeline and fewer registers,
@@ -92,8 +96,8 @@ typedef struct {
     int block_x;    /* double checkerboard: block sides in sites (0 = default: block_x = L, */
     int block_y;    /*   block_y = 16, block_z = 8, both L when L <= 16); see ising_scheme */
     int block_z;
-    int pdl;        /* 1 (ising_default_opts): the z-marching (variant 3) and whole-sweep
-                       (variant 5) kernels are launched with programmatic dependent launch:
+    int pdl;        /* 1 (ising_default_opts): the z-marching (variant 3), whole-sweep
+                       (variant 5) and PLAIN-form kernels are launched with programmatic dependent launch:
                        a sweep's CTAs are scheduled while the previous one drains and wait
                        for its completion before they touch memory (same results, shorter
                        gaps between the launches of one stream); 0: plain stream order,
@@ -311,9 +315,11 @@ int64_t ising_launch_count(const ising_ctx *ctx);
  * 256 and at least the streaming threshold (default 256; ising_batch_set_streamed) are
  * instead swept in the same segment by a single-lattice sweep kernel (the z-marching one
  * by default, the one ising_batch_tune picks after tuning), which streams them faster
- * than slab groups do.  Every lattice follows
- * exactly the trajectory of the single-lattice entry points (same rule, order and
- * random bits), so batching changes speed, not results.
+ * than slab groups do.  In segments of a few sweeps or more, classes of a size with a resident
+ * sweep (ising_opts.variant) run that instead, one class after the other: streamed classes on
+ * their default kernel, and the persistent kernel's classes when all of them have one.  Every
+ * lattice follows exactly the trajectory of the single-lattice entry points (same rule, order
+ * and random bits), so batching changes speed, not results.
  * Records and derived values are concatenated in class order, replica-major within a
  * class: ising_batch_record_words() int64 and 4 * ising_batch_lattices() doubles per
  * measured time; a measurement runs one class per stream, on the tensor cores for L a multiple
@@ -323,7 +329,7 @@ int64_t ising_launch_count(const ising_ctx *ctx);
 typedef struct ising_batch ising_batch;
 int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *replicas, const uint64_t *seeds,
                        const ising_opts *opts);
-/* Enqueue n_mcs sweeps of every lattice: one persistent launch (per 2^30 sweeps). */
+/* Enqueue n_mcs sweeps of every lattice. */
 int ising_batch_sweep(ising_batch *b, int64_t n_mcs);
 int64_t ising_batch_record_words(const ising_batch *b);
 int64_t ising_batch_lattices(const ising_batch *b);

@@ -48,8 +48,9 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
 }
 
 // The same without swizzling, so that a row's eight 16-byte pieces lie at constant distances and the
-// filling warps need no address arithmetic between them: 8 rows x 16 bytes contiguous, 128 bytes from one such block to the next
-// along K, 1024 along M/N; a K slice of 64 e2m1 values starts every 256 bytes.
+// filling warps need no address arithmetic between them: 8 rows x 16 bytes contiguous, 128 bytes
+// from one such block to the next along K, 1024 along M/N; a K slice of 64 e2m1 values starts every
+// 256 bytes.
 __device__ __forceinline__ uint64_t umma_desc_plain(uint32_t saddr)
 {
     return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
