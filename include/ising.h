@@ -97,8 +97,8 @@ typedef struct {
     int block_y;    /*   block_y = 16, block_z = 8, both L when L <= 16); see ising_scheme */
     int block_z;
     int pdl;        /* 1 (ising_default_opts): the z-marching (variant 3), whole-sweep
-                       (variant 5) and PLAIN-form kernels are launched with programmatic dependent launch:
-                       a sweep's CTAs are scheduled while the previous one drains and wait
+                       (variant 5), PLAIN-form and measurement kernels are launched with programmatic
+                       dependent launch: a kernel's CTAs are scheduled while the previous one drains and wait
                        for its completion before they touch memory (same results, shorter
                        gaps between the launches of one stream); 0: plain stream order,
                        which leaves the SMs of a draining kernel to other streams (many

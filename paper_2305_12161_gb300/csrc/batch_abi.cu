@@ -49,6 +49,7 @@ struct ising_batch {
     std::vector<cudaEvent_t> ev;
     int overlap = 0;
     int rule = 0;
+    int pdl = 1;  // programmatic dependent launch of the streamed sweeps and the measurements
     std::vector<BatchClass> cls;
     int64_t nlat = 0, rec_words = 0;
     int64_t t = 0;
@@ -275,9 +276,11 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
                     BCK(b, launch_sweeps_fused(&cur, &nxt, k.L, k.R, k.seed, b->rule, b->t, even, 0, k.cfg.tile_z,
                                                k.cfg.depth, b->d_status, (double)b->timeout_ns * 1e-9, st,
                                                &b->launches, k.cfg.pdl != 0));
-                if (chunk & 1)
-                    BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t + even, 1, 0,
-                                                default_sweep_config(k.L, k.R), st, &b->launches));
+                if (chunk & 1) {
+                    SweepConfig one = default_sweep_config(k.L, k.R);
+                    one.pdl = b->pdl;
+                    BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t + even, 1, 0, one, st, &b->launches));
+                }
             } else {
                 BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, k.cfg, st,
                                             &b->launches));
@@ -304,8 +307,8 @@ int enqueue_measure(ising_batch *b, int64_t *rec, double *der, double c, unsigne
         cudaStream_t st = i == 0 ? b->stream : b->side[i - 1];
         if (i > 0) BCK(b, cudaStreamWaitEvent(st, b->ev[0], 0));
         const int method = !corr ? CORR_NONE : (gram_supported(k.L) ? CORR_TENSOR : CORR_POPCOUNT);
-        BCK(b, launch_measure(k.lat, k.L, k.R, b->t, method, rec + k.rec_off, st, &b->launches, k.xt, b->d_status,
-                              (double)b->timeout_ns * 1e-9));
+        BCK(b, launch_measure(k.lat, k.L, k.R, b->t, method, rec + k.rec_off, st, &b->launches, b->pdl != 0, k.xt,
+                              b->d_status, (double)b->timeout_ns * 1e-9));
         if (der)
             BCK(b, launch_derived(rec + k.rec_off, k.L, k.R, c, flags & ISING_MEAS_CONNECTED, der + 4 * k.der_off,
                                   st, &b->launches));
@@ -340,6 +343,7 @@ int assign_modes(ising_batch *b)
     for (auto &k : b->cls) {
         k.streamed = b->stream_min_L > 0 && k.L >= b->stream_min_L && k.L % 256 == 0;
         k.cfg = default_sweep_config(k.L, k.R);
+        k.cfg.pdl = b->pdl;
         k.automatic = 1;
         if (k.streamed) continue;
         const Geom g = make_geom(k.L);
@@ -450,6 +454,7 @@ int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *r
     }
     b->device = dev;
     b->rule = o.tie;
+    b->pdl = o.pdl != 0;
     DevGuard dg(dev);
     auto bail = [&](int s) {
         ising_batch_destroy(b);
@@ -789,6 +794,7 @@ int ising_batch_set_class_opts(ising_batch *b, int cls, const ising_opts *o)
         return bfail(b, ISING_ENOMEM, "second store of the fused sweep");
     }
     k.cfg = cfg;
+    k.cfg.pdl = b->pdl;
     k.automatic = o->variant == 0;
     if (b->gexec) {  // the cached schedule graph holds the old kernels
         cudaGraphExecDestroy(b->gexec);

@@ -576,8 +576,8 @@ int ising_measure_ex(ising_ctx *c, int64_t *rec, double *derived, double cval, u
     }
     const int inject = method == CORR_TENSOR ? c->inject_stall : 0;
     c->inject_stall = 0;
-    CK(c, launch_measure(c->lat, c->L, c->R, c->t, method, rdst, c->stream, &c->launches, c->xt, c->dev_err,
-                         c->wait_timeout_s, inject));
+    CK(c, launch_measure(c->lat, c->L, c->R, c->t, method, rdst, c->stream, &c->launches, c->cfg.pdl != 0, c->xt,
+                         c->dev_err, c->wait_timeout_s, inject));
     double *ddst = nullptr;
     if (derived) {
         ddst = dev ? derived : c->der_dev;

@@ -872,7 +872,7 @@ size_t corr_mma_scratch_bytes(int L, int R)
 }
 
 template <int PW, int MINB, int READS>
-static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaStream_t s)
+static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaStream_t s, bool pdl)
 {
     auto kern = k_gram_bits<PW, MINB, READS>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -884,7 +884,7 @@ static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaSt
     lc.stream = s;
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     lc.attrs = attr;
-    lc.numAttrs = 1;
+    lc.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&lc, kern, ga);
 }
 
@@ -892,7 +892,7 @@ static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaSt
 // the copies in line order, or null (the kernel then reads the packed store: below L = 512 a word is
 // read by one to three units only).
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *scratch, int *err,
-                            cudaStream_t s, int64_t *launches, double timeout_s, int inject)
+                            cudaStream_t s, int64_t *launches, bool pdl, double timeout_s, int inject)
 {
     if (!gram_supported(L)) return cudaErrorInvalidValue;
     const Geom g = make_geom(L);
@@ -955,10 +955,10 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
         ga.inject = inject && r0 == 0;
         const int grid = std::min(ga.nitems, slots);
         cudaError_t e;
-        if (small) e = launch_gram<12, 2, GR_SMALL>(ga, grid, smem, s);
-        else if (lines && all3) e = launch_gram<24, 1, GR_T>(ga, grid, smem, s);
-        else if (all3) e = launch_gram<24, 1, GR_XL>(ga, grid, smem, s);
-        else e = launch_gram<12, 1, GR_ANY>(ga, grid, smem, s);
+        if (small) e = launch_gram<12, 2, GR_SMALL>(ga, grid, smem, s, pdl);
+        else if (lines && all3) e = launch_gram<24, 1, GR_T>(ga, grid, smem, s, pdl);
+        else if (all3) e = launch_gram<24, 1, GR_XL>(ga, grid, smem, s, pdl);
+        else e = launch_gram<12, 1, GR_ANY>(ga, grid, smem, s, pdl);
         if (e != cudaSuccess) return e;
         if (launches) *launches += !lines ? 1 : (all3 ? 3 : 2);
     }

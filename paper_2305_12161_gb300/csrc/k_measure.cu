@@ -401,7 +401,7 @@ static cudaError_t launch_corr(const uint32_t *lat, const Geom &g, int R, int64_
 }
 
 cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int corr, int64_t *rec, cudaStream_t s,
-                           int64_t *launches, uint32_t *xt_scratch, int *err, double wait_timeout_s,
+                           int64_t *launches, bool pdl, uint32_t *xt_scratch, int *err, double wait_timeout_s,
                            int inject_stall)
 {
     const Geom g = make_geom(L);
@@ -414,13 +414,13 @@ cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int cor
     lc.stream = s;
     cudaLaunchAttribute attr[1] = {pdl_attribute()};
     lc.attrs = attr;
-    lc.numAttrs = 1;
+    lc.numAttrs = pdl ? 1 : 0;
     const cudaError_t ie = cudaLaunchKernelEx(&lc, k_rec_init, rec, L, R, t, corr);
     if (ie != cudaSuccess) return ie;
     if (corr == CORR_TENSOR) {  // M, B and D_a(r) in one pass
         if (!err || !gram_supported(L)) return cudaErrorInvalidValue;
         if (launches) *launches += 1;
-        return launch_corr_mma(lat, L, R, rec, xt_scratch, err, s, launches, wait_timeout_s, inject_stall);
+        return launch_corr_mma(lat, L, R, rec, xt_scratch, err, s, launches, pdl, wait_timeout_s, inject_stall);
     }
     if (L >= 256 && L % 256 == 0) {
         int64_t mb = (g.nw / 4 + 255) / 256;

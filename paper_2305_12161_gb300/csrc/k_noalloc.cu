@@ -65,7 +65,7 @@ extern "C" int ising_measure_derived_noalloc(const uint32_t *lattice, int L, int
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // launch_measure first rewrites every record word it uses (t, zeroed M, B and D),
     // so nothing left over from an earlier call reaches the result.
-    if (ising::launch_measure(lattice, L, replicas, 0, !(flags & ISING_MEAS_NO_CORR), records, s, nullptr) !=
+    if (ising::launch_measure(lattice, L, replicas, 0, !(flags & ISING_MEAS_NO_CORR), records, s, nullptr, false) !=
         cudaSuccess)
         return ISING_ECUDA;
     if (ising::launch_derived(records, L, replicas, c, flags & ISING_MEAS_CONNECTED, derived, s, nullptr) !=

@@ -26,7 +26,7 @@ struct SweepConfig {
     int tile_y;  // rows per tile (z-march; ZFAST: fixed to 256 / (L/256))
     int tile_z;  // planes per tile (z-march)
     int depth;   // ZDEEP: planes in flight beyond the one consumed (2..4)
-    int pdl = 1; // ZFAST, ZFUSE: programmatic dependent launch (0: plain stream order)
+    int pdl = 1; // ZFAST, ZFUSE, plain form, measurement: programmatic dependent launch (0: plain stream order)
 };
 
 bool sweep_config_valid(int L, const SweepConfig &c);
@@ -144,16 +144,17 @@ cudaError_t launch_unpack(const uint32_t *lat, int8_t *plain, int L, int R, cuda
 // tensor-core kernel gave up; the records are then incomplete); xt_scratch is either
 // corr_mma_scratch_bytes(L, R) bytes, which L >= 512 uses for the transposed x axis, or null.
 enum CorrMethod : int { CORR_NONE = 0, CORR_POPCOUNT = 1, CORR_TENSOR = 2 };
-// wait_timeout_s bounds each device-side wait of the tensor-core path (wall time);
-// inject_stall (tests) makes one of its CTAs skip a load so that a wait runs out.
+// pdl: programmatic dependent launch of the measurement's kernels.  wait_timeout_s bounds each
+// device-side wait of the tensor-core path (wall time); inject_stall (tests) makes one of its CTAs skip a
+// load so that a wait runs out.
 cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int corr, int64_t *rec,
-                           cudaStream_t s, int64_t *launches, uint32_t *xt_scratch = nullptr, int *err = nullptr,
-                           double wait_timeout_s = 2.0, int inject_stall = 0);
+                           cudaStream_t s, int64_t *launches, bool pdl, uint32_t *xt_scratch = nullptr,
+                           int *err = nullptr, double wait_timeout_s = 2.0, int inject_stall = 0);
 bool gram_supported(int L);      // sizes the tensor-core kernel takes
 bool corr_mma_supported(int L);  // sizes of the explicit option ISING_CORR_TENSOR
 size_t corr_mma_scratch_bytes(int L, int R);
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *xt_scratch, int *err,
-                            cudaStream_t s, int64_t *launches, double timeout_s, int inject);
+                            cudaStream_t s, int64_t *launches, bool pdl, double timeout_s, int inject);
 // derived: R x [e, m, l_E, l_C]
 cudaError_t launch_derived(const int64_t *rec, int L, int R, double c, bool connected, double *derived,
                            cudaStream_t s, int64_t *launches);
