@@ -75,6 +75,8 @@ struct ising_batch {
     int64_t *d_rec = nullptr;
     double *d_der = nullptr;
     // cached schedule graph
+    bool coop = false;       // a cooperative launch was enqueued (set by enqueue_segment)
+    bool graph_coop = false; // the graph holds one
     cudaGraphExec_t gexec = nullptr;
     std::vector<int64_t> gkey;
 };
@@ -205,8 +207,9 @@ int upload_plan(ising_batch *b)
     return ISING_OK;
 }
 
-// Enqueue one segment of n MCS (split at 2^30 sweeps per launch).
-int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
+// Enqueue one segment of n MCS (split at 2^30 sweeps per launch).  grid: the resident sweeps that are
+// cooperative launches may be used.
+int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool grid = true)
 {
     while (n > 0) {
         const int chunk = (int)std::min<int64_t>(n, 1 << 30);
@@ -221,7 +224,7 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
         for (size_t i = 0; i < b->cls.size(); ++i) {
             const auto &k = b->cls[i];
             res[i] = !b->no_resident && (k.automatic || !k.streamed) && resident_plan(k.L, k.R, b->sms, &rp[i]) &&
-                     chunk >= rp[i].min_n;
+                     chunk >= rp[i].min_n && (grid || rp[i].cluster);
             if (!k.streamed && !res[i]) all_small = false;
         }
         for (size_t i = 0; i < b->cls.size(); ++i) {
@@ -236,6 +239,7 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
         // otherwise
         if (first_side == 0 && nstreamed > 0) BCK(b, cudaEventRecord(b->ev[0], b->stream));
         if (persistent) {
+            b->coop = true;
             BCK(b, cudaMemsetAsync(b->d_barriers, 0, sizeof(unsigned) * (size_t)std::max(1, b->ngroups), b->stream));
             BCK(b, launch_batch(b->d_tasks, (int)b->h_tasks.size(), b->d_lats, b->rule, (uint32_t)b->t, chunk,
                                 b->d_barriers, b->d_status, b->timeout_ns, b->missing_cta, cta_ns, b->smem,
@@ -245,6 +249,7 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns)
         for (size_t i = 0; i < b->cls.size(); ++i) {
             const auto &k = b->cls[i];
             if (!res[i]) continue;
+            if (!rp[i].cluster) b->coop = true;
             const cudaError_t e = launch_sweeps_resident(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, rp[i], b->d_status,
                                                          (double)b->timeout_ns * 1e-9, b->stream, &b->launches);
             if (e == cudaErrorNotSupported) {
@@ -515,7 +520,11 @@ int ising_batch_sweep(ising_batch *b, int64_t n)
     if (n < 0 || b->t + n > (int64_t)0xffffffffll) return bfail(b, ISING_EINVAL, "bad sweep count");
     if (n == 0) return ISING_OK;
     DevGuard dg(b->device);
-    return enqueue_segment(b, n, nullptr);
+    // in a caller's capture no resident grid, as in a context: nothing here orders the replays of the
+    // caller's graph against other cooperative launches
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BCK(b, cudaStreamIsCapturing(b->stream, &cap));
+    return enqueue_segment(b, n, nullptr, cap == cudaStreamCaptureStatusNone);
 }
 
 int64_t ising_batch_record_words(const ising_batch *b) { return b ? b->rec_words : -1; }
@@ -586,6 +595,7 @@ int ising_batch_run(ising_batch *b, const int64_t *times, int K, int64_t *rec, d
         }
         cudaGraph_t graph = nullptr;
         BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+        b->coop = false;
         int st = ISING_OK;
         for (int k = 0; k < K && st == ISING_OK; ++k) {
             st = enqueue_segment(b, times[k] - b->t, nullptr);
@@ -604,8 +614,14 @@ int ising_batch_run(ising_batch *b, const int64_t *times, int K, int64_t *rec, d
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) return bcuda(b, e, "cudaGraphInstantiate");
         b->gkey = key;
+        b->graph_coop = b->coop;
     }
-    BCK(b, cudaGraphLaunch(b->gexec, b->stream));
+    if (b->graph_coop) {  // the replay as a whole takes its place among the process's cooperative launches
+        const CoopOrder order(b->stream);
+        BCK(b, cudaGraphLaunch(b->gexec, b->stream));
+    } else {
+        BCK(b, cudaGraphLaunch(b->gexec, b->stream));
+    }
     b->t = times[K - 1];
     if (!dev) {
         BCK(b, cudaMemcpyAsync(rec, rdst, sizeof(int64_t) * b->rec_words * K, cudaMemcpyDeviceToHost, b->stream));

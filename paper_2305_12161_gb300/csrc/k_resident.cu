@@ -671,7 +671,8 @@ static cudaError_t resident_cluster(uint32_t *lat, int L, int R, uint64_t seed, 
 
 // Cooperative launches of this process on one device run one after the other, whatever their streams:
 // two that were resident in part would wait for each other's SMs until their bounds.  (Not while a
-// stream is being captured: an event recorded outside cannot order a graph.)
+// stream is being captured: an event recorded outside cannot order a graph.  The launch of the graph is
+// ordered instead.)
 namespace {
 struct CoopChain {
     std::mutex m;

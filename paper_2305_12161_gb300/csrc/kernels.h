@@ -75,8 +75,8 @@ cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, i
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
                                    int64_t *launches);
 
-// Scope around a cooperative launch on stream s: it runs after the previous one of this process on
-// the current device (nothing is ordered while s is being captured).
+// Scope around a cooperative launch on stream s, or the launch of a graph that holds some: it runs after
+// the previous one of this process on the current device (nothing is ordered while s is being captured).
 class CoopOrder {
 public:
     explicit CoopOrder(cudaStream_t s);

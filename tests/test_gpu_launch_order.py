@@ -1,4 +1,5 @@
-"""Order of launches on a stream and between streams: the option pdl = 0 in the measurement."""
+"""Order of launches on a stream and between streams: the option pdl = 0 in the measurement, and
+cooperative launches of contexts and batches on streams of their own."""
 import ctypes
 
 import numpy as np
@@ -48,3 +49,76 @@ def test_measurement_in_plain_stream_order(ising, L, kw):
             edges[pdl] = _programmatic_edges(stream, lambda: (q.measure_device(rec), q.measure_device(rec)))
     assert edges[0] == 0 and edges[1] > 0
     assert np.array_equal(recs[0], recs[1])
+
+
+def test_replayed_batch_waits_for_a_context_s_resident_sweep(ising):
+    # 144 CTAs each, more than one per SM together: the replay waits, although CTAs this small could share
+    # an SM
+    import torch
+    times, classes = [4, 8], [(192, 3, 1)]
+    with ising.Batch(classes) as b:
+        want, _ = b.run(times)
+    sa, sb = torch.cuda.Stream(), torch.cuda.Stream()
+    with ising.Ising(192, replicas=3, seed=9, stream=sa) as q, ising.Batch(classes, stream=sb) as b:
+        rec = torch.empty((len(times), b.record_words), dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        q.sweep(16)
+        b.run(times, rec=rec, device=True)  # captures
+        b.reinit()
+        q.sync()
+        b.sync()
+        ea, eb = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        q.sweep(4000)
+        ea.record(sa)
+        b.run(times, rec=rec, device=True)
+        eb.record(sb)
+        q.sync()
+        b.sync()
+        assert ea.elapsed_time(eb) > 0
+        assert np.array_equal(rec.cpu().numpy(), want)
+
+
+def test_context_sweeps_between_batch_replays(ising):
+    import torch
+    classes, times = [(512, 1, 9), (256, 2, 30)], [12, 40, 41, 80]
+    with ising.Batch(classes) as b:
+        want, _ = b.run(times)
+    with ising.Ising(512, replicas=1, seed=4) as p, ising.Ising(320, replicas=2, seed=6) as r:
+        p.sweep(6 * 24)
+        r.sweep(6 * 24)
+        states = [p.get_packed(0), r.get_packed(1)]
+    with ising.Ising(512, replicas=1, seed=4, stream=torch.cuda.Stream()) as p, \
+            ising.Ising(320, replicas=2, seed=6, stream=torch.cuda.Stream()) as r, \
+            ising.Batch(classes, stream=torch.cuda.Stream()) as b:
+        rec = torch.empty((len(times), b.record_words), dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(6):
+            p.sweep(24)
+            b.reinit()
+            b.run(times, rec=rec, device=True)
+            r.sweep(24)
+        for o in (p, r, b):
+            o.sync()
+        assert np.array_equal(rec.cpu().numpy(), want)
+        assert np.array_equal(p.get_packed(0), states[0]) and np.array_equal(r.get_packed(1), states[1])
+
+
+def test_batch_sweep_in_a_caller_s_capture(ising):
+    # no resident grid there: the classes run on the persistent kernel and as streamed half-sweeps
+    import torch
+    classes, n = [(192, 2, 3), (256, 2, 8), (64, 2, 50)], 12
+    with ising.Batch(classes) as a:
+        a.sweep(n)
+        want = [a.get_packed(ci, r) for ci, c in enumerate(classes) for r in range(c[1])]
+    stream = torch.cuda.Stream()
+    with ising.Batch(classes, stream=stream) as b:
+        b.sync()
+        g = torch.cuda.CUDAGraph()
+        l0 = b.launch_count()
+        with torch.cuda.graph(g, stream=stream):
+            b.sweep(n)
+        assert b.launch_count() - l0 == 1 + 2 * n
+        with torch.cuda.stream(stream):
+            g.replay()
+        got = [b.get_packed(ci, r) for ci, c in enumerate(classes) for r in range(c[1])]
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
