@@ -75,8 +75,8 @@ struct ising_batch {
     int64_t *d_rec = nullptr;
     double *d_der = nullptr;
     // cached schedule graph
-    bool coop = false;       // a cooperative launch was enqueued (set by enqueue_segment)
-    bool graph_coop = false; // the graph holds one
+    int coop = 0;        // CTAs of the largest cooperative launch enqueued (enqueue_segment adds to it)
+    int graph_coop = 0;  // of the graph's largest one
     cudaGraphExec_t gexec = nullptr;
     std::vector<int64_t> gkey;
 };
@@ -239,7 +239,7 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
         // otherwise
         if (first_side == 0 && nstreamed > 0) BCK(b, cudaEventRecord(b->ev[0], b->stream));
         if (persistent) {
-            b->coop = true;
+            b->coop = std::max(b->coop, (int)b->h_tasks.size());
             BCK(b, cudaMemsetAsync(b->d_barriers, 0, sizeof(unsigned) * (size_t)std::max(1, b->ngroups), b->stream));
             BCK(b, launch_batch(b->d_tasks, (int)b->h_tasks.size(), b->d_lats, b->rule, (uint32_t)b->t, chunk,
                                 b->d_barriers, b->d_status, b->timeout_ns, b->missing_cta, cta_ns, b->smem,
@@ -249,7 +249,7 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
         for (size_t i = 0; i < b->cls.size(); ++i) {
             const auto &k = b->cls[i];
             if (!res[i]) continue;
-            if (!rp[i].cluster) b->coop = true;
+            if (!rp[i].cluster) b->coop = std::max(b->coop, std::min(k.R, rp[i].per_launch) * rp[i].ctas);
             const cudaError_t e = launch_sweeps_resident(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, rp[i], b->d_status,
                                                          (double)b->timeout_ns * 1e-9, b->stream, &b->launches);
             if (e == cudaErrorNotSupported) {
@@ -595,7 +595,7 @@ int ising_batch_run(ising_batch *b, const int64_t *times, int K, int64_t *rec, d
         }
         cudaGraph_t graph = nullptr;
         BCK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        b->coop = false;
+        b->coop = 0;
         int st = ISING_OK;
         for (int k = 0; k < K && st == ISING_OK; ++k) {
             st = enqueue_segment(b, times[k] - b->t, nullptr);
@@ -616,8 +616,8 @@ int ising_batch_run(ising_batch *b, const int64_t *times, int K, int64_t *rec, d
         b->gkey = key;
         b->graph_coop = b->coop;
     }
-    if (b->graph_coop) {  // the replay as a whole takes its place among the process's cooperative launches
-        const CoopOrder order(b->stream);
+    if (b->graph_coop > 0) {  // the replay as a whole takes its place among the process's cooperative launches
+        const CoopOrder order(b->stream, b->graph_coop);
         BCK(b, cudaGraphLaunch(b->gexec, b->stream));
     } else {
         BCK(b, cudaGraphLaunch(b->gexec, b->stream));

@@ -330,7 +330,7 @@ cudaError_t launch_batch(const BatchTask *tasks, int ntasks, const BatchLattice 
     cfg.numAttrs = 1;
     void *args[] = {(void *)&tasks, (void *)&lats, (void *)&t0, (void *)&n_mcs, (void *)&barriers,
                     (void *)&status, (void *)&timeout_ns, (void *)&missing_cta, (void *)&cta_ns};
-    const CoopOrder order(s);
+    const CoopOrder order(s, ntasks);
     return cudaLaunchKernelExC(&cfg, fn, args);
 }
 

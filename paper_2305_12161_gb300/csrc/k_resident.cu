@@ -669,37 +669,87 @@ static cudaError_t resident_cluster(uint32_t *lat, int L, int R, uint64_t seed, 
 }
 
 
-// Cooperative launches of this process on one device run one after the other, whatever their streams:
-// two that were resident in part would wait for each other's SMs until their bounds.  (Not while a
-// stream is being captured: an event recorded outside cannot order a graph.  The launch of the graph is
-// ordered instead.)
+// Cooperative launches of this process on one device run side by side while their CTAs, counted at one
+// per SM, fit the device, and wait for earlier ones otherwise: grids that were resident in part would
+// wait for each other's SMs until their bounds.  Launches that are ordered one behind the other form a
+// chain, as wide as its widest launch, and the chains in flight never add up to more CTAs than SMs.  (Two
+// 192^3 on streams of their own: 4.5 us per sweep of both side by side, 9.0 one after the other.  Not
+// while a stream is being captured: an event recorded outside cannot order a graph.  The launch of the
+// graph is ordered instead.)
 namespace {
 struct CoopChain {
-    std::mutex m;
-    cudaEvent_t ev = nullptr;
+    cudaEvent_t ev = nullptr;  // end of its last launch
+    cudaStream_t stream = nullptr;
+    int ctas = 0;              // 0: free
+    uint64_t seq = 0;
 };
-CoopChain g_coop[64];
+struct CoopDevice {
+    std::mutex m;
+    CoopChain chain[16];
+    uint64_t seq = 0;
+};
+CoopDevice g_coop[64];
 }  // namespace
 
-CoopOrder::CoopOrder(cudaStream_t s) : stream(s)
+CoopOrder::CoopOrder(cudaStream_t s, int ctas) : stream(s)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return;
     int d = -1;
     if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return;
     dev = d;
-    CoopChain &c = g_coop[dev];
-    c.m.lock();
-    if (c.ev) cudaStreamWaitEvent(stream, c.ev, 0);
-    else if (cudaEventCreateWithFlags(&c.ev, cudaEventDisableTiming) != cudaSuccess) c.ev = nullptr;
+    CoopDevice &g = g_coop[dev];
+    g.m.lock();
+    // an event may be queried while some other stream is being captured
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const int sms = device_sms();
+    width = std::max(1, std::min(ctas, sms));
+    const int need = width;
+    int busy = 0;
+    auto join = [&](CoopChain &c) {  // this launch continues c
+        cudaStreamWaitEvent(stream, c.ev, 0);
+        width = std::max(width, c.ctas);
+        busy -= c.ctas;
+        c.ctas = 0;
+    };
+    auto oldest = [&]() -> CoopChain & {
+        CoopChain *o = nullptr;
+        for (CoopChain &c : g.chain)
+            if (c.ctas && (!o || c.seq < o->seq)) o = &c;
+        return *o;
+    };
+    for (CoopChain &c : g.chain) {
+        if (c.ctas && cudaEventQuery(c.ev) == cudaSuccess) c.ctas = 0;
+        busy += c.ctas;
+    }
+    cudaGetLastError();  // "not ready" is kept as the last error
+    for (CoopChain &c : g.chain)
+        if (c.ctas && c.stream == stream) join(c);
+    while (busy + need > sms) join(oldest());
+    for (slot = 0; slot < 16 && g.chain[slot].ctas; ++slot) {
+    }
+    if (slot == 16) {
+        CoopChain &c = oldest();
+        slot = (int)(&c - g.chain);
+        join(c);
+    }
+    CoopChain &c = g.chain[slot];
+    if (!c.ev && cudaEventCreateWithFlags(&c.ev, cudaEventDisableTiming) != cudaSuccess) c.ev = nullptr;
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 CoopOrder::~CoopOrder()
 {
     if (dev < 0) return;
-    CoopChain &c = g_coop[dev];
-    if (c.ev) cudaEventRecord(c.ev, stream);
-    c.m.unlock();
+    CoopDevice &g = g_coop[dev];
+    CoopChain &c = g.chain[slot];
+    if (c.ev && cudaEventRecord(c.ev, stream) == cudaSuccess) {
+        c.stream = stream;
+        c.ctas = width;
+        c.seq = ++g.seq;
+    }
+    g.m.unlock();
 }
 
 // Whether and how R lattices of size L are swept resident (host arithmetic; sms: the device's SMs).
@@ -776,7 +826,7 @@ cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, i
             if (p.cluster) {
                 e = resident_cluster(l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, p.groups, s);
             } else {
-                const CoopOrder order(s);
+                const CoopOrder order(s, nr * p.ctas);
                 e = resident_grid(l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, bar, err, timeout_s, s);
             }
             // a device that cannot hold the clusters or the grid (a partition of the GPU) refuses the

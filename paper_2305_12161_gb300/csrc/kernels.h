@@ -75,18 +75,19 @@ cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, i
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
                                    int64_t *launches);
 
-// Scope around a cooperative launch on stream s, or the launch of a graph that holds some: it runs after
-// the previous one of this process on the current device (nothing is ordered while s is being captured).
+// Scope around a cooperative launch of `ctas` CTAs on stream s, or the launch of a graph whose largest one
+// has that many: it waits for those of this process on the current device beside which its CTAs would
+// not fit at one per SM (nothing is ordered while s is being captured).
 class CoopOrder {
 public:
-    explicit CoopOrder(cudaStream_t s);
+    CoopOrder(cudaStream_t s, int ctas);
     ~CoopOrder();
     CoopOrder(const CoopOrder &) = delete;
     CoopOrder &operator=(const CoopOrder &) = delete;
 
 private:
     cudaStream_t stream;
-    int dev = -1;
+    int dev = -1, slot = 0, width = 0;
 };
 
 // Double-checkerboard update (Supp. Methods I A): blocks of bx*by*bz sites, red blocks

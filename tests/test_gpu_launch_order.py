@@ -78,6 +78,46 @@ def test_replayed_batch_waits_for_a_context_s_resident_sweep(ising):
         assert np.array_equal(rec.cpu().numpy(), want)
 
 
+def test_resident_sweeps_that_fit_run_side_by_side(ising):
+    # 48 CTAs each: the short call ends inside the long one; two more fill the device and a fourth waits
+    import torch
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    ctx = [ising.Ising(192, replicas=1, seed=40 + i, stream=s) for i, s in enumerate(streams)]
+    for q in ctx:
+        q.sweep(4)
+        q.sync()
+    ev = [torch.cuda.Event(enable_timing=True) for _ in ctx]
+    for q, s, e, n in zip(ctx, streams, ev, (8000, 8, 8000, 8)):
+        q.sweep(n)
+        e.record(s)
+    for q in ctx:
+        q.sync()
+    assert ev[1].elapsed_time(ev[0]) > 0
+    for i, q in enumerate(ctx):
+        with ising.Ising(192, replicas=1, seed=40 + i, variant=ising.VARIANT_WORD) as p:
+            p.sweep(q.t)
+            assert np.array_equal(p.get_packed(0), q.get_packed(0)), i
+        q.destroy()
+
+
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_many_contexts_in_any_order(ising, seed):
+    # widths from 12 to 150 CTAs on eleven streams, in a random order
+    import torch
+    rng = np.random.default_rng(seed)
+    spec = [(192, 1), (192, 3), (192, 12), (256, 1), (256, 2), (256, 9), (320, 1), (320, 4), (384, 1), (512, 1), (192, 1)]
+    ctx = [ising.Ising(L, replicas=R, seed=100 * i + 1, stream=torch.cuda.Stream()) for i, (L, R) in enumerate(spec)]
+    for _ in range(120):
+        ctx[int(rng.integers(len(ctx)))].sweep(int(rng.integers(3, 40)))
+    for (L, R), q, i in zip(spec, ctx, range(len(spec))):
+        q.sync()
+        with ising.Ising(L, replicas=R, seed=100 * i + 1) as p:
+            p.sweep(q.t)
+            for r in range(R):
+                assert np.array_equal(p.get_packed(r), q.get_packed(r)), (L, R, r)
+        q.destroy()
+
+
 def test_context_sweeps_between_batch_replays(ising):
     import torch
     classes, times = [(512, 1, 9), (256, 2, 30)], [12, 40, 41, 80]
