@@ -7,6 +7,7 @@
 namespace ising {
 
 constexpr int BATCH_THREADS = 256;
+constexpr int BATCH_MAX_SMEM = 96 * 1024;  // largest lattice kept in a CTA's shared memory
 constexpr int BATCH_LOCAL = 0;   // CTA owns whole lattices, kept in shared memory
 constexpr int BATCH_GROUP = 1;   // CTA is one rank of a group sharing a lattice
 constexpr int BATCH_STATUS_TIMEOUT = 1;

@@ -354,7 +354,7 @@ int assign_modes(ising_batch *b)
         const Geom g = make_geom(k.L);
         for (int r = 0; r < k.R; ++r)
             b->h_lats.push_back(BatchLattice{k.lat + (int64_t)r * 2 * g.nw, k.seed + (uint64_t)r, k.L, 0});
-        if (lattice_bytes(k.L) <= 96 * 1024) max_local = std::max<int>(max_local, (int)lattice_bytes(k.L));
+        if (lattice_bytes(k.L) <= BATCH_MAX_SMEM) max_local = std::max<int>(max_local, (int)lattice_bytes(k.L));
     }
     int nstreamed = 0;
     for (const auto &k : b->cls) nstreamed += k.streamed;

@@ -298,14 +298,14 @@ done:
 
 cudaError_t batch_occupancy(int smem_bytes, int *blocks_per_sm)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_batch<TIE_GLAUBER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_batch<TIE_ALWAYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_batch<TIE_NEVER>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-    if (e != cudaSuccess) return e;
+    // the most any batch asks for: a limit set to this batch's need would refuse the launches of a batch
+    // created earlier with a larger one
+    for (const void *fn : {(const void *)k_batch<TIE_GLAUBER>, (const void *)k_batch<TIE_ALWAYS>, (const void *)k_batch<TIE_NEVER>}) {
+        const cudaError_t a = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, BATCH_MAX_SMEM);
+        if (a != cudaSuccess) return a;
+    }
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<TIE_GLAUBER>, BATCH_THREADS, smem_bytes);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch<TIE_GLAUBER>, BATCH_THREADS, smem_bytes);
     *blocks_per_sm = occ;
     return e;
 }

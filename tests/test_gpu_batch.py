@@ -219,3 +219,16 @@ def test_config4_mix_in_the_bench_configuration(ising):
             with ising.Ising(L, replicas=1, seed=seed) as q:
                 q.set_spins(s, 0)
                 assert np.array_equal(b.get_packed(ci, 0), q.get_packed(0)), L
+
+
+def test_a_later_batch_leaves_an_earlier_one_s_launches_alone(ising):
+    # the persistent kernel keeps 64^3 lattices in shared memory; the second batch needs none of it
+    classes = [(32, 2, 1), (64, 3, 10)]
+    with ising.Batch(classes) as a, ising.Batch([(576, 1, 5)]) as b:
+        b.sweep(1)
+        a.sweep(4)
+        for ci, (L, R, seed) in enumerate(classes):
+            with ising.Ising(L, replicas=R, seed=seed, variant=ising.VARIANT_WORD) as q:
+                q.sweep(4)
+                for r in range(R):
+                    assert np.array_equal(a.get_packed(ci, r), q.get_packed(r)), (L, r)
