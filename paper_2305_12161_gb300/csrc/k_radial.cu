@@ -479,16 +479,13 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
     const int fold_threads = ((nx + passes - 1) / passes + 31) / 32 * 32;
     const unsigned grid = (unsigned)(sms * std::max(1, 2048 / fold_threads));
     const int chunk = std::max(1, std::min(16, nx * nx / (4 * (int)grid)));
-    const size_t smem = (size_t)nb * sizeof(double);
+    const size_t smem = (size_t)nb * sizeof(double);  // 28 KB at L = 4096: within the default limit
     if (!p->count) {
         if ((e = cudaMallocAsync((void **)&p->count, sizeof(unsigned long long) * nb, s)) != cudaSuccess) {
             p->count = nullptr;
             return e;
         }
         if ((e = cudaMemsetAsync(p->count, 0, sizeof(unsigned long long) * nb, s)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_radial_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-            return e;
         k_radial_count<<<grid, fold_threads, smem, s>>>(L, chunk, nb, p->count);
         if (launches) *launches += 1;
     }
@@ -509,8 +506,6 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
         *cufft_status = cs;
         return cudaErrorUnknown;
     }
-    if ((e = cudaFuncSetAttribute(k_power<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
     k_power<T><<<grid, fold_threads, smem, s>>>(reinterpret_cast<C *>(p->buf), L, chunk, nb, sumS);
     if (prec)
         cs = cufftExecZ2D(iv, reinterpret_cast<cufftDoubleComplex *>(p->buf), reinterpret_cast<cufftDoubleReal *>(p->buf));
@@ -522,7 +517,6 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
     }
     const double invN = 1.0 / ((double)L * (double)L * (double)L);  // exact: N is a power of two
     auto corr = (int64_t)L * L * L <= (1 << 27) ? k_radial_corr<T, true> : k_radial_corr<T, false>;
-    if ((e = cudaFuncSetAttribute(corr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     corr<<<grid, fold_threads, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, chunk, P, nb, invN, sumG, inexact);
     k_radial_finish<<<1, 256, 0, s>>>(L, nb, c, sumG, sumS, p->count, inexact, out, cnt);
     if (launches) *launches += 4;  // own kernels; the two cuFFT executions are library launches

@@ -561,7 +561,10 @@ static cudaError_t launch_res(const ResArgs &ra, int R, cudaStream_t s)
     const int threads = ra.P * U / G;
     const size_t smem = (size_t)2 * (ra.P + 2) * U * sizeof(uint4);
     auto kern = k_resident<RULE, KIND, G, MAXT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is the same whatever the plan (two CTAs per lattice need the most): another thread may launch
+    // the kernel with another plan between this call and the launch
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         2 * ((KIND == RES_W1 ? 32 : 64) + 2) * U * (int)sizeof(uint4));
     if (e == cudaSuccess && ra.CS > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
@@ -589,13 +592,15 @@ static cudaError_t res_rule(ResArgs ra, int R, int G, cudaStream_t s)
     }
 }
 
+constexpr int RESG_MAX_SMEM = 220 * 1024;  // of every plan; the kernel's limit, as above
+
 template <int RULE, int W>
 static cudaError_t launch_resg(const ResGArgs &ra, int R, cudaStream_t s)
 {
     constexpr int U = ResPlane<W>::U;
     const size_t smem = (size_t)2 * ra.P * ResPlane<W>::PU * sizeof(uint4);
     auto kern = k_resident_grid<RULE, W>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, RESG_MAX_SMEM);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)(R * ra.NC));
@@ -792,7 +797,7 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
     double best = 1e300;
     for (int P = 4; P <= L / 2; P += 4) {
         if (L % P != 0 || P * U / 4 > 1024 || L / P > sms || (W >= 6 && P != 4)) continue;
-        if ((size_t)2 * P * resg_plane(W) * sizeof(uint4) > 220 * 1024) continue;
+        if ((size_t)2 * P * resg_plane(W) * sizeof(uint4) > RESG_MAX_SMEM) continue;
         const int per = std::min(R, sms / (L / P));
         const int rounds = (R + per - 1) / per;
         const double us = whole ? std::max(3.4, 1.2 + 1.35e-3 * P * U) : std::max(4.9, 3.5 + 2.05e-3 * P * U);

@@ -113,3 +113,31 @@ def test_batches_replayed_on_two_streams(ising):
         b.sync()
         assert np.array_equal(rec.cpu().numpy(), w)
         b.destroy()
+
+
+def test_threads_with_different_plans(ising):
+    # 135 and 20 KB of shared memory per CTA of one kernel, launched from two threads
+    import threading
+    import torch
+    spec, bad = [(128, 64, 1000 * i + 1) if i % 2 else (128, 12, 1000 * i + 1) for i in range(8)], []
+    ctx = [ising.Ising(L, replicas=R, seed=s, stream=torch.cuda.Stream()) for L, R, s in spec]
+
+    def work(q):
+        try:
+            for _ in range(1500):
+                q.sweep(1)
+            q.sync()
+        except ising.IsingError as e:
+            bad.append(str(e))
+
+    threads = [threading.Thread(target=work, args=(q,)) for q in ctx]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+    for (L, R, s), q in zip(spec, ctx):
+        with ising.Ising(L, replicas=1, seed=s + R - 1, variant=ising.VARIANT_WORD) as p:
+            p.sweep(1500)
+            assert np.array_equal(p.get_packed(0), q.get_packed(R - 1))
+        q.destroy()
