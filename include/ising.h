@@ -315,9 +315,10 @@ int64_t ising_launch_count(const ising_ctx *ctx);
  * 256 and at least the streaming threshold (default 256; ising_batch_set_streamed) are
  * instead swept in the same segment by a single-lattice sweep kernel (the z-marching one
  * by default, the one ising_batch_tune picks after tuning), which streams them faster
- * than slab groups do.  In segments of a few sweeps or more, classes of a size with a resident
- * sweep (ising_opts.variant) run that instead, one class after the other: streamed classes on
- * their default kernel, and the persistent kernel's classes when all of them have one.  Every
+ * than slab groups do.  Classes of a size with a resident sweep (ising_opts.variant) run that
+ * instead where an estimate finds it faster for the segment, the classes of one size in one
+ * launch (or one per group of lattices), one size after the other: streamed classes on their
+ * default kernel, and the persistent kernel's classes when all of them have one.  Every
  * lattice follows exactly the trajectory of the single-lattice entry points (same rule, order
  * and random bits), so batching changes speed, not results.
  * Records and derived values are concatenated in class order, replica-major within a

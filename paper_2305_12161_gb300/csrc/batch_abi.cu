@@ -23,7 +23,8 @@ namespace {
 struct BatchClass {
     int L, R;
     uint64_t seed;
-    uint32_t *lat;       // R * 2 * nw words
+    uint32_t *lat;       // R * 2 * nw words, behind the earlier classes of its size
+    bool owner;          // the size's first class: its `lat` is the size's allocation
     int64_t rec_off;     // offset of this class's records in a batch record block
     int64_t der_off;     // offset (in replicas) of this class's derived rows
     int streamed;        // swept by a single-lattice sweep kernel instead of the persistent one
@@ -31,6 +32,14 @@ struct BatchClass {
     int automatic;       // cfg is the default: long segments may run the resident sweep instead
     uint32_t *alt;       // second store of the fused whole-sweep kernel (allocated when chosen)
     uint32_t *xt;        // tensor-core correlation scratch (L >= 512), else null
+};
+
+// Classes of one size, behind one another in the size's allocation, that are swept resident together:
+// their lattices' keys are `count` entries of d_seeds from `first` on.
+struct ResidentGroup {
+    int L, count, first, streamed;
+    std::vector<int> cls;
+    ResidentPlan plan;
 };
 
 bool packed_L_ok(int L) { return (L >= 64 && L % 64 == 0) || L == 4 || L == 8 || L == 16 || L == 32; }
@@ -70,6 +79,8 @@ struct ising_batch {
     uint64_t timeout_ns = 2000000000ull;
     int missing_cta = -1;
     int no_resident = 0;     // the device refused the resident sweep's launch
+    std::vector<ResidentGroup> groups;
+    uint64_t *d_seeds = nullptr;
     int stream_min_L = 256;  // classes with L >= this (and L % 256 == 0) are streamed
     // measurement scratch
     int64_t *d_rec = nullptr;
@@ -207,6 +218,105 @@ int upload_plan(ising_batch *b)
     return ISING_OK;
 }
 
+// Groups of the classes that may be swept resident: every class of the persistent kernel and the streamed
+// ones on their default kernel, by size.  (A class with a kernel of its own parts the ones around it.)
+int build_groups(ising_batch *b)
+{
+    b->groups.clear();
+    std::vector<uint64_t> seeds;
+    std::vector<char> seen(b->cls.size(), 0);
+    for (size_t i = 0; i < b->cls.size(); ++i) {
+        ResidentGroup *g = nullptr;
+        for (size_t j = i; j < b->cls.size(); ++j) {
+            const BatchClass &k = b->cls[j];
+            if (seen[j] || k.L != b->cls[i].L) continue;
+            seen[j] = 1;
+            ResidentPlan p{};
+            if ((k.streamed && !k.automatic) || !resident_plan(k.L, k.R, b->sms, &p)) {
+                g = nullptr;
+                continue;
+            }
+            if (!g) {
+                b->groups.push_back(ResidentGroup{k.L, 0, (int)seeds.size(), k.streamed, {}, p});
+                g = &b->groups.back();
+            }
+            g->cls.push_back((int)j);
+            g->count += k.R;
+            for (int r = 0; r < k.R; ++r) seeds.push_back(k.seed + (uint64_t)r);
+        }
+    }
+    for (ResidentGroup &g : b->groups) resident_plan(g.L, g.count, b->sms, &g.plan);
+    cudaFree(b->d_seeds);
+    b->d_seeds = nullptr;
+    if (seeds.empty()) return ISING_OK;
+    if (cudaMalloc(&b->d_seeds, seeds.size() * sizeof(uint64_t)) != cudaSuccess) {
+        b->d_seeds = nullptr;
+        b->groups.clear();
+        return ISING_ENOMEM;
+    }
+    BCK(b, cudaMemcpyAsync(b->d_seeds, seeds.data(), seeds.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, b->stream));
+    BCK(b, cudaStreamSynchronize(b->stream));
+    return ISING_OK;
+}
+
+// Which classes a segment of n sweeps runs resident (res, by class); true when the persistent kernel's
+// are among them, all or none.  The cheapest of the four combinations (the persistent kernel's classes
+// resident or not, the streamed ones that can be resident or not).  A resident size costs its launches and
+// its sweeps (the plan).  What is left costs per sweep the longer of a floor of latency and its spins:
+// the persistent kernel 0.064 us times the largest L or 0.28 us per million spins, and 5.6 us to start;
+// streamed kernels 6.8 us or 0.09 us per million, and 1 us.  Measured, us per sweep over calls of 64:
+// sixteen classes of one 64^3 3.1 on the persistent kernel and 1.3 in one resident launch (18.8 with a
+// launch per class), sixteen of one 192^3 32.0 and 7.9, eight of one 256^3 25.8 streamed and 7.2; 8 x 64^3 +
+// 2 x 192^3 + 320^3 20.5 and 11.9, but over calls of two sweeps 23.3 and 26.2.
+bool choose_resident(const ising_batch *b, int64_t n, bool grid, bool small_allowed, std::vector<char> &res)
+{
+    double res_us[2] = {0, 0};  // resident: [0] the persistent kernel's classes, [1] streamed ones
+    std::vector<const ResidentGroup *> usable[2];
+    std::vector<char> can(b->cls.size(), 0);
+    for (const ResidentGroup &g : b->groups) {
+        if (b->no_resident || n < g.plan.min_n || !(grid || g.plan.cluster)) continue;
+        usable[g.streamed].push_back(&g);
+        res_us[g.streamed] += g.plan.start_us + (double)n * g.plan.us;
+        for (const int i : g.cls) can[i] = 1;
+    }
+    bool small = false, small_ok = small_allowed;
+    for (size_t i = 0; i < b->cls.size(); ++i) {
+        if (b->cls[i].streamed) continue;
+        small = true;
+        small_ok = small_ok && can[i];
+    }
+    auto rest_us = [&](bool p, bool s) {  // what runs neither of p, s resident costs
+        double wp = 0, fp = 0, ws = 0, fs = 0;
+        for (size_t i = 0; i < b->cls.size(); ++i) {
+            const BatchClass &k = b->cls[i];
+            const double m = 1e-6 * k.R * k.L * (double)k.L * k.L;
+            if (!k.streamed && !p) {
+                wp += 0.28 * m;
+                fp = std::max(fp, 0.064 * k.L);
+            } else if (k.streamed && !(s && can[i])) {
+                ws += 0.09 * m;
+                fs = std::max(fs, 6.8);
+            }
+        }
+        wp = std::max(wp, fp);
+        ws = std::max(ws, fs);
+        return (wp > 0 ? 5.6 : 0.0) + (ws > 0 ? 1.0 : 0.0) + (double)n * (b->overlap ? std::max(wp, ws) : wp + ws);
+    };
+    double best = 1e300;
+    bool bp = false, bs = false;
+    for (int c = 3; c >= 0; --c) {
+        const bool p = (c & 1) != 0, s = (c & 2) != 0;
+        if ((p && !(small && small_ok)) || (s && usable[1].empty())) continue;
+        const double us = (p ? res_us[0] : 0.0) + (s ? res_us[1] : 0.0) + rest_us(p, s);
+        if (us < best) best = us, bp = p, bs = s;
+    }
+    for (int k = 0; k < 2; ++k)
+        if (k == 0 ? bp : bs)
+            for (const ResidentGroup *g : usable[k])
+                for (const int i : g->cls) res[i] = 1;
+    return bp;
+}
+
 // Enqueue one segment of n MCS (split at 2^30 sweeps per launch).  grid: the resident sweeps that are
 // cooperative launches may be used.
 int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool grid = true)
@@ -214,23 +324,12 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
     while (n > 0) {
         const int chunk = (int)std::min<int64_t>(n, 1 << 30);
         int nstreamed = 0, si = 0;
-        // classes swept resident in shared memory (k_resident.cu), on the batch's stream one after the
-        // other (each fills the GPU): streamed classes on their default kernel, and the persistent
-        // kernel's classes when every one of them can be (the tuner's probes, which time that kernel's
-        // CTAs, and the failure injection into it keep it)
-        std::vector<ResidentPlan> rp(b->cls.size());
+        // classes swept resident in shared memory (k_resident.cu), one size after the other on the batch's
+        // stream (the tuner's probes, which time the persistent kernel's CTAs, and the failure injection
+        // into it keep it)
         std::vector<char> res(b->cls.size(), 0);
-        bool all_small = cta_ns == nullptr && b->missing_cta < 0;
-        for (size_t i = 0; i < b->cls.size(); ++i) {
-            const auto &k = b->cls[i];
-            res[i] = !b->no_resident && (k.automatic || !k.streamed) && resident_plan(k.L, k.R, b->sms, &rp[i]) &&
-                     chunk >= rp[i].min_n && (grid || rp[i].cluster);
-            if (!k.streamed && !res[i]) all_small = false;
-        }
-        for (size_t i = 0; i < b->cls.size(); ++i) {
-            if (!b->cls[i].streamed) res[i] = res[i] && all_small;
-            else nstreamed += !res[i];
-        }
+        const bool all_small = choose_resident(b, chunk, grid, cta_ns == nullptr && b->missing_cta < 0, res);
+        for (size_t i = 0; i < b->cls.size(); ++i) nstreamed += b->cls[i].streamed && !res[i];
         const bool persistent = !b->h_tasks.empty() && !all_small;
         // side streams: every streamed class when they overlap the persistent launch, else all
         // but the first, which follows the persistent launch on the batch's stream
@@ -246,18 +345,22 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
                                 b->stream));
             b->launches += 1;
         }
-        for (size_t i = 0; i < b->cls.size(); ++i) {
-            const auto &k = b->cls[i];
-            if (!res[i]) continue;
-            if (!rp[i].cluster) b->coop = std::max(b->coop, std::min(k.R, rp[i].per_launch) * rp[i].ctas);
-            const cudaError_t e = launch_sweeps_resident(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, rp[i], b->d_status,
-                                                         (double)b->timeout_ns * 1e-9, b->stream, &b->launches);
-            if (e == cudaErrorNotSupported) {
-                // refused before this class's first launch: its sweeps one launch per half-sweep
-                b->no_resident = 1;
-                BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, k.cfg, b->stream, &b->launches));
-            } else {
+        for (const ResidentGroup &g : b->groups) {
+            if (!res[g.cls[0]]) continue;
+            if (!g.plan.cluster) b->coop = std::max(b->coop, std::min(g.count, g.plan.per_launch) * g.plan.ctas);
+            const BatchClass &k0 = b->cls[g.cls[0]];
+            const cudaError_t e =
+                launch_sweeps_resident(k0.lat, g.L, g.count, k0.seed, b->rule, b->t, chunk, 0, g.plan, b->d_status,
+                                       (double)b->timeout_ns * 1e-9, b->stream, &b->launches,
+                                       g.cls.size() > 1 ? b->d_seeds + g.first : nullptr);
+            if (e != cudaErrorNotSupported) {
                 BCK(b, e);
+                continue;
+            }
+            b->no_resident = 1;  // refused before the group's first launch: one launch per half-sweep
+            for (const int i : g.cls) {
+                const BatchClass &k = b->cls[i];
+                BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, k.cfg, b->stream, &b->launches));
             }
         }
         if (first_side == 1 && nstreamed > 1) BCK(b, cudaEventRecord(b->ev[0], b->stream));
@@ -383,7 +486,7 @@ int assign_modes(ising_batch *b)
     if (b->occ < 1) return bfail(b, ISING_ECUDA, "batch kernel does not fit an SM");
     b->capacity = b->occ * b->sms;
     int s = build_plan(b);
-    if (s != ISING_OK) return s;
+    if (s != ISING_OK || (s = build_groups(b)) != ISING_OK) return s;
     return upload_plan(b);
 }
 
@@ -417,7 +520,7 @@ int ising_batch_destroy(ising_batch *b)
         if (b->stream) cudaStreamSynchronize(b->stream);
         if (b->gexec) cudaGraphExecDestroy(b->gexec);
         for (auto &k : b->cls) {
-            cudaFree(k.lat);
+            if (k.owner) cudaFree(k.lat);
             cudaFree(k.alt);
             cudaFree(k.xt);
         }
@@ -425,6 +528,7 @@ int ising_batch_destroy(ising_batch *b)
         cudaFree(b->d_tasks);
         cudaFree(b->d_barriers);
         cudaFree(b->d_status);
+        cudaFree(b->d_seeds);
         cudaFree(b->d_cta_ns);
         cudaFree(b->d_rec);
         cudaFree(b->d_der);
@@ -473,25 +577,28 @@ int ising_batch_create(ising_batch **out, int nclass, const int *L, const int *r
     }
     int64_t rec_off = 0, der_off = 0;
     for (int c = 0; c < nclass; ++c) {
-        BatchClass k{L[c], replicas[c], seeds[c], nullptr, rec_off, der_off, 0, SweepConfig{VARIANT_WORD, 0, 0, 0},
-                     1, nullptr, nullptr};
+        BatchClass k{L[c], replicas[c], seeds[c], nullptr, false, rec_off, der_off, 0,
+                     SweepConfig{VARIANT_WORD, 0, 0, 0}, 1, nullptr, nullptr};
         const int64_t bytes = lattice_bytes(L[c]) * replicas[c];
-        if (cudaMalloc(&k.lat, (size_t)bytes) != cudaSuccess) {
-            b->cls.push_back(k);
-            return bail(ISING_ENOMEM);
+        for (const auto &p : b->cls)
+            if (p.L == k.L) k.lat = p.lat + lattice_bytes(p.L) / 4 * p.R;
+        if (!k.lat) {
+            int64_t all = 0;
+            for (int d = c; d < nclass; ++d)
+                if (L[d] == L[c]) all += lattice_bytes(L[d]) * replicas[d];
+            if (cudaMalloc(&k.lat, (size_t)all) != cudaSuccess) return bail(ISING_ENOMEM);
+            k.owner = true;
         }
         // L >= 512: the tensor-core measurement's scratch is allocated here, never while a schedule
         // is being captured
         if (L[c] >= 512 && corr_mma_supported(L[c]) &&
             cudaMalloc(&k.xt, corr_mma_scratch_bytes(L[c], replicas[c])) != cudaSuccess) {
             k.xt = nullptr;
-            cudaFree(k.lat);
-            k.lat = nullptr;
             b->cls.push_back(k);
             return bail(ISING_ENOMEM);
         }
-        if (L[c] < 64 && cudaMemsetAsync(k.lat, 0, (size_t)bytes, b->stream) != cudaSuccess) return bail(ISING_ECUDA);
-        if (launch_init_packed(k.lat, L[c], replicas[c], seeds[c], b->stream) != cudaSuccess) {
+        if ((L[c] < 64 && cudaMemsetAsync(k.lat, 0, (size_t)bytes, b->stream) != cudaSuccess) ||
+            launch_init_packed(k.lat, L[c], replicas[c], seeds[c], b->stream) != cudaSuccess) {
             b->cls.push_back(k);
             return bail(ISING_ECUDA);
         }
@@ -812,6 +919,7 @@ int ising_batch_set_class_opts(ising_batch *b, int cls, const ising_opts *o)
     k.cfg = cfg;
     k.cfg.pdl = b->pdl;
     k.automatic = o->variant == 0;
+    if ((s = build_groups(b)) != ISING_OK) return bfail(b, s, "table of the resident classes");
     if (b->gexec) {  // the cached schedule graph holds the old kernels
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;

@@ -31,6 +31,7 @@ struct ResArgs {
     uint4 *lat;     // replica 0
     int64_t nw4;    // uint4 per sublattice
     uint64_t seed;
+    const uint64_t *seeds;  // Philox keys of the launch's lattices, or null: seed + replica
     int L, P, CS;
     uint32_t t0;
     int n;          // sweeps
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResArgs ra)
             z = z < 0 ? z + L : (z >= L ? z - L : z);
             rsm[q * sub + pl * U + nu] = __ldcg(lat + (int64_t)q * ra.nw4 + (int64_t)z * U + nu);
         }
-    res_keys(keys, S);
+    res_keys(keys, ra.seeds ? ra.seeds[r] : S);
     const int s = tid % U, zl = G * (tid / U);
     const uint32_t grp0 = (uint32_t)((c * P + zl) * U + s);
     // first uint4 of the thread's column in a sublattice (plane zl - 1 is storage plane zl)
@@ -259,6 +260,7 @@ struct ResGArgs {
     uint4 *lat;      // first replica of the launch
     int64_t nw4;
     uint64_t seed;
+    const uint64_t *seeds;  // as in ResArgs
     int P, NC;
     uint32_t t0;
     int n, mixed;
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
                 }
             }
         }
-    res_keys(keys, S);
+    res_keys(keys, ra.seeds ? ra.seeds[r] : S);
     const int s = ONE ? tid : tid % U, zl = ONE ? 0 : 4 * (tid / U);
     const uint32_t grp0 = (uint32_t)((c * P + zl) * U + unit_of(s));
     const bool lo = ONE || zl == 0, hi = ONE || zl + 4 == P;
@@ -629,11 +631,12 @@ static cudaError_t resg_rule(const ResGArgs &ra, int W, int R, cudaStream_t s)
     }
 }
 
-static cudaError_t resident_grid(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
+static cudaError_t resident_grid(const uint64_t *seeds, uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                         int cycle, int NC, unsigned *bar, int *err, double timeout_s, cudaStream_t s)
 {
     const Geom g = make_geom(L);
     ResGArgs ra{};
+    ra.seeds = seeds;
     ra.lat = reinterpret_cast<uint4 *>(lat);
     ra.nw4 = g.nw / 4;
     ra.seed = seed;
@@ -652,11 +655,12 @@ static cudaError_t resident_grid(uint32_t *lat, int L, int R, uint64_t seed, int
     }
 }
 
-static cudaError_t resident_cluster(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
+static cudaError_t resident_cluster(const uint64_t *seeds, uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                        int cycle, int CS, int G, cudaStream_t s)
 {
     const Geom g = make_geom(L);
     ResArgs ra{};
+    ra.seeds = seeds;
     ra.lat = reinterpret_cast<uint4 *>(lat);
     ra.nw4 = g.nw / 4;
     ra.seed = seed;
@@ -787,6 +791,8 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
         }
         p.per_launch = std::min(R, 4096);
         p.min_n = 1;
+        p.us = L == 64 ? std::max(1.0, 0.3 + 0.009 * R) : std::max(1.35, 0.3 + 0.095 * R);
+        p.start_us = 4.5;
         p.cluster = true;
         *out = p;
         return true;
@@ -803,6 +809,8 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
         const double us = whole ? std::max(3.4, 1.2 + 1.35e-3 * P * U) : std::max(4.9, 3.5 + 2.05e-3 * P * U);
         if (rounds * us < best) {
             best = rounds * us;
+            p.us = best;
+            p.start_us = 12.0 * rounds;
             p.ctas = L / P;
             p.per_launch = per;
         }
@@ -817,7 +825,7 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
 
 cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
-                                   int64_t *launches)
+                                   int64_t *launches, const uint64_t *seeds)
 {
     const int64_t words = 2 * make_geom(L).nw;
     unsigned *bar = reinterpret_cast<unsigned *>(err + 1);
@@ -827,12 +835,13 @@ cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, i
         for (int r0 = 0; r0 < R; r0 += p.per_launch) {
             const int nr = std::min(p.per_launch, R - r0);
             uint32_t *l = lat + (int64_t)r0 * words;
+            const uint64_t *sr = seeds ? seeds + r0 : nullptr;
             cudaError_t e;
             if (p.cluster) {
-                e = resident_cluster(l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, p.groups, s);
+                e = resident_cluster(sr, l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, p.groups, s);
             } else {
                 const CoopOrder order(s, nr * p.ctas);
-                e = resident_grid(l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, bar, err, timeout_s, s);
+                e = resident_grid(sr, l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, bar, err, timeout_s, s);
             }
             // a device that cannot hold the clusters or the grid (a partition of the GPU) refuses the
             // first launch, before anything is enqueued

@@ -68,12 +68,14 @@ struct ResidentPlan {
     int groups;      // Philox groups per thread and half-sweep
     int per_launch;  // lattices per launch
     int min_n;       // sweeps per call from which it is the faster way
+    double us;       // of a sweep of all lattices, about
+    double start_us; // of the launches, beside their sweeps, about
 };
 bool resident_plan(int L, int R, int sms, ResidentPlan *out);
-// Returns cudaErrorNotSupported, with nothing enqueued, where the device cannot hold the launch.
+// Replica r has the Philox key seed + r, or seeds[r] (device memory; cycle 01 only).  Returns cudaErrorNotSupported, with nothing enqueued, where the device cannot hold the launch.
 cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
-                                   int64_t *launches);
+                                   int64_t *launches, const uint64_t *seeds = nullptr);
 
 // Scope around a cooperative launch of `ctas` CTAs on stream s, or the launch of a graph whose largest one
 // has that many: it waits for those of this process on the current device beside which its CTAs would

@@ -141,3 +141,44 @@ def test_threads_with_different_plans(ising):
             p.sweep(1500)
             assert np.array_equal(p.get_packed(0), q.get_packed(R - 1))
         q.destroy()
+
+
+def _batch_states(b, classes):
+    return [b.get_packed(ci, r) for ci, (L, R, _) in enumerate(classes) for r in range(R)]
+
+
+def _word_states(ising, classes, n):
+    """The same sweeps by the one-word-per-thread half-sweep kernel, in a context per class."""
+    out = []
+    for L, R, seed in classes:
+        with ising.Ising(L, replicas=R, seed=seed, variant=ising.VARIANT_WORD) as q:
+            q.sweep(n)
+            out += [q.get_packed(r) for r in range(R)]
+    return out
+
+
+@pytest.mark.parametrize("classes,launches,without", [
+    ([(64, 1, 5), (64, 3, 70), (128, 1, 90), (64, 1, 2**64 - 1), (128, 2, 300)], 2, None),
+    # ten 256^3 take three launches, nine (more planes per CTA) one
+    ([(192, 1, 1), (256, 1, 20), (192, 2, 30), (256, 2, 40), (512, 1, 50), (256, 7, 60)], 5, 3),
+    ([(320, 1, 1), (384, 1, 2), (448, 1, 3), (320, 1, 4)], 3, None)])
+def test_batch_classes_of_one_size_share_launches(ising, classes, launches, without):
+    n = 24
+    want = _word_states(ising, classes, n)
+    with ising.Batch(classes) as b:
+        l0 = b.launch_count()
+        b.sweep(n)
+        # one launch per size and group of lattices that fit the device together
+        assert b.launch_count() - l0 == launches
+        assert all(np.array_equal(x, y) for x, y in zip(_batch_states(b, classes), want))
+        b.reinit()
+        rec, _ = b.run([5, n])
+        assert all(np.array_equal(x, y) for x, y in zip(_batch_states(b, classes), want))
+        # a class with a kernel of its own leaves the others together
+        if without:
+            b.set_class_config(1, variant=ising.VARIANT_ZFAST, tile_z=8)
+            b.reinit()
+            l0 = b.launch_count()
+            b.sweep(n)
+            assert b.launch_count() - l0 == without + 2 * n
+            assert all(np.array_equal(x, y) for x, y in zip(_batch_states(b, classes), want))
