@@ -355,17 +355,18 @@ int ising_batch_plan(const ising_batch *b, int *ntasks, int *nlocal, int *ngroup
 /* Autotuner: probe rounds of probe_mcs sweeps (they advance the batch) time every CTA,
  * set the relative cost of whole-lattice CTAs from the measured time per spin and
  * rebuild the work list; *w_local_out receives the chosen weight.  Then every streamed
- * class, one after the other, keeps whichever of its default kernel and the kernel that
- * ising_tune_sweep picks for its L and replica count alone gives the faster whole segment
+ * class, one after the other, keeps whichever of its default kernel and the one that is
+ * fastest for its L and replica count alone gives the faster whole segment
  * (the streamed classes of a segment run side by side on their own streams, forked from
  * and joined back into the batch's stream, so they compete for the SMs); last, it keeps
  * the faster of the streamed classes beside or after the persistent launch
- * (ising_batch_set_overlap). */
+ * (ising_batch_set_overlap).  All of this is for the segments that do not run resident sweeps:
+ * no probe does, and classes of a size that has them keep them for their other segments. */
 int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out);
 /* Sweep kernel of streamed class `cls` (Methods, "Checkerboard update"; every choice gives
  * the same trajectory): opts->variant, tile_y, tile_z and depth as for ising_create_ex,
- * variant 0 = the default for the class's L and replica count; the other fields are
- * ignored.  Variant 5 (both sublattices per launch, up to 16 replicas of the class per
+ * variant 0 = the default for the class's L and replica count, and resident sweeps where
+ * they are faster (none with any other variant); the other fields are ignored.  Variant 5 (both sublattices per launch, up to 16 replicas of the class per
  * launch) allocates a second store of the class's size, kept until ising_batch_destroy;
  * a segment then runs its whole sweeps in pairs between the two stores and an odd last
  * sweep in place, so the state is always in the first store between segments.
@@ -373,8 +374,8 @@ int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out);
  * ISING_ENOMEM: the second store could not be allocated.  Drops the cached schedule graph.
  * ising_batch_set_streamed puts every streamed class back on its default kernel. */
 int ising_batch_set_class_opts(ising_batch *b, int cls, const ising_opts *opts);
-/* The sweep kernel of class `cls` into opts (variant -1: the class is swept by the
- * persistent kernel); ISING_EINVAL for a bad class or NULL pointer. */
+/* The sweep kernel of class `cls` into opts, for segments that do not run it resident (variant
+ * -1: the class is swept by the persistent kernel); ISING_EINVAL for a bad class or NULL pointer. */
 int ising_batch_get_class_opts(const ising_batch *b, int cls, ising_opts *opts);
 /* on = 1: within a segment the streamed classes run beside the persistent launch (every one
  * on a side stream forked before it); on = 0 (the default): after it.  The lattices of the

@@ -16,6 +16,12 @@
 #include "common.cuh"
 #include "kernels.h"
 
+namespace ising {
+// ising_abi.cu
+int tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base, bool resident, ising_opts *best,
+               double *best_ms_per_mcs);
+}  // namespace ising
+
 using namespace ising;
 
 namespace {
@@ -29,7 +35,7 @@ struct BatchClass {
     int64_t der_off;     // offset (in replicas) of this class's derived rows
     int streamed;        // swept by a single-lattice sweep kernel instead of the persistent one
     SweepConfig cfg;     // that kernel's configuration (streamed classes)
-    int automatic;       // cfg is the default: long segments may run the resident sweep instead
+    int automatic;       // the caller set no kernel: segments may run the resident sweep instead
     uint32_t *alt;       // second store of the fused whole-sweep kernel (allocated when chosen)
     uint32_t *xt;        // tensor-core correlation scratch (L >= 512), else null
 };
@@ -79,6 +85,7 @@ struct ising_batch {
     uint64_t timeout_ns = 2000000000ull;
     int missing_cta = -1;
     int no_resident = 0;     // the device refused the resident sweep's launch
+    bool probing = false;    // the tuner times the other kernels
     std::vector<ResidentGroup> groups;
     uint64_t *d_seeds = nullptr;
     int stream_min_L = 256;  // classes with L >= this (and L % 256 == 0) are streamed
@@ -274,7 +281,7 @@ bool choose_resident(const ising_batch *b, int64_t n, bool grid, bool small_allo
     std::vector<const ResidentGroup *> usable[2];
     std::vector<char> can(b->cls.size(), 0);
     for (const ResidentGroup &g : b->groups) {
-        if (b->no_resident || n < g.plan.min_n || !(grid || g.plan.cluster)) continue;
+        if (b->no_resident || b->probing || n < g.plan.min_n || !(grid || g.plan.cluster)) continue;
         usable[g.streamed].push_back(&g);
         res_us[g.streamed] += g.plan.start_us + (double)n * g.plan.us;
         for (const int i : g.cls) can[i] = 1;
@@ -325,10 +332,10 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
         const int chunk = (int)std::min<int64_t>(n, 1 << 30);
         int nstreamed = 0, si = 0;
         // classes swept resident in shared memory (k_resident.cu), one size after the other on the batch's
-        // stream (the tuner's probes, which time the persistent kernel's CTAs, and the failure injection
-        // into it keep it)
+        // stream (not in the tuner's probes, which choose among the other kernels; the failure injection into
+        // the persistent kernel keeps it)
         std::vector<char> res(b->cls.size(), 0);
-        const bool all_small = choose_resident(b, chunk, grid, cta_ns == nullptr && b->missing_cta < 0, res);
+        const bool all_small = choose_resident(b, chunk, grid, b->missing_cta < 0, res);
         for (size_t i = 0; i < b->cls.size(); ++i) nstreamed += b->cls[i].streamed && !res[i];
         const bool persistent = !b->h_tasks.empty() && !all_small;
         // side streams: every streamed class when they overlap the persistent launch, else all
@@ -360,7 +367,9 @@ int enqueue_segment(ising_batch *b, int64_t n, unsigned long long *cta_ns, bool 
             b->no_resident = 1;  // refused before the group's first launch: one launch per half-sweep
             for (const int i : g.cls) {
                 const BatchClass &k = b->cls[i];
-                BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, k.cfg, b->stream, &b->launches));
+                SweepConfig cfg = default_sweep_config(k.L, k.R);
+                cfg.pdl = b->pdl;
+                BCK(b, launch_sweeps_packed(k.lat, k.L, k.R, k.seed, b->rule, b->t, chunk, 0, cfg, b->stream, &b->launches));
             }
         }
         if (first_side == 1 && nstreamed > 1) BCK(b, cudaEventRecord(b->ev[0], b->stream));
@@ -811,6 +820,12 @@ int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out)
     if (s) return s;
     if (probe_mcs < 1) return bfail(b, ISING_EINVAL, "probe_mcs must be >= 1");
     DevGuard dg(b->device);
+    // What is tuned is what segments run that are not resident: no probe is.
+    struct Probing {
+        ising_batch *b;
+        explicit Probing(ising_batch *x) : b(x) { b->probing = true; }
+        ~Probing() { b->probing = false; }
+    } probing(b);
     // Probe rounds: run a short segment, read each CTA's elapsed time, and set the LOCAL
     // weight to the measured ratio of time per spin (LOCAL vs GROUP); rebuild the plan.
     // The probe advances the batch (the state stays a valid trajectory: t moves on).
@@ -870,7 +885,7 @@ int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out)
         base.tie = (ising_tie)b->rule;
         base.device = b->device;
         dflt = base;
-        if (ising_tune_sweep(b->cls[c].L, b->cls[c].R, probe_mcs, &base, &alone, nullptr) != ISING_OK) {
+        if (tune_sweep(b->cls[c].L, b->cls[c].R, probe_mcs, &base, false, &alone, nullptr) != ISING_OK) {
             s = bfail(b, ISING_ECUDA, "tuning a streamed class");
             break;
         }
@@ -878,12 +893,10 @@ int ising_batch_tune(ising_batch *b, int probe_mcs, double *w_local_out)
         if ((s = ising_batch_set_class_opts(b, c, &dflt)) != ISING_OK || (s = segment_ms(&ms_dflt)) != ISING_OK ||
             (s = ising_batch_set_class_opts(b, c, &alone)) != ISING_OK || (s = segment_ms(&ms_alone)) != ISING_OK)
             break;
-        // a size with a resident sweep keeps its default, which runs it in all but the shortest
-        // segments: the probes are too short to show it
-        ResidentPlan rp{};
-        if (ms_dflt <= ms_alone || resident_plan(b->cls[c].L, b->cls[c].R, b->sms, &rp))
-            s = ising_batch_set_class_opts(b, c, &dflt);
+        if (ms_dflt <= ms_alone && (s = ising_batch_set_class_opts(b, c, &dflt)) != ISING_OK) break;
+        b->cls[c].automatic = 1;  // the tuned kernel is for the segments that are not resident
     }
+    if (s == ISING_OK && (s = build_groups(b)) != ISING_OK) s = bfail(b, s, "table of the resident classes");
     // the streamed classes beside the persistent launch, or after it
     if (s == ISING_OK && !b->h_tasks.empty() && ising_batch_streamed_classes(b) > 0) {
         float ms_after = 0.f, ms_beside = 0.f;

@@ -739,8 +739,13 @@ int ising_sync(ising_ctx *c)
     return check_device_waits(c);
 }
 
-int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base, ising_opts *best,
-                     double *best_ms_per_mcs)
+}  // extern "C"
+
+namespace ising {
+
+// ising_tune_sweep; resident: the automatic variant's resident sweep is a candidate too.
+int tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base, bool resident, ising_opts *best,
+               double *best_ms_per_mcs)
 {
     if (!best || probe_mcs < 1 || replicas < 1 || !packed_L_ok(L)) return ISING_EINVAL;
     ising_opts o;
@@ -750,7 +755,7 @@ int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base,
     std::vector<SweepConfig> cands;
     cands.push_back(SweepConfig{VARIANT_WORD, 0, 0, 0});
     ResidentPlan rp{};
-    if (resident_plan(L, replicas, device_sms(), &rp)) cands.push_back(SweepConfig{VARIANT_AUTO, 0, 0, 0});
+    if (resident && resident_plan(L, replicas, device_sms(), &rp)) cands.push_back(SweepConfig{VARIANT_AUTO, 0, 0, 0});
     const int tzs[] = {4, 8, 16, 32, 64};
     if (L >= 256 && L % 256 == 0) {
         const int W4 = L / 256;
@@ -823,4 +828,10 @@ int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base,
     return ISING_OK;
 }
 
-}  // extern "C"
+}  // namespace ising
+
+extern "C" int ising_tune_sweep(int L, int replicas, int probe_mcs, const ising_opts *base, ising_opts *best,
+                                double *best_ms_per_mcs)
+{
+    return tune_sweep(L, replicas, probe_mcs, base, true, best, best_ms_per_mcs);
+}

@@ -232,3 +232,26 @@ def test_a_later_batch_leaves_an_earlier_one_s_launches_alone(ising):
                 q.sweep(4)
                 for r in range(R):
                     assert np.array_equal(a.get_packed(ci, r), q.get_packed(r)), (L, r)
+
+
+def test_tuner_times_the_kernels_it_chooses_between(ising):
+    # no probe runs resident sweeps, which are one launch per size: at least 3 work-list rounds of 1 + 16
+    # launches, the class's default over 8 + 16 sweeps of two launches, the other candidate and the two
+    # overlap settings over as many of one or more, each beside the persistent launches
+    classes, n = [(64, 2, 1), (256, 1, 20)], 40
+    with ising.Batch(classes) as b:
+        l0 = b.launch_count()
+        b.tune(probe_mcs=8)
+        assert b.launch_count() - l0 >= 3 * 17 + (2 + 48) + (2 + 24) + 2 * (2 + 24)
+        # long segments still run resident, and short ones the tuned kernel
+        b.reinit()
+        l0 = b.launch_count()
+        b.sweep(n)
+        assert b.launch_count() - l0 == 2
+        b.sweep(1)
+        b.sweep(3)
+        for ci, (L, R, seed) in enumerate(classes):
+            with ising.Ising(L, replicas=R, seed=seed, variant=ising.VARIANT_WORD) as q:
+                q.sweep(n + 4)
+                for r in range(R):
+                    assert np.array_equal(b.get_packed(ci, r), q.get_packed(r)), (L, r)
