@@ -227,6 +227,11 @@ int ising_measure_radial(ising_ctx *ctx, int replica, int precision, double cval
  * flag, and the synchronising call returns ISING_ETIMEOUT (the context is then poisoned).
  * No fault is raised on the device. */
 int ising_inject_corr_stall(ising_ctx *ctx, double timeout_s);
+/* The same for the resident sweeps of L = 192 .. 512: in the next call that runs them block 0 leaves
+ * out one message to its neighbour (barrier = 0) or its arrival at the launch's first barrier
+ * (barrier = 1).  The waits of the other blocks run out after timeout_s, every block returns, later
+ * resident sweeps leave at once, and the next synchronising call returns ISING_ETIMEOUT. */
+int ising_inject_sweep_stall(ising_ctx *ctx, int barrier, double timeout_s);
 
 /* Free the scratch that measurements keep in the context (the radial measurement's transform
  * buffer and work area, the tensor-core correlation's expanded lattice) and the staging

@@ -38,6 +38,7 @@ struct ising_ctx {
     int xt_refused = 0;          // that scratch could not be allocated (AUTO then measures without it)
     double wait_timeout_s = 2.0; // bound of each device-side wait (tensor-core path)
     int inject_stall = 0;        // test hook: the next tensor-core measurement loses one load
+    int inject_sweep = 0;        // test hook: the next resident grid loses a message (1) or an arrival (2)
     int64_t t = 0;
     int poisoned = 0;
     int64_t launches = 0;
@@ -421,7 +422,8 @@ int ising_sweep(ising_ctx *c, int64_t n)
     ResidentPlan rp{};
     if (use_resident(c, n, &rp)) {
         e = launch_sweeps_resident(c->lat, c->L, c->R, c->seed, c->opts.tie, c->t, n, c->opts.cycle, rp, c->dev_err,
-                                   c->wait_timeout_s, c->stream, &c->launches);
+                                   c->wait_timeout_s, c->stream, &c->launches, nullptr, c->inject_sweep);
+        if (!rp.cluster) c->inject_sweep = 0;
         if (e == cudaSuccess) {
             c->t += n;
             return ISING_OK;
@@ -543,6 +545,17 @@ int ising_inject_corr_stall(ising_ctx *c, double timeout_s)
     if (!(timeout_s > 0) || timeout_s > 60) return fail(c, ISING_EINVAL, "timeout must be in (0, 60] s");
     c->wait_timeout_s = timeout_s;
     c->inject_stall = 1;
+    return ISING_OK;
+}
+
+int ising_inject_sweep_stall(ising_ctx *c, int barrier, double timeout_s)
+{
+    int s = check_ctx(c);
+    if (s) return s;
+    if (barrier != 0 && barrier != 1) return fail(c, ISING_EINVAL, "barrier must be 0 or 1");
+    if (!(timeout_s > 0) || timeout_s > 60) return fail(c, ISING_EINVAL, "timeout must be in (0, 60] s");
+    c->wait_timeout_s = timeout_s;
+    c->inject_sweep = 1 + barrier;
     return ISING_OK;
 }
 

@@ -267,6 +267,7 @@ struct ResGArgs {
     unsigned *bar;   // two zero counters: arrivals, departures (left zero)
     int *err;
     uint64_t timeout_ns;
+    int inject;      // tests: block 0 leaves out one message (1) or the first barrier (2) and the waits run out
 };
 
 __device__ __forceinline__ uint64_t res_timer_ns()
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
         }
     }
     __syncthreads();
-    if (*(volatile int *)&s_fail == 0) return;
+    if (*(volatile int *)&s_fail == 0 || (ra.inject == 2 && blockIdx.x == 0)) return;
     // the starting state's boundary planes are the messages of step 1
     for (int q = 0; q < 2; ++q) {
         const uint4 *col = gsm_res + q * sub + F + s;
@@ -425,7 +426,7 @@ __global__ void __launch_bounds__(1024) k_resident_grid(const ResGArgs ra)
             msg_st(msg(c, q, 0), v.x, v.y, 1u);
             msg_st(msg(c, q, 0) + U, v.z, v.w, 1u);
         }
-        if (hi) {
+        if (hi && !(ra.inject == 1 && blockIdx.x == 0)) {
             const uint4 v = col[(P - 1) * PU];
             msg_st(msg(c, q, 1), v.x, v.y, 1u);
             msg_st(msg(c, q, 1) + U, v.z, v.w, 1u);
@@ -632,10 +633,11 @@ static cudaError_t resg_rule(const ResGArgs &ra, int W, int R, cudaStream_t s)
 }
 
 static cudaError_t resident_grid(const uint64_t *seeds, uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
-                                        int cycle, int NC, unsigned *bar, int *err, double timeout_s, cudaStream_t s)
+                                        int cycle, int NC, unsigned *bar, int *err, double timeout_s, cudaStream_t s, int inject)
 {
     const Geom g = make_geom(L);
     ResGArgs ra{};
+    ra.inject = inject;
     ra.seeds = seeds;
     ra.lat = reinterpret_cast<uint4 *>(lat);
     ra.nw4 = g.nw / 4;
@@ -825,7 +827,7 @@ bool resident_plan(int L, int R, int sms, ResidentPlan *out)
 
 cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
-                                   int64_t *launches, const uint64_t *seeds)
+                                   int64_t *launches, const uint64_t *seeds, int inject)
 {
     const int64_t words = 2 * make_geom(L).nw;
     unsigned *bar = reinterpret_cast<unsigned *>(err + 1);
@@ -841,7 +843,8 @@ cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, i
                 e = resident_cluster(sr, l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, p.groups, s);
             } else {
                 const CoopOrder order(s, nr * p.ctas);
-                e = resident_grid(sr, l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, bar, err, timeout_s, s);
+                e = resident_grid(sr, l, L, nr, seed + (uint64_t)r0, rule, t0, chunk, cycle, p.ctas, bar, err, timeout_s, s,
+                                  first ? inject : 0);
             }
             // a device that cannot hold the clusters or the grid (a partition of the GPU) refuses the
             // first launch, before anything is enqueued

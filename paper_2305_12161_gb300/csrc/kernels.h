@@ -72,10 +72,11 @@ struct ResidentPlan {
     double start_us; // of the launches, beside their sweeps, about
 };
 bool resident_plan(int L, int R, int sms, ResidentPlan *out);
-// Replica r has the Philox key seed + r, or seeds[r] (device memory; cycle 01 only).  Returns cudaErrorNotSupported, with nothing enqueued, where the device cannot hold the launch.
+// Replica r has the Philox key seed + r, or seeds[r] (device memory; cycle 01 only).  inject (tests): a wait of
+// the first grid launch runs out (1 a neighbour's planes, 2 a barrier of all CTAs).  Returns cudaErrorNotSupported, with nothing enqueued, where the device cannot hold the launch.
 cudaError_t launch_sweeps_resident(uint32_t *lat, int L, int R, uint64_t seed, int rule, int64_t t0, int64_t n,
                                    int cycle, const ResidentPlan &p, int *err, double timeout_s, cudaStream_t s,
-                                   int64_t *launches, const uint64_t *seeds = nullptr);
+                                   int64_t *launches, const uint64_t *seeds = nullptr, int inject = 0);
 
 // Scope around a cooperative launch of `ctas` CTAs on stream s, or the launch of a graph whose largest one
 // has that many: it waits for those of this process on the current device beside which its CTAs would

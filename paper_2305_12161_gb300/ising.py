@@ -79,6 +79,7 @@ def lib() -> ctypes.CDLL:
                 "ising_radial_bins": (ctypes.c_int64, [ctypes.c_int]),
                 "ising_release_scratch": (ctypes.c_int, [vp]),
                 "ising_inject_corr_stall": (ctypes.c_int, [vp, ctypes.c_double]),
+                "ising_inject_sweep_stall": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_double]),
                 "ising_measure_radial": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, ctypes.c_double, vp, vp,
                                                         vp, vp, vp]),
                 "ising_get_spins": (ctypes.c_int, [vp, ctypes.c_int, vp]),
@@ -275,6 +276,10 @@ class Ising:
     def inject_corr_stall(self, timeout_s: float = 0.5) -> None:
         """Test hook: the next tensor-core measurement's bounded wait runs out (ISING_ETIMEOUT)."""
         self._check(lib().ising_inject_corr_stall(self._h, timeout_s), "ising_inject_corr_stall")
+
+    def inject_sweep_stall(self, barrier: bool = False, timeout_s: float = 0.5) -> None:
+        """Test hook: a bounded wait of the next resident grid sweep runs out (ISING_ETIMEOUT)."""
+        self._check(lib().ising_inject_sweep_stall(self._h, int(barrier), timeout_s), "ising_inject_sweep_stall")
 
     def release_scratch(self) -> None:
         """Free the measurement scratch kept in the context (radial FFT buffer, etc.)."""

@@ -182,3 +182,26 @@ def test_batch_classes_of_one_size_share_launches(ising, classes, launches, with
             b.sweep(n)
             assert b.launch_count() - l0 == without + 2 * n
             assert all(np.array_equal(x, y) for x, y in zip(_batch_states(b, classes), want))
+
+
+@pytest.mark.parametrize("barrier", [False, True])
+@pytest.mark.parametrize("L,R", [(192, 3), (256, 1), (512, 1)])
+def test_a_wait_that_runs_out_ends_with_a_status(ising, L, R, barrier):
+    # block 0 leaves out a message or a barrier arrival: every block returns, a queued sweep leaves at
+    # once, and the context reports the timeout
+    import time
+    with ising.Ising(L, replicas=R, seed=5) as q:
+        q.sweep(16)
+        q.sync()
+        q.inject_sweep_stall(barrier, timeout_s=0.3)
+        t0 = time.time()
+        q.sweep(16)
+        q.sweep(5000)
+        with pytest.raises(ising.IsingError) as e:
+            q.sync()
+        assert e.value.status == ising.ISING_ETIMEOUT and "resident" in str(e.value)
+        assert time.time() - t0 < 10
+        with pytest.raises(ising.IsingError) as e:
+            q.sweep(1)
+        assert e.value.status == ising.ISING_EPOISONED
+    _same(ising, L, R, [16])
