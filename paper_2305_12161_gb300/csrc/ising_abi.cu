@@ -449,9 +449,9 @@ int ising_sweep(ising_ctx *c, int64_t n)
     return ISING_OK;
 }
 
-// Synchronise the context's stream and report a device-side wait that gave up (the
-// tensor-core correlation's bounded mbarrier waits) as ISING_ETIMEOUT, which poisons the
-// context.
+// Synchronise the context's stream and report a device-side wait that gave up (of a sweep or of the
+// tensor-core correlation) as ISING_ETIMEOUT, which poisons the context.  Every call that hands
+// results or state to the host ends with it.
 static int check_device_waits(ising_ctx *c)
 {
     int h = 0;
@@ -512,7 +512,7 @@ int ising_measure_radial(ising_ctx *c, int replica, int precision, double cval, 
     CK(c, cudaMemcpyAsync(hc.data(), cnt, sizeof(int64_t) * hc.size(), cudaMemcpyDeviceToHost, c->stream));
     cudaFreeAsync(cnt, c->stream);
     cudaFreeAsync(out, c->stream);
-    CK(c, cudaStreamSynchronize(c->stream));
+    if ((s = check_device_waits(c)) != ISING_OK) return s;
     std::copy(h.begin(), h.begin() + nb, C);
     std::copy(h.begin() + nb, h.begin() + 2 * nb, S);
     if (ell) *ell = h[2 * nb];
@@ -630,8 +630,7 @@ int ising_get_spins(ising_ctx *c, int replica, int8_t *host_out)
         cudaFreeAsync(tmp, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "get_spins");
     }
-    CK(c, cudaStreamSynchronize(c->stream));
-    return ISING_OK;
+    return check_device_waits(c);
 }
 
 int ising_set_spins(ising_ctx *c, int replica, const int8_t *host_in)
@@ -673,8 +672,7 @@ int ising_get_packed(ising_ctx *c, int replica, uint32_t *words, unsigned flags)
     const bool dev = flags & ISING_PTR_DEVICE;
     CK(c, cudaMemcpyAsync(words, c->lat + (size_t)replica * 2 * c->g.nw, bytes,
                           dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-    if (!dev) CK(c, cudaStreamSynchronize(c->stream));
-    return ISING_OK;
+    return dev ? ISING_OK : check_device_waits(c);
 }
 
 int ising_set_packed(ising_ctx *c, int replica, const uint32_t *words, unsigned flags)

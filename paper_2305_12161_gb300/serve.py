@@ -176,6 +176,7 @@ class QuenchServer:
         still = []
         for a in self.active:
             if a.done_issuing() and all(e.query() for e in a.inflight):
+                a.ctx.sync()  # a device-side wait that gave up is an error here, not a result
                 rec = a.rec.cpu().numpy()
                 der = a.der.cpu().numpy()
                 self.results.append(Result(a.req, a.times, rec, der, a.admitted_s, self.now()))

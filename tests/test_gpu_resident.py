@@ -205,3 +205,29 @@ def test_a_wait_that_runs_out_ends_with_a_status(ising, L, R, barrier):
             q.sweep(1)
         assert e.value.status == ising.ISING_EPOISONED
     _same(ising, L, R, [16])
+
+
+@pytest.mark.parametrize("read", ["spins", "packed", "radial", "measure"])
+def test_a_read_reports_the_timeout(ising, read):
+    # the lattice holds messages after a sweep that gave up: no call hands it out as a state
+    with ising.Ising(256, replicas=1, seed=5) as q:
+        q.inject_sweep_stall(timeout_s=0.3)
+        q.sweep(16)
+        with pytest.raises(ising.IsingError) as e:
+            {"spins": q.get_spins, "packed": q.get_packed, "radial": q.measure_radial, "measure": q.measure}[read]()
+        assert e.value.status == ising.ISING_ETIMEOUT
+
+
+def test_the_server_reports_the_timeout(ising):
+    from paper_2305_12161_gb300 import serve
+    srv = serve.QuenchServer(tune=False)
+    srv.t0 = 0.0
+    srv.submit(serve.Request(id=0, L=192, t_max=16, replicas=1, seed=3, K=1))
+    srv._admit()
+    srv.active[0].ctx.inject_sweep_stall(timeout_s=0.3)
+    with pytest.raises(ising.IsingError) as e:
+        while srv.active:
+            for a in srv.active:
+                srv._issue(a)
+            srv._retire()
+    assert e.value.status == ising.ISING_ETIMEOUT and not srv.results
