@@ -232,6 +232,9 @@ int ising_inject_corr_stall(ising_ctx *ctx, double timeout_s);
  * (barrier = 1).  The waits of the other blocks run out after timeout_s, every block returns, later
  * resident sweeps leave at once, and the next synchronising call returns ISING_ETIMEOUT. */
 int ising_inject_sweep_stall(ising_ctx *ctx, int barrier, double timeout_s);
+/* The context measures from now on as if its correlation scratch could not be allocated: with
+ * ISING_CORR_AUTO from the packed lattice. */
+int ising_inject_scratch_refusal(ising_ctx *ctx);
 
 /* Free the scratch that measurements keep in the context (the radial measurement's transform
  * buffer and work area, the tensor-core correlation's expanded lattice) and the staging

@@ -548,6 +548,17 @@ int ising_inject_corr_stall(ising_ctx *c, double timeout_s)
     return ISING_OK;
 }
 
+int ising_inject_scratch_refusal(ising_ctx *c)
+{
+    int s = check_ctx(c);
+    if (s) return s;
+    DeviceGuard dg(c->device);
+    if (c->xt) CK(c, cudaFreeAsync(c->xt, c->stream));
+    c->xt = nullptr;
+    c->xt_refused = 1;
+    return ISING_OK;
+}
+
 int ising_inject_sweep_stall(ising_ctx *c, int barrier, double timeout_s)
 {
     int s = check_ctx(c);

@@ -80,6 +80,7 @@ def lib() -> ctypes.CDLL:
                 "ising_release_scratch": (ctypes.c_int, [vp]),
                 "ising_inject_corr_stall": (ctypes.c_int, [vp, ctypes.c_double]),
                 "ising_inject_sweep_stall": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_double]),
+                "ising_inject_scratch_refusal": (ctypes.c_int, [vp]),
                 "ising_measure_radial": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, ctypes.c_double, vp, vp,
                                                         vp, vp, vp]),
                 "ising_get_spins": (ctypes.c_int, [vp, ctypes.c_int, vp]),
@@ -280,6 +281,10 @@ class Ising:
     def inject_sweep_stall(self, barrier: bool = False, timeout_s: float = 0.5) -> None:
         """Test hook: a bounded wait of the next resident grid sweep runs out (ISING_ETIMEOUT)."""
         self._check(lib().ising_inject_sweep_stall(self._h, int(barrier), timeout_s), "ising_inject_sweep_stall")
+
+    def inject_scratch_refusal(self) -> None:
+        """Test hook: measure as if the correlation scratch could not be allocated."""
+        self._check(lib().ising_inject_scratch_refusal(self._h), "ising_inject_scratch_refusal")
 
     def release_scratch(self) -> None:
         """Free the measurement scratch kept in the context (radial FFT buffer, etc.)."""

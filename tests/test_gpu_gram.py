@@ -50,3 +50,19 @@ def test_line_order_units_equal_bit_counts(ising, L, R):
             a.sweep(n)
             b.sweep(n)
             assert np.array_equal(a.measure(), b.measure()), n
+
+
+@pytest.mark.parametrize("L,R", [(512, 3), (640, 1), (768, 2), (1024, 1)])
+def test_without_scratch_equals_bit_counts(ising, L, R):
+    """The packed lattice read in place at sizes that otherwise have copies in line order: the x axis
+    transposed by the filling warps, A tiles of off-diagonal units in shared memory."""
+    with ising.Ising(L, replicas=R, seed=29) as a, \
+            ising.Ising(L, replicas=R, seed=29, corr=ising.CORR_POPCOUNT) as b:
+        a.measure()
+        a.inject_scratch_refusal()
+        for n in (0, 3):
+            a.sweep(n)
+            b.sweep(n)
+            l0 = a.launch_count()
+            assert np.array_equal(a.measure(), b.measure()), n
+            assert a.launch_count() - l0 == 2  # the record's initialisation and the products
