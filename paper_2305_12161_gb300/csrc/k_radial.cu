@@ -202,23 +202,11 @@ __device__ __forceinline__ void fold_walk(int L, int chunk, Fn fn, End end)
     }
 }
 
-// Sum of four run sums in double.  Single precision: as an unevaluated pair of floats (Knuth's
-// two-sum, exact up to the last additions, 2^-48), because the device adds two doubles per clock and
-// SM: one addition instead of three.
-__device__ __forceinline__ double sum4(const double (&v)[4]) { return v[0] + v[1] + v[2] + v[3]; }
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+// Sum of four run sums in double.
+template <typename T>
+__device__ __forceinline__ double sum4(const T (&v)[4])
 {
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-__device__ __forceinline__ double sum4(const float (&v)[4])
-{
-    float a, b, c, ea, eb, ec;
-    two_sum(v[0], v[1], a, ea);
-    two_sum(v[2], v[3], b, eb);
-    two_sum(a, b, c, ec);
-    return (double)c + (double)__fadd_rn(__fadd_rn(ea, eb), ec);
+    return ((double)v[0] + (double)v[1]) + ((double)v[2] + (double)v[3]);
 }
 
 // 3. |F|^2 per mode of the half spectrum; S sums per bin; (P, 0) written back.
@@ -515,7 +503,7 @@ static cudaError_t run_radial(RadialPlans *p, const uint32_t *lat_r, int L, doub
         *cufft_status = cs;
         return cudaErrorUnknown;
     }
-    const double invN = 1.0 / ((double)L * (double)L * (double)L);  // exact: N is a power of two
+    const double invN = 1.0 / ((double)L * (double)L * (double)L);  // exact where L is a power of two
     auto corr = (int64_t)L * L * L <= (1 << 27) ? k_radial_corr<T, true> : k_radial_corr<T, false>;
     corr<<<grid, fold_threads, smem, s>>>(reinterpret_cast<const T *>(p->buf), L, chunk, P, nb, invN, sumG, inexact);
     k_radial_finish<<<1, 256, 0, s>>>(L, nb, c, sumG, sumS, p->count, inexact, out, cnt);
