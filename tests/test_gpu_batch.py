@@ -255,3 +255,71 @@ def test_tuner_times_the_kernels_it_chooses_between(ising):
                 q.sweep(n + 4)
                 for r in range(R):
                     assert np.array_equal(b.get_packed(ci, r), q.get_packed(r)), (L, r)
+
+
+# ---- the persistent kernel and the streamed classes, which sizes with a resident sweep no longer reach by
+# default: a class of L = 32 keeps the persistent kernel for all of them, and a class with a sweep kernel of
+# its own is streamed.  The reference is the one-word-per-thread half-sweep kernel.
+
+def _word_batch(ising, classes, n):
+    out = []
+    for L, R, seed in classes:
+        with ising.Ising(L, replicas=R, seed=seed, variant=ising.VARIANT_WORD) as q:
+            q.sweep(n)
+            out += [q.get_packed(r) for r in range(R)]
+    return out
+
+
+def _batch_equal(b, classes, want):
+    got = [b.get_packed(ci, r) for ci, (L, R, _) in enumerate(classes) for r in range(R)]
+    assert all(np.array_equal(x, y) for x, y in zip(got, want))
+
+
+def test_slab_groups_of_the_persistent_kernel(ising):
+    classes, n = [(32, 2, 90), (64, 8, 1), (192, 2, 5), (256, 2, 9), (320, 1, 70), (512, 1, 11)], 9
+    want = _word_batch(ising, classes, n)
+    with ising.Batch(classes) as b:
+        b.set_streamed(0)
+        assert b.streamed_classes() == 0 and b.plan()["groups"] >= 6
+        l0 = b.launch_count()
+        b.sweep(n)
+        assert b.launch_count() - l0 == 1
+        _batch_equal(b, classes, want)
+
+
+def test_work_lists_of_other_weights(ising):
+    classes, n = [(32, 4, 3), (64, 16, 2), (128, 4, 40)], 6
+    want = _word_batch(ising, classes, n)
+    plans = set()
+    with ising.Batch(classes) as b:
+        for wl in (1.0, 0.05, 0.25, 4.0, 20.0):
+            b.set_weights(wl, 1.0)
+            plans.add(tuple(b.plan().values()))
+            b.reinit()
+            l0 = b.launch_count()
+            b.sweep(n)
+            assert b.launch_count() - l0 == 1
+            _batch_equal(b, classes, want)
+    assert len(plans) > 1
+
+
+def test_streamed_kernels_beside_and_after_the_persistent_launch(ising):
+    classes, times = [(32, 3, 200), (64, 6, 3), (128, 2, 30), (256, 3, 60), (512, 2, 90)], [4, 9]
+    want = _word_batch(ising, classes, times[-1])
+    recs = {}
+    for on in (False, True):
+        with ising.Batch(classes) as b:
+            b.set_overlap(on)
+            b.set_class_config(3, variant=ising.VARIANT_ZFAST, tile_z=8)
+            b.set_class_config(4, variant=ising.VARIANT_ZFUSE, tile_z=16, depth=10)
+            l0 = b.launch_count()
+            b.sweep(times[0])
+            b.sweep(times[1] - times[0])
+            # per call the persistent launch, two half-sweeps of 256^3, a launch per sweep of 512^3 and an
+            # odd last one in place
+            assert b.launch_count() - l0 == (1 + 8 + 4) + (1 + 10 + 4 + 2)
+            _batch_equal(b, classes, want)
+            b.reinit()
+            recs[on], _ = b.run(times)
+            _batch_equal(b, classes, want)
+    assert np.array_equal(recs[False], recs[True])
