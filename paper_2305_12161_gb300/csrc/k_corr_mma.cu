@@ -287,7 +287,7 @@ struct GramArgs {
     int64_t RL, nw;            // record length; words per sublattice
     int L, W;
     int nsb, nunits, nitems;
-    int split_x, split_yz;     // slices of the lines: x axis, y and z axes
+    int split;                 // slices of an axis's lines
     int nrep;
     int stage_bytes, nst;      // ring of stages
     int ncols, scale_col;      // tensor memory: columns allocated, first of the 32 scale columns
@@ -629,10 +629,9 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
     uint32_t nitem = 0;  // items done: phase of `done`
     uint32_t nturn = 0;  // turns this issuer has waited for: phase of its `turn`
     for (int item = blockIdx.x; item < ga.nitems; item += gridDim.x, ++nitem) {
-        const int items_x = ga.nrep * ga.split_x * ga.nunits, items_y = ga.nrep * ga.split_yz * ga.nunits;
-        const int axis = item < items_x ? 0 : (item < items_x + items_y ? 1 : 2);
-        const int split = axis == 0 ? ga.split_x : ga.split_yz;
-        int rest = item - (axis == 0 ? 0 : (axis == 1 ? items_x : items_x + items_y));
+        const int split = ga.split, items_axis = ga.nrep * split * ga.nunits;
+        const int axis = item < items_axis ? 0 : (item < 2 * items_axis ? 1 : 2);
+        int rest = item - axis * items_axis;
         const GramUnit un = gram_unit(rest % ga.nunits, ga.nsb, L);
         rest /= ga.nunits;
         const int r = rest / split, sl = rest - r * split;
@@ -936,22 +935,18 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
                 k_lines_yz<<<dim3((unsigned)(L / 32), (unsigned)L, (unsigned)(2 * nr)), 256, 0, s>>>(ga.lat, g, scratch,
                                                                                                      ga.rep_words);
         }
-        // slices of the lines: the counts whose items take the fewest stages over the CTAs, counting an
-        // item's start and read-back as 8 stages, and a stage of the x axis as 1.5 where the kernel
-        // transposes it (so that axis is cut finer: eight L = 256 replicas 54 -> X256 us)
+        // slices of the lines: the count whose items take the fewest stages over the CTAs, counting an item's
+        // start and read-back as 8 stages.  The same for the three axes: with the x axis cut half as fine
+        // again where the kernel transposes it, a record of eight L = 256 replicas took 46.0 us instead of
+        // 43.5, of two L = 320 79.6 instead of 68.2, of six L = 128 14.2 instead of 13.2.
         ga.nrep = nr;
         const int64_t base = (int64_t)nr * ga.nunits;
-        const double wx = lines ? 1.0 : 1.5;
-        double best = 1e300;
+        int64_t best = INT64_MAX;
         for (int sp = 1; sp <= std::min(nk, 64); ++sp) {
-            const int sx = std::min(nk, (int)(wx * sp + 0.5));
-            const int64_t items = base * (sx + 2 * sp);
-            const double tx = wx * ((nk + sx - 1) / sx) + 8.0, ty = (double)((nk + sp - 1) / sp) + 8.0;
-            const int64_t rounds = (items + slots - 1) / slots;
-            const double cost = (double)rounds * std::max(tx, ty);
-            if (cost < best * 0.999) best = cost, ga.split_x = sx, ga.split_yz = sp;
+            const int64_t rounds = (base * 3 * sp + slots - 1) / slots, cost = rounds * ((nk + sp - 1) / sp + 8);
+            if (cost < best) best = cost, ga.split = sp;
         }
-        ga.nitems = (int)(base * (ga.split_x + 2 * ga.split_yz));
+        ga.nitems = (int)(base * 3 * ga.split);
         ga.inject = inject && r0 == 0;
         const int grid = std::min(ga.nitems, slots);
         cudaError_t e;
