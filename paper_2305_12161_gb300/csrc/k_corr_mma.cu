@@ -13,14 +13,14 @@
 // write them into the shared-memory tiles (and, for off-diagonal units of line-order copies, the
 // tensor-memory A tile) that tcgen05.mma reads.  At L = 2048 a measurement takes 8.7 ms against
 // 21.1 with e4m3 operands staged through global memory (8.6 GB written and re-read per axis, and
-// half the tensor rate); eight L = 256 replicas take 0.054 ms against 0.51 by bit counts, 512 of
+// half the tensor rate); eight L = 256 replicas take 0.044 ms against 0.51 by bit counts, 512 of
 // L = 64 0.04 against 0.28.  At L = 2048 the filling warps' instructions bound it: a stage of four
 // products is 512 cycles of tensor work and takes about 760.
 //
 // Only the upper block triangle of G is computed (G is symmetric): an entry j < k stands for
 // both ordered pairs, i.e. for the distances k - j and L - (k - j).  B is the sum of the three
 // axes' D_a(1), and M is counted by the warps that read the z axis's words, so a measurement
-// is one pass of this kernel (plus, for L >= 512, a transposition of the lattice for the x axis).
+// is one pass of this kernel (plus, for most L >= 512, copies of the lattice in the order it reads).
 #include <algorithm>
 
 #include "common.cuh"
@@ -191,7 +191,8 @@ __device__ __forceinline__ void sts128(uint32_t addr, const uint4 &v)
 }
 
 // ---------------------------------------------------------------------------------
-// Line order for L >= 512, where each word is read by several CTAs: per axis a copy of the packed
+// Line order for L >= 512 (the x axis for multiples of 128, all three for multiples of 256), where each
+// word is read by several CTAs: per axis a copy of the packed
 // lattice, N / 8 bytes, in which uint4 (2 c + h) L + p holds half h of the 256 lines of chunk c
 // at position p, so that a warp of 32 positions reads 512 consecutive bytes.  Read from the
 // packed store the words of 32 positions lie 128 bytes (y) or a plane (z) apart: at L = 2048 a
@@ -287,7 +288,7 @@ struct GramArgs {
     int64_t RL, nw;            // record length; words per sublattice
     int L, W;
     int nsb, nunits, nitems;
-    int split;                 // slices of an axis's lines
+    int split_x, split_yz;     // slices of the lines: x axis, y and z axes
     int nrep;
     int stage_bytes, nst;      // ring of stages
     int ncols, scale_col;      // tensor memory: columns allocated, first of the 32 scale columns
@@ -568,7 +569,7 @@ __device__ __forceinline__ bool fill_stages_ahead(const Fill &f, uint32_t g0, in
 //
 // READS: which readers the instantiation holds (fewer keep more warps within the registers).
 // MINB CTAs share an SM.
-enum GramReads : int { GR_SMALL, GR_T, GR_XL, GR_ANY };  // XL + YZ1; T alone; XL + YZ4; all
+enum GramReads : int { GR_SMALL, GR_T, GR_XL, GR_ANY };  // XL + YZ1; T alone; XL + YZ4; XL or T, and YZ1
 
 template <int PW, int MINB, int READS>
 __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArgs ga)
@@ -629,9 +630,10 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
     uint32_t nitem = 0;  // items done: phase of `done`
     uint32_t nturn = 0;  // turns this issuer has waited for: phase of its `turn`
     for (int item = blockIdx.x; item < ga.nitems; item += gridDim.x, ++nitem) {
-        const int split = ga.split, items_axis = ga.nrep * split * ga.nunits;
-        const int axis = item < items_axis ? 0 : (item < 2 * items_axis ? 1 : 2);
-        int rest = item - axis * items_axis;
+        const int items_x = ga.nrep * ga.split_x * ga.nunits, items_y = ga.nrep * ga.split_yz * ga.nunits;
+        const int axis = item < items_x ? 0 : (item < items_x + items_y ? 1 : 2);
+        const int split = axis == 0 ? ga.split_x : ga.split_yz;
+        int rest = item - (axis == 0 ? 0 : (axis == 1 ? items_x : items_x + items_y));
         const GramUnit un = gram_unit(rest % ga.nunits, ga.nsb, L);
         rest /= ga.nunits;
         const int r = rest / split, sl = rest - r * split;
@@ -719,7 +721,7 @@ __global__ void __launch_bounds__(32 * (PW + 2), MINB) k_gram_bits(const GramArg
                     } else if (READS == GR_ANY && axis == 0) {
                         ReadT rd(ga.lines + (int64_t)r * ga.rep_words + (int64_t)axis * 2 * ga.nw, L, p, c0 + set, nsets);
                         ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
-                    } else if (READS == GR_XL || (READS == GR_ANY && W % 4 == 0)) {
+                    } else if (READS == GR_XL) {
                         ReadYZ4 rd(S0, S1, L, W, axis, p, c0 + set, nsets);
                         ok = fill_stages(fl, g0, set, nsets, n, rd, expand, put);
                     } else {
@@ -888,8 +890,9 @@ static cudaError_t launch_gram(const GramArgs &ga, int grid, size_t smem, cudaSt
 }
 
 // rec: records initialised to D = N / 2 (r >= 1), M = -N, B = 3 N / 2.  scratch: 2 L^3 bytes for
-// the copies in line order, or null (the kernel then reads the packed store: below L = 512 a word is
-// read by one to three units only).
+// the copies in line order, or null (the kernel then reads the packed store: below L = 512, where a word
+// is read by one to three units only, for sizes that corr_mma_supported refuses, and where the scratch
+// could not be allocated).
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *scratch, int *err,
                             cudaStream_t s, int64_t *launches, bool pdl, double timeout_s, int inject)
 {
@@ -935,18 +938,24 @@ cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uin
                 k_lines_yz<<<dim3((unsigned)(L / 32), (unsigned)L, (unsigned)(2 * nr)), 256, 0, s>>>(ga.lat, g, scratch,
                                                                                                      ga.rep_words);
         }
-        // slices of the lines: the count whose items take the fewest stages over the CTAs, counting an item's
-        // start and read-back as 8 stages.  The same for the three axes: with the x axis cut half as fine
-        // again where the kernel transposes it, a record of eight L = 256 replicas took 46.0 us instead of
-        // 43.5, of two L = 320 79.6 instead of 68.2, of six L = 128 14.2 instead of 13.2.
+        // slices of the lines: the counts whose items take the fewest stages over the CTAs, counting an
+        // item's start and read-back as 8 stages, and from L = 512 a stage of the x axis as 1.5 where the
+        // kernel transposes it, so that axis is cut finer.  A record of one L = 576 replica takes 227 us
+        // that way and 246 with equal slices, of one L = 704 439 and 443; of two L = 320 80 and 69, of one
+        // L = 448 89 and 75, of eight L = 256 46 and 44, of six L = 128 14.2 and 13.2.
         ga.nrep = nr;
         const int64_t base = (int64_t)nr * ga.nunits;
-        int64_t best = INT64_MAX;
+        const double wx = lines || L < 512 ? 1.0 : 1.5;
+        double best = 1e300;
         for (int sp = 1; sp <= std::min(nk, 64); ++sp) {
-            const int64_t rounds = (base * 3 * sp + slots - 1) / slots, cost = rounds * ((nk + sp - 1) / sp + 8);
-            if (cost < best) best = cost, ga.split = sp;
+            const int sx = std::min(nk, (int)(wx * sp + 0.5));
+            const int64_t items = base * (sx + 2 * sp);
+            const double tx = wx * ((nk + sx - 1) / sx) + 8.0, ty = (double)((nk + sp - 1) / sp) + 8.0;
+            const int64_t rounds = (items + slots - 1) / slots;
+            const double cost = (double)rounds * std::max(tx, ty);
+            if (cost < best * 0.999) best = cost, ga.split_x = sx, ga.split_yz = sp;
         }
-        ga.nitems = (int)(base * 3 * ga.split);
+        ga.nitems = (int)(base * (ga.split_x + 2 * ga.split_yz));
         ga.inject = inject && r0 == 0;
         const int grid = std::min(ga.nitems, slots);
         cudaError_t e;
