@@ -115,7 +115,7 @@ typedef struct {
  * (ising_release_scratch frees it).  AUTO: TENSOR for L a multiple of 64 in 64..2048, else
  * POPCOUNT; the scratch is allocated as for TENSOR where L >= 512 is a multiple of 128, and the
  * kernel reads the packed lattice where there is none or it cannot be allocated (measured on
- * GB300: eight L = 256 replicas 0.05 ms against 0.51 by POPCOUNT, L = 2048 13 against 136). */
+ * GB300: eight L = 256 replicas 0.044 ms against 0.51 by POPCOUNT, L = 2048 8.7 against 136). */
 typedef enum { ISING_CORR_AUTO = 0, ISING_CORR_POPCOUNT = 1, ISING_CORR_TENSOR = 2 } ising_corr;
 
 /* Sublattice order of a sweep.  01: red (q = 0) then blue every sweep (the paper's main

@@ -32,7 +32,7 @@ struct ising_ctx {
     int8_t *plain = nullptr;     // PLAIN form lattice
     int64_t *rec_dev = nullptr;  // R records
     double *der_dev = nullptr;   // R x 4
-    uint32_t *xt = nullptr;      // tensor-core correlation, L >= 512: bit-transposed lattice (lazy)
+    uint32_t *xt = nullptr;      // tensor-core correlation, L >= 512: copies in line order (lazy)
     int *dev_err = nullptr;      // [0] set by a device-side bounded wait that gave up, [1, 2] counters of
                                  // the resident sweep's barriers
     int xt_refused = 0;          // that scratch could not be allocated (AUTO then measures without it)
@@ -595,7 +595,7 @@ int ising_measure_ex(ising_ctx *c, int64_t *rec, double *derived, double cval, u
             c->xt = nullptr;
             cudaGetLastError();  // a failed allocation is not sticky
             if (c->opts.corr == ISING_CORR_TENSOR) return fail(c, ISING_ENOMEM, "correlation scratch");
-            c->xt_refused = 1;   // automatic choice: the kernel transposes the x axis as it reads
+            c->xt_refused = 1;   // automatic choice: the kernel reads the packed lattice
         }
     }
     const int inject = method == CORR_TENSOR ? c->inject_stall : 0;

@@ -98,7 +98,7 @@ __device__ __forceinline__ U4 fused_draw(uint32_t c0, uint32_t x0_2, uint32_t x2
     return o;
 }
 
-// philox4x32_10_lead with the product form chosen
+// The same with the constants of one replica, read as constant-bank operands.
 template <bool WIDE>
 __device__ __forceinline__ U4 fused_draw(uint32_t c0, const PhiloxLead &ld, const PhiloxKeys &k)
 {

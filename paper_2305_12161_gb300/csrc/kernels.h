@@ -146,7 +146,8 @@ cudaError_t launch_unpack(const uint32_t *lat, int8_t *plain, int L, int R, cuda
 // correlation sums D_a(r) by the chosen method (CORR_NONE writes D_a(r) = -1).
 // CORR_TENSOR needs gram_supported(L) and err (a device int set to 1 if a bounded wait of the
 // tensor-core kernel gave up; the records are then incomplete); xt_scratch is either
-// corr_mma_scratch_bytes(L, R) bytes, which L >= 512 uses for the transposed x axis, or null.
+// corr_mma_scratch_bytes(L, R) bytes, which L >= 512 uses for copies of the axes in the order the kernel
+// reads (x, and y and z where L is a multiple of 256), or null.
 enum CorrMethod : int { CORR_NONE = 0, CORR_POPCOUNT = 1, CORR_TENSOR = 2 };
 // pdl: programmatic dependent launch of the measurement's kernels.  wait_timeout_s bounds each
 // device-side wait of the tensor-core path (wall time); inject_stall (tests) makes one of its CTAs skip a
