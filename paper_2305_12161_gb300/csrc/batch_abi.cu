@@ -273,8 +273,8 @@ int build_groups(ising_batch *b)
 // the persistent kernel 0.064 us times the largest L or 0.28 us per million spins, and 5.6 us to start;
 // streamed kernels 6.8 us or 0.09 us per million, and 1 us.  Measured, us per sweep over calls of 64:
 // sixteen classes of one 64^3 3.1 on the persistent kernel and 1.3 in one resident launch (18.8 with a
-// launch per class), sixteen of one 192^3 32.0 and 7.9, eight of one 256^3 25.8 streamed and 7.2; 8 x 64^3 +
-// 2 x 192^3 + 320^3 20.5 and 11.9, but over calls of two sweeps 23.3 and 26.2.
+// launch per class), sixteen of one 192^3 32.0 and 8.0, eight of one 256^3 25.8 streamed and 6.9; 8 x 64^3 +
+// 2 x 192^3 + 320^3 20.5 and 12.2, but over calls of two sweeps 23.3 and 26.2.
 bool choose_resident(const ising_batch *b, int64_t n, bool grid, bool small_allowed, std::vector<char> &res)
 {
     double res_us[2] = {0, 0};  // resident: [0] the persistent kernel's classes, [1] streamed ones

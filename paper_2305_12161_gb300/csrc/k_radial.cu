@@ -23,7 +23,7 @@
 // added to the CTA's bins in shared memory.  The modes' |F|^2 are summed in their precision over runs
 // of equal bins of 32 consecutive x (a warp scan per row), then in double over the four rows and the
 // bins.  (With a bin, a scan and a 64-bit atomic per value and row these passes took 0.80 and 0.94 ms
-// at L = 512 for 1.07 and 0.54 GB, the count 0.69; now 0.43, 0.36 and 0.06.)
+// at L = 512 for 1.07 and 0.54 GB, the count 0.69; now 0.43, 0.27 and 0.06.)
 // The number of vectors per bin does not depend on the state and is counted once per context.
 // The transform buffer and cuFFT's work area stay allocated in the context between calls.
 //
