@@ -262,6 +262,7 @@ int ising_measure(ising_ctx *ctx, int64_t *out);
  *   e = -3 + 2B/N, m = M/N, l_E = N/B (+inf when B = 0),
  *   l_C = first intersection of C(r) = sum_a (N - 2 D_a(r)) / (3N) with the constant
  *   c (Results: c = 0.5), linearly interpolated; NaN if C does not cross c, r <= L/2.
+ * After a device-side wait that gave up all four are NaN (e and m are finite otherwise).
  * Without ISING_MEAS_DEVICE both pointers are host memory and the call synchronises. */
 int ising_measure_ex(ising_ctx *ctx, int64_t *rec, double *derived, double c, unsigned flags);
 

@@ -428,7 +428,7 @@ int enqueue_measure(ising_batch *b, int64_t *rec, double *der, double c, unsigne
                               b->d_status, (double)b->timeout_ns * 1e-9));
         if (der)
             BCK(b, launch_derived(rec + k.rec_off, k.L, k.R, c, flags & ISING_MEAS_CONNECTED, der + 4 * k.der_off,
-                                  st, &b->launches));
+                                  st, &b->launches, b->d_status));
         if (i > 0) BCK(b, cudaEventRecord(b->ev[i], st));
     }
     for (int i = 1; i < nc; ++i) BCK(b, cudaStreamWaitEvent(b->stream, b->ev[i], 0));

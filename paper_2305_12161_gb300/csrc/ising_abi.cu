@@ -605,7 +605,8 @@ int ising_measure_ex(ising_ctx *c, int64_t *rec, double *derived, double cval, u
     double *ddst = nullptr;
     if (derived) {
         ddst = dev ? derived : c->der_dev;
-        CK(c, launch_derived(rdst, c->L, c->R, cval, flags & ISING_MEAS_CONNECTED, ddst, c->stream, &c->launches));
+        CK(c, launch_derived(rdst, c->L, c->R, cval, flags & ISING_MEAS_CONNECTED, ddst, c->stream, &c->launches,
+                             c->dev_err));
     }
     if (!dev) {
         const int64_t RL = ising_record_len(c->L);

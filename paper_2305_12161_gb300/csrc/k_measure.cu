@@ -444,8 +444,10 @@ cudaError_t launch_measure(const uint32_t *lat, int L, int R, int64_t t, int cor
 // ---------------------------------------------------------------------------------
 // Derived quantities (double precision): e = -3 + 2B/N, m = M/N, l_E = N/B, and the
 // first linear-interpolated crossing l_C of C(r) = sum_a (N - 2 D_a(r)) / (3N) (- m^2
-// when connected) with the constant c (Results: c = 0.5).
-__global__ void k_derived(const int64_t *rec, int L, int R, double c, bool connected, double *out)
+// when connected) with the constant c (Results: c = 0.5).  All four are NaN when *err says that a bounded
+// wait gave up before (e and m are finite otherwise), so that a caller who reads them without asking for
+// the status cannot take them for results.
+__global__ void k_derived(const int64_t *rec, int L, int R, double c, bool connected, double *out, const int *err)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
@@ -456,6 +458,10 @@ __global__ void k_derived(const int64_t *rec, int L, int R, double c, bool conne
     const int64_t *Dx = q + 3, *Dy = q + 3 + (H + 1), *Dz = q + 3 + 2 * (H + 1);
     const double m = __ddiv_rn((double)M, N);
     double *o = out + 4 * (int64_t)r;
+    if (err && *err) {
+        o[0] = o[1] = o[2] = o[3] = __longlong_as_double(0x7ff8000000000000ll);
+        return;
+    }
     o[0] = __dadd_rn(-3.0, __ddiv_rn(__dmul_rn(2.0, (double)B), N));
     o[1] = m;
     o[2] = B == 0 ? __longlong_as_double(0x7ff0000000000000ll) : __ddiv_rn(N, (double)B);
@@ -482,9 +488,9 @@ __global__ void k_derived(const int64_t *rec, int L, int R, double c, bool conne
 }
 
 cudaError_t launch_derived(const int64_t *rec, int L, int R, double c, bool connected, double *derived,
-                           cudaStream_t s, int64_t *launches)
+                           cudaStream_t s, int64_t *launches, const int *err)
 {
-    k_derived<<<(R + 127) / 128, 128, 0, s>>>(rec, L, R, c, connected, derived);
+    k_derived<<<(R + 127) / 128, 128, 0, s>>>(rec, L, R, c, connected, derived, err);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }

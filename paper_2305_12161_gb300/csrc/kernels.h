@@ -160,8 +160,8 @@ bool corr_mma_supported(int L);  // sizes of the explicit option ISING_CORR_TENS
 size_t corr_mma_scratch_bytes(int L, int R);
 cudaError_t launch_corr_mma(const uint32_t *lat, int L, int R, int64_t *rec, uint32_t *xt_scratch, int *err,
                             cudaStream_t s, int64_t *launches, bool pdl, double timeout_s, int inject);
-// derived: R x [e, m, l_E, l_C]
+// derived: R x [e, m, l_E, l_C]; all NaN where *err (may be null) says that a bounded wait gave up.
 cudaError_t launch_derived(const int64_t *rec, int L, int R, double c, bool connected, double *derived,
-                           cudaStream_t s, int64_t *launches);
+                           cudaStream_t s, int64_t *launches, const int *err = nullptr);
 
 }  // namespace ising

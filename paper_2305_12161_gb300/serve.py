@@ -176,9 +176,10 @@ class QuenchServer:
         still = []
         for a in self.active:
             if a.done_issuing() and all(e.query() for e in a.inflight):
-                a.ctx.sync()  # a device-side wait that gave up is an error here, not a result
                 rec = a.rec.cpu().numpy()
                 der = a.der.cpu().numpy()
+                if np.isnan(der[-1, :, 0]).any():  # e is NaN after a device-side wait that gave up
+                    a.ctx.sync()               # raises
                 self.results.append(Result(a.req, a.times, rec, der, a.admitted_s, self.now()))
                 self.updates += a.updates
                 self.used -= self.footprint(a.req)

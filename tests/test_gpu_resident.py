@@ -218,6 +218,23 @@ def test_a_read_reports_the_timeout(ising, read):
         assert e.value.status == ising.ISING_ETIMEOUT
 
 
+def test_derived_values_of_a_sweep_that_gave_up_are_nan(ising):
+    import torch
+    with ising.Ising(192, replicas=2, seed=5) as q, ising.Batch([(192, 1, 5)]) as b:
+        rec = torch.empty((2, q.record_len), dtype=torch.int64, device="cuda")
+        der = torch.zeros((2, 2, 4), dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        q.sweep(16)
+        q.measure_device(rec, der[0])
+        q.inject_sweep_stall(timeout_s=0.3)
+        q.sweep(16)
+        q.measure_device(rec, der[1])
+        torch.cuda.synchronize()
+        assert torch.isfinite(der[0, :, :3]).all() and torch.isnan(der[1]).all()
+        b.sweep(16)
+        assert np.isfinite(b.measure_ex()[1][:, :3]).all()
+
+
 def test_the_server_reports_the_timeout(ising):
     from paper_2305_12161_gb300 import serve
     srv = serve.QuenchServer(tune=False)
